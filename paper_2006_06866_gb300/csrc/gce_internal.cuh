@@ -188,6 +188,90 @@ __device__ __forceinline__ int fold_split(float4 pt, float4 tr, float nphi, floa
     return fold_split_from<PDOT>(fold_split_fpart(pt, tr), pt, tr, nphi, zoff);
 }
 
+// Two points of one trial at once (fma.rn.f32x2: each half is the scalar
+// operation, rounded alone, so the slots are those of fold_split).  The CE
+// kernel's hot loop is bound by instruction issue, and a packed instruction
+// takes one issue slot for two FMAs; the pairing is over points and not over
+// trials because the staged points can be laid out as pairs once per curve
+// (no register moves in the loop), where a trial pair would need every point
+// value duplicated.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ float lo2(f32x2 v) {
+    float a, b;
+    unpack2(v, a, b);
+    return a;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma2_rd(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// A SPLIT32 trial in the registers of the packed fold: every constant twice.
+struct SplitPrep {
+    f32x2 fh, fl, nah, nal;
+};
+__device__ __forceinline__ SplitPrep split_prep(float4 t) {
+    return SplitPrep{dup2(t.x), dup2(t.y), dup2(t.z), dup2(t.w)};
+}
+__device__ __forceinline__ float4 split_trial(const SplitPrep &t) {
+    return make_float4(lo2(t.fh), lo2(t.fl), lo2(t.nah), lo2(t.nal));
+}
+// Two points: {tau_hi, tau_hi'}, {tau_lo, tau_lo'} and the same of tau^2.
+struct SplitPair {
+    f32x2 th, tl, t2h, t2l;
+};
+
+// fold_split_fpart of two points (a - b is written fma(b, -1, a): exact the
+// same value, and no negated operand is needed).
+__device__ __forceinline__ f32x2 fold_split_fpart2(const SplitPair &p, const SplitPrep &tr) {
+    const f32x2 m = dup2(kRound), neg = dup2(-1.0f);
+    const f32x2 t = fma2(p.th, tr.fh, m);
+    const f32x2 r = fma2(p.th, tr.fh, fma2(t, neg, m));
+    return fma2(p.th, tr.fl, fma2(p.tl, tr.fh, r));
+}
+
+// fold_split_from of two points; returns the bit patterns of the two rounding
+// FMAs (slot + bits of kRound).
+template <bool PDOT, bool REDUCE>
+__device__ __forceinline__ void fold_split_from2(f32x2 c, const SplitPair &p, const SplitPrep &tr,
+                                                 float nphi, float zoff, unsigned int &z0,
+                                                 unsigned int &z1) {
+    const f32x2 m = dup2(kRound), nm = dup2(-kRound), neg = dup2(-1.0f);
+    f32x2 x = c;
+    if (PDOT) {
+        const f32x2 t2 = fma2(tr.nah, p.t2h, m);
+        const f32x2 r2 = fma2(tr.nah, p.t2h, fma2(t2, neg, m));
+        c = fma2(tr.nah, p.t2l, c);
+        c = fma2(tr.nal, p.t2h, c);
+        x = add2(c, r2);
+    }
+    if (PDOT || REDUCE) x = fma2(add2(add2(x, m), nm), neg, x);
+    float a, b;
+    unpack2(fma2_rd(x, dup2(nphi), dup2(zoff)), a, b);
+    z0 = __float_as_uint(a);
+    z1 = __float_as_uint(b);
+}
+
 // Eq. 3 in 32-bit-limb fixed point, the phase in units of 2^-32 cycles so that
 // the integer cycles wrap out of a 32-bit word.  With T = T1 2^32 + T0 and
 // F = F1 2^32 + F0, bits 64..95 of T F are

@@ -58,7 +58,9 @@ typedef enum {
     /* binary64 with the operation sequence s = tau*f, b = a*tau,
      * x = fma(-b, tau, s), phi = x - floor(x), j = floor(phi*n_phase) (clamped),
      * f = 1/P, a = (0.5*Pdot)*f*f.  Counts are bit-identical to a CPU binary64
-     * evaluation of that sequence. */
+     * evaluation of that sequence.  (Within FIXED32's range the search evaluates
+     * the sequence itself only for points whose fixed-point phase lies so close
+     * to a phase-bin edge that the two folds could disagree.) */
     GCE_PHASE_FP64 = 0,
     /* FP32 double-float: tau, tau^2, f and a split into (hi, lo) float pairs,
      * error-free products via fmaf, integer cycles removed with a rounding
@@ -121,8 +123,9 @@ typedef struct gce_handle_s *gce_handle;
  * thread).  The handle owns the device workspace, the autotune cache and the
  * captured CUDA graphs.  *h is NULL on failure.
  * The workspace grows to the largest job seen and is kept until gce_destroy:
- * 8 (FP64) or 16 bytes per point, 16 (FP64, SPLIT32) or 32 (FIXED32) bytes per
- * (P, Pdot) trial, 8 k bytes per (curve, warp of a trial tile) for top-k (24 more with
+ * 16 bytes per point (FP64: 24), 16 (SPLIT32) or 32 (FIXED32, FP64) bytes per
+ * (P, Pdot) trial (where FP64's do not fit, 8 per point and 16 per trial, at
+ * the speed of binary64 arithmetic), 8 k bytes per (curve, warp of a trial tile) for top-k (24 more with
  * the significance), and 8 bytes per entry of the c ln c table (longest curve
  * + 1).  A grid of 5,183,995 periods x 512 Pdot values thus holds 42 GB of
  * trial constants in SPLIT32.  Growing a buffer waits for the device. */
@@ -234,7 +237,7 @@ gce_status gce_ce_topk_host(gce_handle h, const double *h_times, const double *h
  * (GCE_ERR_INVALID otherwise).  The call is synchronous on `stream` and folds
  * the device-side input checks into its status.
  * Returns GCE_ERR_NOMEM, launching nothing, when the job needs more than the
- * 32 MiB (about 16 B per point + 32 B per trial + 8 B per (curve, 64 trials,
+ * 32 MiB (about 16 B per point (FP64: 8) + 32 B per trial + 8 B per (curve, 64 trials,
  * k) + 0.5 MiB); use gce_ce_topk for larger jobs.  Returns
  * GCE_ERR_UNSUPPORTED when the bin counts need more shared memory than one CTA
  * of its fixed launch shape (256 threads, 2 trials each) can have.

@@ -82,7 +82,7 @@ struct gce_handle_s {
     int n_sm = 0;
     int smem_optin = 0;
     std::string last_error;
-    DevBuf payload, seg, trialc, order, offsets, cand, stats, table, state, in_times, in_mags,
+    DevBuf payload, tau, seg, trialc, order, offsets, cand, stats, table, state, in_times, in_mags,
         in_periods, in_pdots, out_H, out_idx, band_stats, cand2, stats2;
     int table_n = -1;                    // largest count the table covers
     int *h_order = nullptr;              // pinned staging
@@ -144,6 +144,9 @@ static gce_status ensure(gce_handle h, DevBuf &b, size_t bytes) {
     b.bytes = want;
     return GCE_OK;
 }
+
+// The CE kernel's fold for a job's phase mode: FP64 jobs run the certified one.
+static int kernel_mode(int mode) { return mode == GCE_PHASE_FP64 ? kFoldCertified : mode; }
 
 static int point_bytes(int mode) { return mode == GCE_PHASE_FP64 ? 8 : 16; }
 
@@ -271,7 +274,7 @@ extern "C" gce_status gce_destroy(gce_handle h) {
     cudaSetDevice(h->device);
     cudaDeviceSynchronize();
     for (auto &kv : h->graphs) cudaGraphExecDestroy(kv.second.exec);
-    DevBuf *bufs[] = {&h->payload, &h->seg, &h->trialc, &h->order, &h->offsets, &h->cand, &h->stats,
+    DevBuf *bufs[] = {&h->payload, &h->tau, &h->seg, &h->trialc, &h->order, &h->offsets, &h->cand, &h->stats,
                       &h->table, &h->state, &h->in_times, &h->in_mags, &h->in_periods,
                       &h->in_pdots, &h->out_H, &h->out_idx, &h->band_stats, &h->cand2,
                       &h->stats2};
@@ -316,6 +319,10 @@ struct Plan {
     int n_max, n_tiles, n_ptiles, pd_major, range, half, kv, block, tpt, grid, chunk, table_smem,
         grab;
     int n_groups, tiles_per_group;  // top-k: first merge level (0 groups: none)
+    // the payload's fold mode: kernel_mode(), or GCE_PHASE_FP64 for the diagnostic
+    // jobs and for an FP64 job whose certified payload (24 bytes per point and 32
+    // per trial instead of 8 and 16) does not fit the device
+    int prep_mode;
     size_t smem;
 };
 
@@ -336,8 +343,10 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     pl.range = RANGE_WIDE;
     if (cfg->phase_mode == GCE_PHASE_SPLIT32)
         pl.range = j.n_pdots > 1 ? RANGE_NARROW : t.slot_range == 1 ? RANGE_MID : RANGE_WIDE;
-    // one Pdot value: the SPLIT32 / FIXED32 staging holds 8-byte half points
-    pl.half = (cfg->phase_mode != GCE_PHASE_FP64 && j.n_pdots == 1) ? 1 : 0;
+    // one Pdot value: the staging holds 8-byte half points
+    pl.half = j.n_pdots == 1 ? 1 : 0;
+    const int kmode = kernel_mode(cfg->phase_mode);
+    pl.prep_mode = (j.kind == JOB_GRID || j.kind == JOB_TOPK) ? kmode : cfg->phase_mode;
     // the kernel instantiation: overlapping bins or not
     pl.kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
     const int kv = pl.kv;
@@ -365,11 +374,11 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
         // shrink the staged chunk, then the table, then trials per thread, then the
         // block, until the CTA fits in shared memory
         auto size = [&]() {
-            return main_smem_bytes(cfg->phase_mode, pl.block, pl.tpt, pl.chunk, cfg->n_phase_bins,
+            return main_smem_bytes(kmode, pl.block, pl.tpt, pl.chunk, cfg->n_phase_bins,
                                    cfg->n_mag_bins, pl.table_smem, pl.range, pl.half);
         };
         auto limit = [&]() {
-            return main_dynamic_smem_limit(cfg->phase_mode, pl.tpt, pl.block, kv, (size_t)h->smem_optin);
+            return main_dynamic_smem_limit(kmode, pl.tpt, pl.block, kv, (size_t)h->smem_optin);
         };
         pl.smem = size();
         while (pl.smem > limit()) {
@@ -383,8 +392,8 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
         }
         if (pl.smem > limit())
             return fail(h, GCE_ERR_UNSUPPORTED, "launch shape needs %zu bytes of shared memory", pl.smem);
-        CUDA_TRY(h, main_kernel_attrs(cfg->phase_mode, pl.tpt, pl.block, kv, (size_t)h->smem_optin));
-        const void *kern = main_kernel_ptr(cfg->phase_mode, pl.tpt, pl.block, kv);
+        CUDA_TRY(h, main_kernel_attrs(kmode, pl.tpt, pl.block, kv, (size_t)h->smem_optin));
+        const void *kern = main_kernel_ptr(kmode, pl.tpt, pl.block, kv);
         CUDA_TRY(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, pl.block, pl.smem));
         if (occ < 1) return fail(h, GCE_ERR_UNSUPPORTED, "launch shape does not fit on an SM");
         // A smaller staged chunk costs only more staging passes: take it whenever it
@@ -450,7 +459,8 @@ gce_status mark(gce_handle h, cudaEvent_t e, cudaStream_t s, bool capturing) {
 // Enqueue the whole sequence of one call on stream s (possibly under capture).
 gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, bool capturing) {
     const gce_config *cfg = j.cfg;
-    const int mode = cfg->phase_mode;
+    const int mode = pl.prep_mode;
+    const int kmode = kernel_mode(cfg->phase_mode);
     JobState *st = (JobState *)h->state.p;
     CUDA_TRY(h, cudaMemcpyAsync(h->offsets.p, h->h_offsets, sizeof(long long) * (j.n_curves + 1),
                                 cudaMemcpyHostToDevice, s));
@@ -479,6 +489,7 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
     pa.t0 = cfg->t0;
     pa.payload = h->payload.p;
     pa.seg = (int *)h->seg.p;
+    pa.tau = (double *)h->tau.p;
     pa.state = st;
     pa.bands = j.bands;
     pa.band_stats = (const double2 *)h->band_stats.p;
@@ -520,6 +531,13 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
     ma.overlap = (cfg->flags & GCE_FLAG_OVERLAP) ? 1 : 0;
     ma.half = pl.half;
     ma.kv = pl.kv;
+    ma.tau = (const double *)h->tau.p;
+    ma.periods = j.periods;
+    ma.pdots = j.pdots;
+    if ((j.kind == JOB_GRID || j.kind == JOB_TOPK) && mode == GCE_PHASE_FP64) {
+        ma.tau = (const double *)h->payload.p;  // binary64 fold alone
+        ma.payload = nullptr;
+    }
     ma.state = st;
     const bool timed = (cfg->flags & GCE_FLAG_TIME_KERNEL) != 0;
     gce_status ms;
@@ -527,7 +545,7 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
         case JOB_GRID:
             ma.out = j.out;
             if (timed && (ms = mark(h, h->k0, s, capturing)) != GCE_OK) return ms;
-            CUDA_TRY(h, launch_main(mode, pl.tpt, pl.block, pl.grid, pl.smem, ma, s));
+            CUDA_TRY(h, launch_main(kmode, pl.tpt, pl.block, pl.grid, pl.smem, ma, s));
             ++n_launch;
             if (timed && (ms = mark(h, h->k1, s, capturing)) != GCE_OK) return ms;
             break;
@@ -536,7 +554,7 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
             ma.k = j.k;
             if (j.rho) ma.stats = (TileStats *)h->stats.p;
             if (timed && (ms = mark(h, h->k0, s, capturing)) != GCE_OK) return ms;
-            CUDA_TRY(h, launch_main(mode, pl.tpt, pl.block, pl.grid, pl.smem, ma, s));
+            CUDA_TRY(h, launch_main(kmode, pl.tpt, pl.block, pl.grid, pl.smem, ma, s));
             ++n_launch;
             if (timed && (ms = mark(h, h->k1, s, capturing)) != GCE_OK) return ms;
             if (pl.n_groups > 0) {
@@ -630,9 +648,16 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
     Plan pl;
     gce_status st = make_plan(h, j, pl);
     if (st != GCE_OK) return st;
-    const int mode = j.cfg->phase_mode;
 
     // workspace
+    if (pl.prep_mode == kFoldCertified &&
+        (ensure(h, h->tau, 8 * (size_t)pl.n_points) != GCE_OK ||
+         ensure(h, h->payload, (size_t)point_bytes(kFoldCertified) * pl.n_points) != GCE_OK ||
+         ensure(h, h->trialc, trial_bytes(kFoldCertified) * (size_t)pl.n_trials) != GCE_OK)) {
+        h->last_error.clear();
+        pl.prep_mode = GCE_PHASE_FP64;
+    }
+    const int mode = pl.prep_mode;
     if ((st = ensure(h, h->payload, (size_t)point_bytes(mode) * pl.n_points)) != GCE_OK) return st;
     if ((st = ensure(h, h->seg, sizeof(int) * (size_t)j.n_curves * (j.cfg->n_mag_bins + 1))) != GCE_OK) return st;
     if ((st = ensure(h, h->trialc, trial_bytes(mode) * (size_t)pl.n_trials)) != GCE_OK) return st;
@@ -699,7 +724,8 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
                               j.mean, j.std_dev, j.rho, j.cell_curve, j.cell_trial, j.counts,
                               j.bands, h->payload.p, h->seg.p, h->trialc.p, h->order.p,
                               h->offsets.p, h->cand.p, h->stats.p, h->cand2.p, h->stats2.p,
-                              h->table.p, h->state.p, h->band_stats.p, h->h_order, h->h_offsets};
+                              h->table.p, h->state.p, h->band_stats.p, h->h_order, h->h_offsets,
+                              h->tau.p};
         for (const void *p : ptrs) fp.add(p);
         unsigned long long t0_bits;
         std::memcpy(&t0_bits, &j.cfg->t0, sizeof(t0_bits));
@@ -708,6 +734,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
         fp.add_u((unsigned long long)j.n_bands);
         fp.add_u((unsigned long long)j.n_cells);
         fp.add_u((unsigned long long)pl.n_long);
+        fp.add_u((unsigned long long)pl.prep_mode);
         auto it = h->graphs.find(key);
         if (it != h->graphs.end() && it->second.fp == fp) {
             // same shape and the same arrays as the cached graph: replay it as it is

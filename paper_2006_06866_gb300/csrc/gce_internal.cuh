@@ -22,7 +22,10 @@ struct JobState {
     unsigned long long pdot_max_bits;   // max |Pdot| as binary64 bits
     unsigned long long work;            // next work item (persistent kernel)
     unsigned int err;                   // ERR_* bits
-    unsigned int pad[3];
+    // FP64 jobs prepared for the certified fold: 1 when the job's range is beyond
+    // it, so that the binary64 fold runs on every point (set by k_trials)
+    unsigned int wide;
+    unsigned int pad[2];
 };
 
 enum : unsigned int {
@@ -33,6 +36,17 @@ enum : unsigned int {
     ERR_BAND = 16u,     // filter index outside [0, n_bands)
     ERR_SLOT = 32u,     // checked builds only: a counter slot outside the trial's kept range
 };
+
+// The CE kernel's fold of a GCE_PHASE_FP64 job (not part of the ABI): the FIXED32
+// fold with every point's distance to the phase-bin edges checked against the two
+// folds' error bound, and the binary64 fold for the points within it.
+enum { kFoldCertified = 3 };
+
+// Whether a job's maxima lie inside the FIXED32 fold's range: F < 2^63, and the
+// Pdot cross term small enough for its FP32 path.
+__host__ __device__ inline bool fixed_range_ok(double fmax, double amax, int e_tau) {
+    return !(ldexp(fmax, e_tau) >= 536870912.0 || ldexp(amax, 2 * e_tau) >= 262144.0);
+}
 
 // Fixed-point scaling of the FIXED32 fold, derived from the job's maxima.
 // tau_max < 2^e_tau.  T = tau 2^s (|T| < 2^62), F = f 2^r with s + r = 96, so
@@ -92,6 +106,15 @@ template <> struct ModeTraits<GCE_PHASE_SPLIT32> {
     __device__ static point_t widen(half_t h) { return make_float4(h.x, h.y, 0.0f, 0.0f); }
 };
 template <> struct ModeTraits<GCE_PHASE_FIXED32> {
+    typedef uint4 point_t;
+    typedef uint2 half_t;
+    typedef FixedTrial trial_t;
+    __device__ static point_t widen(half_t h) { return make_uint4(h.x, h.y, 0u, 0u); }
+};
+
+// FP64 jobs: FIXED32 points and trials; the binary64 tau of each point is kept
+// beside them (MainArgs::tau) for the points within the error bound of an edge.
+template <> struct ModeTraits<kFoldCertified> {
     typedef uint4 point_t;
     typedef uint2 half_t;
     typedef FixedTrial trial_t;
@@ -365,6 +388,23 @@ __device__ __forceinline__ unsigned int fold_fixed_bin_from(unsigned int acc, ui
     return __umulhi(fold_fixed_phase_from<PDOT, K0>(acc, pt, t), n_phase);
 }
 
+// The certified fold's margin, in units of 2^-32 cycles: above the distance
+// between the FIXED32 phase and the phase of the binary64 sequence, which the
+// bounds below add up to, and at least twice their sum.
+//   FIXED32 against tau f - a tau^2: T and F rounded to their limbs (1/4 + 1/8),
+//   the floor of hi32(T1 F0) (1), T0 F0 / 2^64 dropped (1/2), T0 >> 9 (F1 2^-23 <=
+//   2^(k-1)), G0 rounded (2^(k-2)), K and the FMA rounded (2^k); with a Pdot term U
+//   and A rounded (1/8), the floor of hi32(A0 U1) (1), A0 U0 dropped (1/2), U0 >> 9
+//   (1/8), one more FMA rounding (2^(k-1)), and, where the two cross terms carry the
+//   FMA result past 2^24, its coarser grid (|A1| / 4 + 2^k).  The binary64 sequence
+//   against the same: 2^-53 (2 |tau f| + 2 |a tau^2| + 3) cycles <= 2^k + 1, as
+//   |tau f| < F1 / 4 <= 2^(20+k) cycles and |a tau^2| < 2^18.
+// Sum: below 5 + 5 2^k + |A1| / 4.
+__device__ __forceinline__ unsigned int certified_margin(unsigned int k, unsigned int a1) {
+    const int a = (int)a1;
+    return 16u + (10u << k) + (unsigned int)(a < 0 ? -a : a);
+}
+
 // ------------------------------------------------------------------ entropy
 
 // The counter slots a trial keeps: logical slots [zmin, zmax] (fine phase
@@ -441,6 +481,7 @@ struct PrepArgs {
     double t0;
     void *payload;             // ModeTraits<MODE>::point_t[sum N], sorted by mag bin per curve
     int *seg;                  // [n_curves][n_mag + 1] segment starts (relative to the curve)
+    double *tau;               // certified FP64 jobs: tau in payload order, else nullptr
     const JobState *state;
     const unsigned char *bands;  // multi-filter input: filter of each point, or nullptr
     const double2 *band_stats;   // [n_curves][n_bands] {median, standard deviation}
@@ -517,6 +558,11 @@ struct MainArgs {
     // single Pdot is not 0 stages chunk / 2 whole points in the same bytes
     int half;
     int kv;                    // CE kernel variant (KV_*): overlapping bins or not
+    // FP64 jobs: every point's binary64 tau in payload order, and the caller's
+    // trial arrays (for the points the certified fold leaves to binary64)
+    const double *tau;
+    const double *periods;
+    const double *pdots;
     JobState *state;
 };
 

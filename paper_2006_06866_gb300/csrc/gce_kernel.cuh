@@ -165,6 +165,40 @@ template <> struct Fold<GCE_PHASE_FIXED32> {
     __device__ __forceinline__ static bool k_zero(const prep_t &t) { return t.k == 0u; }
 };
 
+// FP64 jobs: a FIXED32 trial whose phases come out raised by an error margin (in
+// C; the largest of the thread's trials), so that one comparison bounds the
+// distance to the edges on both sides: with w = (phase + margin) n_phase, the bin
+// is hi32(w), and it is also the binary64 sequence's bin unless lo32(w) < 2 margin
+// n_phase.
+struct CertPrep : FixedPrep {};
+template <> struct Fold<kFoldCertified> {
+    typedef CertPrep prep_t;
+    static constexpr int kSlotBias = 0;
+    __device__ __forceinline__ static prep_t prepare(const FixedTrial &t) {
+        prep_t p;
+        static_cast<FixedPrep &>(p) = fixed_prep(t);
+        return p;
+    }
+    __device__ __forceinline__ static unsigned int margin(const prep_t &p) {
+        return certified_margin(p.k, p.A1);
+    }
+    // a trial past the grid's end: every point in the middle of a bin
+    __device__ __forceinline__ static void park(prep_t &p, int n_phase) {
+        p.C += 0x80000000u / (unsigned int)n_phase;
+    }
+    template <bool PDOT, bool K0>
+    __device__ __forceinline__ static unsigned long long bins(unsigned int fpart, uint4 p,
+                                                              const prep_t &t,
+                                                              const FoldConst &k) {
+        return (unsigned long long)fold_fixed_phase_from<PDOT, K0>(fpart, p, t) *
+               (unsigned int)k.n_phase;
+    }
+    __device__ __forceinline__ static bool has_pdot(const FixedTrial &t) {
+        return (t.i.z | t.i.w) != 0u;
+    }
+    __device__ __forceinline__ static bool k_zero(const prep_t &t) { return t.k == 0u; }
+};
+
 // The increment carries no memory clobber, so the compiler may schedule the
 // next points' shared loads around it; compiler_fence() before and after each
 // hot loop keeps the counters' plain loads and stores on their side of it.
@@ -211,6 +245,56 @@ __device__ __forceinline__ void count_point(const typename ModeTraits<MODE>::poi
                        SHARED ? Fold<MODE>::template offset_from<PDOT, K0, SH, RED>(fp, p, tc[s], fk)
                               : Fold<MODE>::template offset<PDOT, K0, SH, RED>(p, tc[s], fk),
                        fk, inc);
+}
+
+// count_point of an FP64 job: the certified fold's bin, and near lowered to the
+// smallest lo32(w) seen (two trials per three-input minimum).
+template <int TPT, int SH, bool PDOT, bool K0, bool SHARED>
+__device__ __forceinline__ void count_point_cert(const uint4 &p, const CertPrep (&tc)[TPT],
+                                                 const unsigned int (&base)[TPT],
+                                                 const FoldConst &fk, unsigned int inc,
+                                                 unsigned int &near) {
+    unsigned int fp = 0u, lo[TPT];
+    if (SHARED) fp = fold_fixed_fpart(p, tc[0]);
+#pragma unroll
+    for (int s = 0; s < TPT; ++s) {
+        const unsigned long long w = Fold<kFoldCertified>::bins<PDOT, K0>(
+            SHARED ? fp : fold_fixed_fpart(p, tc[s]), p, tc[s], fk);
+        lo[s] = (unsigned int)w;
+        bump<kFoldCertified, SH>(base[s], (unsigned int)(w >> 32) << SH, fk, inc);
+    }
+    if (TPT == 1) near = min(near, lo[0]);
+#pragma unroll
+    for (int s = 0; s + 1 < TPT; s += 2) near = __vimin3_u32(near, lo[s], lo[s + 1]);
+}
+
+// The points of [ka, kb) of one trial that the certified fold may have put in the
+// wrong bin are decided by the binary64 sequence, and those that it did put there
+// are moved.  Rare (a point-trial comes here with probability 2 margin n_phase
+// 2^-32, about 3e-7 at 15 bins), so everything is read anew from global memory.
+template <int SH>
+__device__ __noinline__ void recount_near(const FixedTrial *tr, const double *tau, double period,
+                                          double pdot, const void *pts, bool half, int ka, int kb,
+                                          unsigned int base, unsigned int inc, unsigned int margin,
+                                          FoldConst fk) {
+    CertPrep t = Fold<kFoldCertified>::prepare(*tr);
+    t.C += margin;
+    const unsigned int thr = 2u * margin * (unsigned int)fk.n_phase;
+    const double f = 1.0 / period;
+    const double a = (0.5 * pdot) * f * f;
+    for (int k = ka; k < kb; ++k) {
+        typedef ModeTraits<kFoldCertified> MT;
+        const uint4 p = half ? MT::widen(static_cast<const uint2 *>(pts)[k])
+                             : static_cast<const uint4 *>(pts)[k];
+        const unsigned long long w =
+            Fold<kFoldCertified>::bins<true, false>(fold_fixed_fpart(p, t), p, t, fk);
+        if ((unsigned int)w >= thr) continue;
+        const unsigned int bin = (unsigned int)(w >> 32);
+        const unsigned int j = (unsigned int)fold_fp64<true>(tau[k], f, a, fk.nphi_d, fk.n_phase);
+        if (j == bin) continue;
+        bump<kFoldCertified, SH>(base, bin << SH, fk, 0u - inc);
+        bump<kFoldCertified, SH>(base, j << SH, fk, inc);
+    }
 }
 
 // Two points (SPLIT32, packed fold) counted as count_point does.
@@ -284,17 +368,23 @@ template <int MODE, int TPT, int SH, bool PDOT, bool K0, bool RED, bool SHARED, 
 __device__ __forceinline__ void count_points(
     const void *__restrict__ pts, int ka, int kb,
     const typename Fold<MODE>::prep_t (&tc)[TPT], const unsigned int (&base)[TPT],
-    const FoldConst &fk, unsigned int inc) {
+    const FoldConst &fk, unsigned int inc, unsigned int &near) {
     typedef ModeTraits<MODE> MT;
     static_assert(!(HALF && PDOT), "half points carry no tau^2");
     // points unrolled by 16 (8 with the longer Pdot fold): measured faster than 8
     // and 4 on every workload without a Pdot axis, and than 16 with one
     constexpr int UNROLL = PDOT ? 8 : 16;
-    constexpr bool PAIRS = HALF && MODE == GCE_PHASE_FIXED32;
+    constexpr bool PAIRS = HALF && (MODE == GCE_PHASE_FIXED32 || MODE == kFoldCertified);
+    auto one = [&](const typename MT::point_t &p) {
+        if constexpr (MODE == kFoldCertified)
+            count_point_cert<TPT, SH, PDOT, K0, SHARED>(p, tc, base, fk, inc, near);
+        else
+            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(p, tc, base, fk, inc);
+    };
     if constexpr (MODE == GCE_PHASE_SPLIT32) {
         int k = ka;
         if ((k & 1) && k < kb) {
-            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(staged_point<HALF>(pts, k), tc, base, fk, inc);
+            one(staged_point<HALF>(pts, k));
             ++k;
         }
         constexpr int UNROLL2 = UNROLL / 2;
@@ -302,13 +392,13 @@ __device__ __forceinline__ void count_points(
         for (; k + 1 < kb; k += 2)
             count_pair<TPT, SH, PDOT, RED, SHARED>(staged_pair<HALF, PDOT>(pts, k >> 1), tc, base, fk, inc);
         if (k < kb)
-            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(staged_point<HALF>(pts, k), tc, base, fk, inc);
+            one(staged_point<HALF>(pts, k));
     } else if constexpr (PAIRS) {
         typedef typename MT::half_t half_t;
         const half_t *hp = static_cast<const half_t *>(pts);
         int k = ka;
         if ((k & 1) && k < kb) {
-            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(MT::widen(hp[k]), tc, base, fk, inc);
+            one(MT::widen(hp[k]));
             ++k;
         }
         constexpr int UNROLL2 = UNROLL / 2;
@@ -317,18 +407,18 @@ __device__ __forceinline__ void count_points(
             const uint4 q = *reinterpret_cast<const uint4 *>(hp + k);
             half_t h0, h1;
             split_pair(q, h0, h1);
-            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(MT::widen(h0), tc, base, fk, inc);
-            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(MT::widen(h1), tc, base, fk, inc);
+            one(MT::widen(h0));
+            one(MT::widen(h1));
         }
         if (k < kb)
-            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(MT::widen(hp[k]), tc, base, fk, inc);
+            one(MT::widen(hp[k]));
     } else {
 #pragma unroll UNROLL
         for (int k = ka; k < kb; ++k) {
             const typename MT::point_t p =
                 HALF ? MT::widen(static_cast<const typename MT::half_t *>(pts)[k])
                      : static_cast<const typename MT::point_t *>(pts)[k];
-            count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(p, tc, base, fk, inc);
+            one(p);
         }
     }
 }
@@ -337,10 +427,10 @@ template <int MODE, int TPT, int SH, bool PDOT, bool K0, bool RED = false, bool 
 __device__ __forceinline__ void count_points_any(
     bool shared, const void *__restrict__ pts, int ka, int kb,
     const typename Fold<MODE>::prep_t (&tc)[TPT], const unsigned int (&base)[TPT],
-    const FoldConst &fk, unsigned int inc) {
+    const FoldConst &fk, unsigned int inc, unsigned int &near) {
     constexpr bool SH_OK = PDOT && TPT > 1;  // sharing pays only with a Pdot term
-    if (SH_OK && shared) count_points<MODE, TPT, SH, PDOT, K0, RED, SH_OK, HALF>(pts, ka, kb, tc, base, fk, inc);
-    else count_points<MODE, TPT, SH, PDOT, K0, RED, false, HALF>(pts, ka, kb, tc, base, fk, inc);
+    if (SH_OK && shared) count_points<MODE, TPT, SH, PDOT, K0, RED, SH_OK, HALF>(pts, ka, kb, tc, base, fk, inc, near);
+    else count_points<MODE, TPT, SH, PDOT, K0, RED, false, HALF>(pts, ka, kb, tc, base, fk, inc, near);
 }
 
 // c_ij of one phase bin at the end of a magnitude segment (low - snapshot), with
@@ -675,8 +765,9 @@ constexpr int main_min_blocks(int tpt, int log2b, int kv) {
                     : (log2b >= 9 ? 1 : (log2b == 8 ? 2 : (log2b == 7 ? 4 : 8)));
 }
 
-template <int MODE, int TPT, int LOG2B, int KV>
-__global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k_main(MainArgs a) {
+// LAYMODE: the fold mode that the launch's shared memory was laid out for.
+template <int MODE, int LAYMODE, int TPT, int LOG2B, int KV>
+__device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     // the counter formats are fixed per instantiation (a kernel that carried
     // the overlapping-bin format with a run-time choice measured slower on the
     // path that never used it)
@@ -685,15 +776,13 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
     typedef typename ModeTraits<MODE>::point_t point_t;
     typedef typename ModeTraits<MODE>::trial_t trial_t;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long s_item;
-
-    if (a.state->err) return;  // inputs failed the device checks: no work
 
     constexpr int B = 1 << LOG2B;
     constexpr int SH = LOG2B + 2;  // log2 of the byte stride between a thread's slots
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_phase = a.n_phase, n_mag = a.n_mag;
     constexpr bool SPLIT = MODE == GCE_PHASE_SPLIT32;
+    constexpr bool CERT = MODE == kFoldCertified;
     constexpr int ovl = OVL ? 1 : 0;  // 50 %-overlapping phase bins
     const int range = SPLIT ? a.range : (int)RANGE_WIDE;
     const SlotRange zr = slot_range(MODE, n_phase, range);
@@ -703,7 +792,7 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
 
     // the regions at the offsets the host sized the launch with (the table first,
     // so that its address is a constant)
-    const MainSmemLayout lay = main_smem_layout(MODE, B, TPT, a.chunk, n_phase, n_mag, a.table_smem,
+    const MainSmemLayout lay = main_smem_layout(LAYMODE, B, TPT, a.chunk, n_phase, n_mag, a.table_smem,
                                                 range, a.half);
     unsigned long long *s_tab = reinterpret_cast<unsigned long long *>(smem);
     point_t *s_pts = reinterpret_cast<point_t *>(smem + lay.pts);
@@ -712,7 +801,8 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
 
     for (int i = tid; i < a.table_smem; i += B) s_tab[i] = a.table[i];
 
-    const point_t *g_pts = reinterpret_cast<const point_t *>(a.payload);
+    // (the binary64 fold of an FP64 job beyond the certified range reads tau)
+    const point_t *g_pts = reinterpret_cast<const point_t *>(MODE == LAYMODE ? a.payload : a.tau);
     const trial_t *g_tr = reinterpret_cast<const trial_t *>(a.trialc);
     unsigned int *my_cnt = s_cnt + tid;
     // counters start at zero; every work item's final sweep clears the words it
@@ -750,6 +840,7 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
     typename Fold<MODE>::prep_t tc[TPT];
     long long tt[TPT];
     bool pdot = false, k0 = true;
+    unsigned int margin = 0u;  // FP64: the certified fold's margin (0: no trial in the grid)
     bool red = false;  // SPLIT32: this warp's folds re-reduce the residual (narrow window)
     const bool pdm = a.pd_major != 0;
     int wl[TPT];           // word offset (from my_cnt) of each trial's first window slot
@@ -791,6 +882,7 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
         if (tile != cur_tile) {
             cur_tile = tile;
             bool any_pdot = false, all_k0 = true;
+            margin = 0u;
             // trial indices (n_trials marks a slot past the grid): a run of B x TPT
             // flat indices, or B periods x TPT Pdot values (period-major tiles)
             long long p_idx = 0;
@@ -813,11 +905,19 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
                     any_pdot |= Fold<MODE>::has_pdot(tr);
                 }
                 tc[s] = Fold<MODE>::prepare(tr);
+                if constexpr (CERT) {
+                    if (tt[s] < a.n_trials) margin = max(margin, Fold<MODE>::margin(tc[s]));
+                    else Fold<MODE>::park(tc[s], n_phase);
+                }
                 all_k0 &= Fold<MODE>::k_zero(tc[s]);
+            }
+            if constexpr (CERT) {
+#pragma unroll
+                for (int s = 0; s < TPT; ++s) tc[s].C += margin;
             }
             // the fold variant is chosen per warp (a warp vote, no CTA barrier)
             pdot = __any_sync(0xffffffffu, any_pdot);
-            k0 = MODE != GCE_PHASE_FIXED32 || __all_sync(0xffffffffu, all_k0);
+            k0 = (MODE != GCE_PHASE_FIXED32 && !CERT) || __all_sync(0xffffffffu, all_k0);
             // live logical slots [L, R] of this warp's counters (warp-uniform)
             int L = 0, R = n_phase - 1;
             if (SPLIT) {
@@ -896,21 +996,37 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
                     const unsigned int inc = pk2 ? ((ended & 1) ? kPk2IncB : 1u) + kPk2IncC : 1u;
                     compiler_fence();
                     const void *pp = s_pts;
+                    unsigned int near = 0xffffffffu;
                     constexpr bool HP = MODE != GCE_PHASE_FP64;  // half points exist
                     if (k0) {
-                        if (pdot) count_points_any<MODE, TPT, SH, true, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
+                        if (pdot) count_points_any<MODE, TPT, SH, true, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
                         // (red: the warp's slot window is the narrow one, so its folds
                         // must re-reduce, with half points as with whole ones)
-                        else if (SPLIT && red && half) count_points_any<MODE, TPT, SH, false, true, SPLIT, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
-                        else if (SPLIT && red) count_points_any<MODE, TPT, SH, false, true, SPLIT>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
-                        else if (HP && half) count_points_any<MODE, TPT, SH, false, true, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
-                        else count_points_any<MODE, TPT, SH, false, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
-                    } else if (MODE == GCE_PHASE_FIXED32) {
-                        if (pdot) count_points_any<MODE, TPT, SH, true, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
-                        else if (half) count_points_any<MODE, TPT, SH, false, false, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
-                        else count_points_any<MODE, TPT, SH, false, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc);
+                        else if (SPLIT && red && half) count_points_any<MODE, TPT, SH, false, true, SPLIT, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                        else if (SPLIT && red) count_points_any<MODE, TPT, SH, false, true, SPLIT>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                        else if (HP && half) count_points_any<MODE, TPT, SH, false, true, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                        else count_points_any<MODE, TPT, SH, false, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                    } else if (MODE == GCE_PHASE_FIXED32 || CERT) {
+                        if (pdot) count_points_any<MODE, TPT, SH, true, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                        else if (half) count_points_any<MODE, TPT, SH, false, false, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                        else count_points_any<MODE, TPT, SH, false, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
                     }
                     compiler_fence();
+                    if constexpr (CERT) {
+                        if (near < 2u * margin * (unsigned int)n_phase) {
+                            // undecided points in this run: decide them before the
+                            // counts are read
+#pragma unroll
+                            for (int s = 0; s < TPT; ++s) {
+                                if (tt[s] >= a.n_trials) continue;
+                                const long long q = tt[s] / a.n_periods;
+                                recount_near<SH>(reinterpret_cast<const FixedTrial *>(a.trialc) + tt[s],
+                                                 a.tau + off + lo, a.periods[tt[s] - q * a.n_periods],
+                                                 a.pdots[q], pp, half, ka - lo, kb - lo, base[s], inc, margin, fk);
+                            }
+                            compiler_fence();
+                        }
+                    }
                 }
                 if (s1 > s0 && s1 > lo && s1 <= hi) {
                     // end of non-empty magnitude segment i: sweep its counts (FMT_PK2:
@@ -998,6 +1114,25 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
     }
 }
 
+// The CE kernel.  An FP64 job runs the certified fold (MODE kFoldCertified), or,
+// where its range is beyond that fold or the host laid it out for binary64 alone
+// (no payload), the binary64 fold on every point.  Binary64 arithmetic runs at 2
+// lanes per clock and SM and bounds that fold: 19.4 ms on 100 curves x 1000 points
+// x 2e4 periods, 22.5 ms on 23 x 487 x 1e4 x 16 Pdot.  The certified fold, bound
+// like FIXED32 by the integer multiplies of the FMA-heavy pipe and by latency,
+// takes 1.13 and 1.33 ms for the same counts.
+template <int MODE, int TPT, int LOG2B, int KV>
+__global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k_main(MainArgs a) {
+    __shared__ long long s_item;
+    if (a.state->err) return;  // inputs failed the device checks: no work
+    if constexpr (MODE == kFoldCertified) {
+        if (a.payload == nullptr || a.state->wide) {
+            ce_items<GCE_PHASE_FP64, MODE, TPT, LOG2B, KV>(a, s_item);
+            return;
+        }
+    }
+    ce_items<MODE, MODE, TPT, LOG2B, KV>(a, s_item);
+}
 
 template <int MODE, int TPT, int LOG2B>
 cudaError_t launch_main_t(int grid, size_t smem, const MainArgs &a, cudaStream_t s) {

@@ -18,6 +18,7 @@ __global__ void k_init(JobState *st) {
     st->pdot_max_bits = 0ull;
     st->err = 0u;
     st->work = 0ull;
+    st->wide = 0u;
 }
 
 // Non-negative binary64 values order like their bit patterns, so maxima and
@@ -76,6 +77,15 @@ __global__ void k_scan(const double *__restrict__ times, const double *__restric
     }
 }
 
+// Whether an FP64 job is beyond the certified fold's range (from the job's
+// maxima, so every thread that asks agrees).
+__device__ inline bool beyond_certified(const JobState *st, int e_tau) {
+    const double pmin = __longlong_as_double((long long)st->pmin_bits);
+    const double dmax = __longlong_as_double((long long)st->pdot_max_bits);
+    const double fmax_ = 1.0 / pmin;
+    return !fixed_range_ok(fmax_, 0.5 * dmax * fmax_ * fmax_, e_tau);
+}
+
 // Per flat trial t = q n_periods + p: f = 1/P, a = (0.5 Pdot) f f (the oracle's
 // sequence), stored in the fold mode's format.
 template <int MODE>
@@ -97,19 +107,23 @@ __global__ void k_trials(TrialArgs a) {
                 // |x| < 1 needs |c| + |c2| < 1/2: cycles < 2^21 and Pdot cycles < 2^19
                 bad = tau_max * fmax_ >= 2097152.0 || amax * tau_max * tau_max >= 524288.0;
             } else if (MODE == GCE_PHASE_FIXED32) {
-                // F < 2^63, and the Pdot cross term small enough for its FP32 path
-                bad = ldexp(fmax_, fs.e_tau) >= 536870912.0 ||
-                      ldexp(amax, 2 * fs.e_tau) >= 262144.0;
+                bad = !fixed_range_ok(fmax_, amax, fs.e_tau);
             }
             if (bad) atomicOr(&a.state->err, ERR_RANGE);
         }
+        if (MODE == kFoldCertified) a.state->wide = beyond_certified(a.state, fs.e_tau) ? 1u : 0u;
     }
+    const bool wide = MODE == kFoldCertified && beyond_certified(a.state, fs.e_tau);
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (long long)gridDim.x * blockDim.x) {
         const int p = (int)(t % a.n_periods);
         const int q = (int)(t / a.n_periods);
         const double f = 1.0 / a.periods[p];
         const double aa = (0.5 * a.pdots[q]) * f * f;
+        if (MODE == kFoldCertified && wide) {  // {f, a}, read by the binary64 fold
+            reinterpret_cast<double2 *>(a.trialc)[t] = make_double2(f, aa);
+            continue;
+        }
         trial_t v;
         if constexpr (MODE == GCE_PHASE_FP64) {
             v.x = f;
@@ -360,6 +374,7 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
             v.y = 0x4B000000u | (t0 >> 9);                               // 2^23 + (T0 >> 9)
             v.z = (unsigned int)u1;
             v.w = 0x4B000000u | (((unsigned int)u0 ^ 0x80000000u) >> 9);  // 2^23 + ((U0+2^31) >> 9)
+            if (MODE == kFoldCertified) a.tau[lo + pos] = tau;
         }
         out[pos] = v;
     }
@@ -403,6 +418,7 @@ cudaError_t launch_trials(int mode, const TrialArgs &a, cudaStream_t s) {
     switch (mode) {
         case GCE_PHASE_FP64: k_trials<GCE_PHASE_FP64><<<g, 256, 0, s>>>(a); break;
         case GCE_PHASE_SPLIT32: k_trials<GCE_PHASE_SPLIT32><<<g, 256, 0, s>>>(a); break;
+        case kFoldCertified: k_trials<kFoldCertified><<<g, 256, 0, s>>>(a); break;
         default: k_trials<GCE_PHASE_FIXED32><<<g, 256, 0, s>>>(a); break;
     }
     return cudaGetLastError();
@@ -421,6 +437,7 @@ cudaError_t launch_prep(int mode, const PrepArgs &a, cudaStream_t s) {
     switch (mode) {
         case GCE_PHASE_FP64: k_prep<GCE_PHASE_FP64><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
         case GCE_PHASE_SPLIT32: k_prep<GCE_PHASE_SPLIT32><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
+        case kFoldCertified: k_prep<kFoldCertified><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
         default: k_prep<GCE_PHASE_FIXED32><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
     }
     return cudaGetLastError();

@@ -65,11 +65,11 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // Layout of one call inside g_scratch: the c ln c table first (filled once per
 // device), then the per-call buffers.
 struct Layout {
-    size_t state, offsets, order, seg, trialc, payload, cand, end;
+    size_t state, offsets, order, seg, trialc, payload, tau, cand, end;
 };
 
 Layout layout(long long n_points, int n_curves, long long n_trials, int n_mag, int point_bytes,
-              long long n_lists, int k) {
+              int tau_bytes, long long n_lists, int k) {
     Layout L;
     size_t o = align256(8 * kTableEntries);
     L.state = o;
@@ -84,6 +84,8 @@ Layout layout(long long n_points, int n_curves, long long n_trials, int n_mag, i
     o = align256(o + 32 * (size_t)n_trials);
     L.payload = o;
     o = align256(o + (size_t)point_bytes * (size_t)n_points);
+    L.tau = o;
+    o = align256(o + (size_t)tau_bytes * (size_t)n_points);
     L.cand = o;
     o = align256(o + 8 * (size_t)n_curves * (size_t)n_lists * (size_t)k);
     L.end = o;
@@ -155,7 +157,8 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     for (const void *a : arrays)
         if (!on_device(a, dev)) return fail(GCE_ERR_INVALID, "an array is on another device");
     cudaStream_t s = (cudaStream_t)stream;
-    const int mode = cfg->phase_mode;
+    // FP64 jobs run the CE kernel's certified fold
+    const int kmode = cfg->phase_mode == GCE_PHASE_FP64 ? (int)kFoldCertified : cfg->phase_mode;
 
     // launch shape: block 256, 2 trials per thread, the curve staged in chunks
     long long n_max = 1;
@@ -167,25 +170,32 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     int chunk = (int)((n_max + 31) / 32 * 32);
     if (chunk > 1024) chunk = 1024;
     int table_smem = (int)(n_max + 1 < 1024 ? n_max + 1 : 1024);
-    const int range = (mode == GCE_PHASE_SPLIT32 && n_pdots > 1) ? RANGE_NARROW : RANGE_WIDE;
-    const int half = (mode != GCE_PHASE_FP64 && n_pdots == 1) ? 1 : 0;
-    const size_t smem = main_smem_bytes(mode, block, tpt, chunk, cfg->n_phase_bins,
+    const int range = (kmode == GCE_PHASE_SPLIT32 && n_pdots > 1) ? RANGE_NARROW : RANGE_WIDE;
+    const int half = n_pdots == 1 ? 1 : 0;
+    const size_t smem = main_smem_bytes(kmode, block, tpt, chunk, cfg->n_phase_bins,
                                         cfg->n_mag_bins, table_smem, range, half);
     const int kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
-    if (smem > main_dynamic_smem_limit(mode, tpt, block, kv, (size_t)d->smem_optin))
+    if (smem > main_dynamic_smem_limit(kmode, tpt, block, kv, (size_t)d->smem_optin))
         return fail(GCE_ERR_UNSUPPORTED, "bin counts too large for this entry point");
     const TileGrid tg = tile_grid(n_periods, n_pdots, block, tpt);
     const long long n_tiles = tg.n_tiles;
-    const int point_bytes = mode == GCE_PHASE_FP64 ? 8 : 16;
     const long long n_lists = n_tiles * (block / 32);  // one candidate list per warp and tile
-    const Layout L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, point_bytes, n_lists, k);
+    // the certified payload and its tau take 24 bytes per point; where they don't
+    // fit, the binary64 payload's 8 may
+    int mode = kmode;
+    Layout L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 16,
+                      kmode == kFoldCertified ? 8 : 0, n_lists, k);
+    if (L.end > kScratchBytes && kmode == kFoldCertified) {
+        mode = GCE_PHASE_FP64;
+        L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 8, 0, n_lists, k);
+    }
     if (L.end > kScratchBytes)
         return fail(GCE_ERR_NOMEM, "job needs more than the 32 MiB of built-in scratch");
 
-    e = main_kernel_attrs(mode, tpt, block, kv, (size_t)d->smem_optin);
+    e = main_kernel_attrs(kmode, tpt, block, kv, (size_t)d->smem_optin);
     if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, main_kernel_ptr(mode, tpt, block, kv), block, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, main_kernel_ptr(kmode, tpt, block, kv), block, smem);
     if (e != cudaSuccess || occ < 1) return fail(GCE_ERR_CUDA, "occupancy query failed");
     const long long n_items = (long long)n_curves * n_tiles;
     long long grid = (long long)d->n_sm * occ;
@@ -220,13 +230,17 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     pa.t0 = cfg->t0;
     pa.payload = b + L.payload;
     pa.seg = reinterpret_cast<int *>(b + L.seg);
+    pa.tau = reinterpret_cast<double *>(b + L.tau);
     pa.state = state;
     pa.bands = nullptr;
     pa.band_stats = nullptr;
     pa.n_bands = 0;
     if ((e = launch_prep(mode, pa, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     MainArgs ma;
-    ma.payload = b + L.payload;
+    ma.payload = mode == GCE_PHASE_FP64 ? nullptr : b + L.payload;
+    ma.tau = reinterpret_cast<const double *>(b + (mode == GCE_PHASE_FP64 ? L.payload : L.tau));
+    ma.periods = periods;
+    ma.pdots = pdots;
     ma.offsets = offsets;
     ma.seg = reinterpret_cast<const int *>(b + L.seg);
     ma.trialc = b + L.trialc;
@@ -256,7 +270,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     ma.half = half;
     ma.kv = kv;
     ma.state = state;
-    if ((e = launch_main(mode, tpt, block, (int)grid, smem, ma, s)) != cudaSuccess)
+    if ((e = launch_main(kmode, tpt, block, (int)grid, smem, ma, s)) != cudaSuccess)
         return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     e = launch_topk_merge(ma.cand, n_curves, (int)n_lists, k, topk_H, (long long *)topk_idx,
                           nullptr, nullptr, nullptr, nullptr, state, s);

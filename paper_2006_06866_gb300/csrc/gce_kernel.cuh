@@ -186,12 +186,16 @@ template <> struct Fold<kFoldCertified> {
     __device__ __forceinline__ static void park(prep_t &p, int n_phase) {
         p.C += 0x80000000u / (unsigned int)n_phase;
     }
+    // bin = hi32(w), lo = lo32(w): the two registers of one widening multiply (the
+    // product as a 64-bit C value cost two more instructions per point-trial, 14 %
+    // of the kernel's time at 256 threads x 2 trials)
     template <bool PDOT, bool K0>
-    __device__ __forceinline__ static unsigned long long bins(unsigned int fpart, uint4 p,
-                                                              const prep_t &t,
-                                                              const FoldConst &k) {
-        return (unsigned long long)fold_fixed_phase_from<PDOT, K0>(fpart, p, t) *
-               (unsigned int)k.n_phase;
+    __device__ __forceinline__ static void bins(unsigned int fpart, uint4 p, const prep_t &t,
+                                                const FoldConst &k, unsigned int &bin,
+                                                unsigned int &lo) {
+        asm("{.reg .u64 w; mul.wide.u32 w, %2, %3; mov.b64 {%0, %1}, w;}"
+            : "=r"(lo), "=r"(bin)
+            : "r"(fold_fixed_phase_from<PDOT, K0>(fpart, p, t)), "r"((unsigned int)k.n_phase));
     }
     __device__ __forceinline__ static bool has_pdot(const FixedTrial &t) {
         return (t.i.z | t.i.w) != 0u;
@@ -258,10 +262,10 @@ __device__ __forceinline__ void count_point_cert(const uint4 &p, const CertPrep 
     if (SHARED) fp = fold_fixed_fpart(p, tc[0]);
 #pragma unroll
     for (int s = 0; s < TPT; ++s) {
-        const unsigned long long w = Fold<kFoldCertified>::bins<PDOT, K0>(
-            SHARED ? fp : fold_fixed_fpart(p, tc[s]), p, tc[s], fk);
-        lo[s] = (unsigned int)w;
-        bump<kFoldCertified, SH>(base[s], (unsigned int)(w >> 32) << SH, fk, inc);
+        unsigned int bin;
+        Fold<kFoldCertified>::bins<PDOT, K0>(SHARED ? fp : fold_fixed_fpart(p, tc[s]), p, tc[s], fk,
+                                             bin, lo[s]);
+        bump<kFoldCertified, SH>(base[s], bin << SH, fk, inc);
     }
     if (TPT == 1) near = min(near, lo[0]);
 #pragma unroll
@@ -286,10 +290,9 @@ __device__ __noinline__ void recount_near(const FixedTrial *tr, const double *ta
         typedef ModeTraits<kFoldCertified> MT;
         const uint4 p = half ? MT::widen(static_cast<const uint2 *>(pts)[k])
                              : static_cast<const uint4 *>(pts)[k];
-        const unsigned long long w =
-            Fold<kFoldCertified>::bins<true, false>(fold_fixed_fpart(p, t), p, t, fk);
-        if ((unsigned int)w >= thr) continue;
-        const unsigned int bin = (unsigned int)(w >> 32);
+        unsigned int bin, lo;
+        Fold<kFoldCertified>::bins<true, false>(fold_fixed_fpart(p, t), p, t, fk, bin, lo);
+        if (lo >= thr) continue;
         const unsigned int j = (unsigned int)fold_fp64<true>(tau[k], f, a, fk.nphi_d, fk.n_phase);
         if (j == bin) continue;
         bump<kFoldCertified, SH>(base, bin << SH, fk, 0u - inc);

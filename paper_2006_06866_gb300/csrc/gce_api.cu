@@ -164,15 +164,59 @@ static int ilog2_ceil(long long v) {
     return e;
 }
 
-static gce_tuning default_tuning(int mode, int n_max) {
+static int most_tpt(int mode) { return mode == GCE_PHASE_FP64 ? 2 : 4; }
+
+// The counter range of a job's SPLIT32 fold: narrow with a Pdot axis (every fold
+// re-reduced), else the shape's (mid: warps with many cycles re-reduce).
+static int split_range(int mode, int n_pdots, int slot_range) {
+    if (mode != GCE_PHASE_SPLIT32) return RANGE_WIDE;
+    return n_pdots > 1 ? RANGE_NARROW : slot_range == 1 ? RANGE_MID : RANGE_WIDE;
+}
+
+// The launch shape of a job that was not tuned: 128 threads, and as many trials per
+// thread as leave about 16 warps of counters on an SM.  More trials share a point's
+// loads (and with a Pdot axis its period part) and give the fold independent chains;
+// more warps hide the sweeps.  SM cycles per warp and point-trial, 40 curves x 600
+// points x 1e5 trials, SPLIT32 / FIXED32, against the shape used before (256 x 2):
+//   15 bins 128 x 4 3.53 / 4.53 (3.80 / 4.78), 20 bins 3.89 / 4.75 (4.11 / 5.08), 24
+//   bins 4.41 / 5.02 and 128 x 2 4.29 / 5.08; 16 Pdot values: 15 bins 128 x 4 4.59 /
+//   5.13 (5.51 / 6.02), 31 bins 5.78 / 6.47 (6.29 / 6.87), 40 bins 7.27 / 8.23 and
+//   128 x 2 6.93 / 7.46; 50 bins 128 x 2 6.67 / 7.50 (8.84 / 7.18), 50 overlapping
+//   bins 128 x 1 6.12 / 7.03 (9.15 / 7.22) and with Pdot 128 x 2 8.01 / 9.08 (8.01 /
+//   8.77); 100 bins 128 x 1 11.2 / 11.6 (29.2 / 13.8).
+static gce_tuning default_tuning(const gce_config *cfg, int pd_axis) {
+    const int mode = cfg->phase_mode;
+    const bool overlap = (cfg->flags & GCE_FLAG_OVERLAP) != 0;
     gce_tuning t;
-    t.block = 256;
-    t.tpt = 2;
+    t.block = 128;
     t.ctas_per_sm = 0;
-    t.chunk = mode == GCE_PHASE_FP64 ? 4096 : 2048;
-    t.slot_range = 0;
-    (void)n_max;
+    t.chunk = 2048;
+    t.slot_range = 1;
+    const int slots = slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, pd_axis ? 2 : 1, 1));
+    t.tpt = slots <= (pd_axis ? 33 : 26) ? 4 : slots <= (overlap && !pd_axis ? 48 : 64) ? 2 : 1;
+    t.tpt = std::min(t.tpt, most_tpt(mode));
     return t;
+}
+
+// Fewer trials per thread where the job's trials would not fill the device
+// otherwise.  w: warps per scheduler with one trial per thread.  SM cycles per warp
+// and point-trial of 300-point curves, SPLIT32 at 1 / 2 / 4 trials per thread: w =
+// 2.6 16.3 / 18.9 / -, w = 5.1 13.6 / 10.8 / 13.1, w = 8.2 - / 8.9 / 9.8, w = 16 - /
+// 6.9 / 7.5, w = 41 - / 5.8 / 5.7; FP64, whose warps wait longer, w = 8.2 12.8 / 13.8,
+// w = 16 10.5 / 9.2.
+// Jobs with the significance keep at least two wherever 256 threads x 2 trials have
+// always fitted (100 slots): its moments are summed per list of 64 trials.
+static void fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_trials,
+                       int n_curves, int n_sm, bool stats) {
+    const int mode = cfg->phase_mode;
+    const long long warps = (n_trials + 31) / 32 * n_curves, schedulers = 4ll * n_sm;
+    const bool few = warps <= (mode == GCE_PHASE_FP64 ? 9 : 3) * schedulers;
+    if (warps <= 20 * schedulers) t.tpt = std::min(t.tpt, 2);
+    if (few && !stats) t.tpt = 1;
+    if (stats && slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, n_pdots, 0)) <= 100) {
+        t.tpt = std::max(t.tpt, 2);
+        if (few) t.block = 64;
+    }
 }
 
 static bool tuning_ok(const gce_tuning &t, int mode) {
@@ -188,13 +232,16 @@ static TuneKey tune_key(const gce_config *cfg, int n_obs, int pd_axis) {
                    ilog2_ceil(std::max(n_obs, 1)), pd_axis);
 }
 
-// The cached shape for the key; a Pdot-axis job without its own entry uses the
-// plain one.
-static gce_tuning lookup_tuning(gce_handle h, const gce_config *cfg, int n_max, int pd_axis) {
+// The cached shape for the key (a Pdot-axis job without its own entry uses the
+// plain one), or the default one (*tuned = false).
+static gce_tuning lookup_tuning(gce_handle h, const gce_config *cfg, int n_max, int pd_axis,
+                                bool *tuned = nullptr) {
+    if (tuned) *tuned = true;
     auto it = h->tune.find(tune_key(cfg, n_max, pd_axis));
+    if (it == h->tune.end() && pd_axis) it = h->tune.find(tune_key(cfg, n_max, 0));
     if (it != h->tune.end()) return it->second;
-    if (pd_axis) return lookup_tuning(h, cfg, n_max, 0);
-    return default_tuning(cfg->phase_mode, n_max);
+    if (tuned) *tuned = false;
+    return default_tuning(cfg, pd_axis);
 }
 
 extern "C" const char *gce_status_string(gce_status s) {
@@ -314,7 +361,8 @@ struct Job {
 
 struct Plan {
     long long n_points, n_trials, n_items, n_long_items;
-    long long n_lists;    // top-k candidate lists (and moment records) per curve: tiles x warps
+    long long n_lists;    // top-k candidate lists per curve: tiles x warps
+    int stats_per;        // moment records per candidate list
     int n_long, n_short;  // curves taken curve-major / tile-major (see MainArgs)
     int n_max, n_tiles, n_ptiles, pd_major, range, half, kv, block, tpt, grid, chunk, table_smem,
         grab;
@@ -336,13 +384,12 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     long long nmax = 1;
     for (int c = 0; c < j.n_curves; ++c) nmax = std::max<long long>(nmax, j.h_offsets[c + 1] - j.h_offsets[c]);
     pl.n_max = (int)nmax;
-    const gce_tuning t = j.force ? *j.force : lookup_tuning(h, cfg, pl.n_max, j.n_pdots > 1 ? 1 : 0);
+    bool tuned = true;
+    gce_tuning t = j.force ? *j.force : lookup_tuning(h, cfg, pl.n_max, j.n_pdots > 1 ? 1 : 0, &tuned);
+    if (!tuned)
+        fit_to_job(t, cfg, j.n_pdots, pl.n_trials, j.n_curves, h->n_sm, j.rho != nullptr);
     const int kk = j.kind == JOB_TOPK ? j.k : 0;
-    // SPLIT32's kept slot range: narrow with a Pdot axis (every fold re-reduced),
-    // else the tuned one (mid: warps with many cycles re-reduce)
-    pl.range = RANGE_WIDE;
-    if (cfg->phase_mode == GCE_PHASE_SPLIT32)
-        pl.range = j.n_pdots > 1 ? RANGE_NARROW : t.slot_range == 1 ? RANGE_MID : RANGE_WIDE;
+    pl.range = split_range(cfg->phase_mode, j.n_pdots, t.slot_range);
     // one Pdot value: the staging holds 8-byte half points
     pl.half = j.n_pdots == 1 ? 1 : 0;
     const int kmode = kernel_mode(cfg->phase_mode);
@@ -422,7 +469,7 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
         }
         h->shapes[skey] = LaunchShape{pl.block, pl.tpt, pl.chunk, pl.table_smem, occ, pl.smem};
     }
-    const TileGrid tg = tile_grid(j.n_periods, j.n_pdots, pl.block, pl.tpt);
+    const TileGrid tg = job_tiles(j.n_periods, j.n_pdots, pl.block, pl.tpt);
     pl.n_tiles = (int)tg.n_tiles;
     pl.n_ptiles = tg.n_ptiles;
     pl.pd_major = tg.pd_major;
@@ -434,8 +481,9 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
         if (j.h_offsets[c + 1] - j.h_offsets[c] <= kShortCurve) ++pl.n_short;
     pl.n_long = j.n_curves - pl.n_short;
     pl.n_long_items = (long long)pl.n_long * pl.n_tiles;
-    // each warp of a tile writes its own candidate list and moments
+    // each warp of a tile writes its own candidate list and its trial lists' moments
     pl.n_lists = (long long)pl.n_tiles * (pl.block / 32);
+    pl.stats_per = pl.tpt == 4 ? 2 : 1;
     pl.n_groups = j.kind == JOB_TOPK ? topk_groups(pl.n_lists, j.k, &pl.tiles_per_group) : 0;
     if (j.kind != JOB_TOPK) pl.tiles_per_group = 0;
     if (t.ctas_per_sm > 0) occ = std::min(occ, t.ctas_per_sm);
@@ -562,16 +610,16 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
                 TileStats *stats2 = j.rho ? (TileStats *)h->stats2.p : nullptr;
                 CUDA_TRY(h, launch_topk_reduce((const unsigned long long *)h->cand.p, j.n_curves,
                                                (int)pl.n_lists, j.k, pl.tiles_per_group, pl.n_groups,
-                                               ma.stats, (unsigned long long *)h->cand2.p, stats2,
+                                               pl.stats_per, ma.stats, (unsigned long long *)h->cand2.p, stats2,
                                                st, s));
                 CUDA_TRY(h, launch_topk_merge((const unsigned long long *)h->cand2.p, j.n_curves,
-                                              pl.n_groups, j.k, j.topk_H, (long long *)j.topk_idx,
+                                              pl.n_groups, j.k, 1, j.topk_H, (long long *)j.topk_idx,
                                               stats2, j.mean, j.std_dev, j.rho, st, s));
                 n_launch += 2;
             } else {
                 CUDA_TRY(h, launch_topk_merge((const unsigned long long *)h->cand.p, j.n_curves,
-                                              (int)pl.n_lists, j.k, j.topk_H, (long long *)j.topk_idx,
-                                              ma.stats, j.mean, j.std_dev, j.rho, st, s));
+                                              (int)pl.n_lists, j.k, pl.stats_per, j.topk_H,
+                                              (long long *)j.topk_idx, ma.stats, j.mean, j.std_dev, j.rho, st, s));
                 ++n_launch;
             }
             break;
@@ -670,7 +718,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
         (st = ensure(h, h->cand, 8 * (size_t)j.n_curves * pl.n_lists * j.k)) != GCE_OK)
         return st;
     if (j.kind == JOB_TOPK && j.rho &&
-        (st = ensure(h, h->stats, sizeof(TileStats) * (size_t)j.n_curves * pl.n_lists)) != GCE_OK)
+        (st = ensure(h, h->stats, sizeof(TileStats) * (size_t)j.n_curves * pl.n_lists * pl.stats_per)) != GCE_OK)
         return st;
     if (j.kind == JOB_TOPK && pl.n_groups > 0 &&
         (st = ensure(h, h->cand2, 8 * (size_t)j.n_curves * pl.n_groups * j.k)) != GCE_OK)
@@ -1001,8 +1049,8 @@ static std::vector<gce_tuning> tune_candidates(int mode, int n_obs, int slot_ran
         for (int tp : tpts)
             for (int ch : chunks) {
                 if (ch > 512 && ch >= 2 * n_obs) continue;  // same plan as a smaller chunk
-                if (tp == 4 && mode == GCE_PHASE_FP64) continue;  // not built
-                gce_tuning c = default_tuning(mode, n_obs);
+                if (tp > most_tpt(mode)) continue;  // not built
+                gce_tuning c{};
                 c.block = b;
                 c.tpt = tp;
                 c.chunk = ch;
@@ -1089,7 +1137,7 @@ extern "C" gce_status gce_autotune_job(gce_handle h, const double *times, const 
     cudaStream_t s = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     gce_status result = GCE_OK;
-    gce_tuning best = default_tuning(cfg->phase_mode, (int)nmax);
+    gce_tuning best = default_tuning(cfg, n_pdots > 1 ? 1 : 0);
     gce_config c2cfg = *cfg;
     c2cfg.flags = (c2cfg.flags | GCE_FLAG_NO_GRAPH) & ~GCE_FLAG_TIME_KERNEL;
     do {
@@ -1164,7 +1212,7 @@ extern "C" gce_status gce_autotune(gce_handle h, const gce_config *cfg, int32_t 
     cudaStream_t s = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     gce_status result = GCE_OK;
-    gce_tuning best[2] = {default_tuning(cfg->phase_mode, n_obs), default_tuning(cfg->phase_mode, n_obs)};
+    gce_tuning best[2] = {default_tuning(cfg, 0), default_tuning(cfg, 1)};
     gce_config c2 = *cfg;
     c2.flags |= GCE_FLAG_NO_GRAPH;
     do {

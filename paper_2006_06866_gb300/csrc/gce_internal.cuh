@@ -524,6 +524,29 @@ inline TileGrid tile_grid(long long n_periods, long long n_pdots, int block, int
     return g;
 }
 
+// Trial lists.  The trials of a warp whose threads have two or four are one or two
+// lists of 64, and the moments of Eq. 5 are summed per list, so that they come out
+// the same in every launch shape: flat list l holds trials t and t + 256 for the 32
+// consecutive t from 512 (l / 8) + 32 (l % 8); with several Pdot values a list is 32
+// consecutive periods x 2 consecutive Pdot values (tile_grid's tiles).
+__host__ __device__ inline long long flat_list_trial(long long l) {
+    return (l >> 3) * 512 + (l & 7) * 32;
+}
+inline long long flat_lists(long long n_trials) {
+    const long long rest = n_trials % 512;
+    return n_trials / 512 * 8 + (rest >= 256 ? 8 : (rest + 31) / 32);
+}
+// The tiles of a job: flat jobs with two or four trials per thread are cut into
+// runs of block x tpt / 64 lists.
+inline TileGrid job_tiles(long long n_periods, long long n_pdots, int block, int tpt) {
+    TileGrid g = tile_grid(n_periods, n_pdots, block, tpt);
+    if (!g.pd_major && tpt > 1) {
+        const long long per = (long long)block * tpt / 64;
+        g.n_tiles = (flat_lists(n_periods * n_pdots) + per - 1) / per;
+    }
+    return g;
+}
+
 struct MainArgs {
     const void *payload;
     const long long *offsets;
@@ -605,8 +628,9 @@ GCE_MAIN_TU(fixed32, 4)
 #undef GCE_MAIN_TU
 cudaError_t launch_main(int mode, int tpt, int block, int grid, size_t smem,
                         const MainArgs &a, cudaStream_t s);
+// stats: stats_per moment records per candidate list
 cudaError_t launch_topk_merge(const unsigned long long *cand, int n_curves, int n_tiles,
-                              int k, float *topk_H, long long *topk_idx, const TileStats *stats,
+                              int k, int stats_per, float *topk_H, long long *topk_idx, const TileStats *stats,
                               double *mean, double *std_dev, float *rho, const JobState *st,
                               cudaStream_t s);
 cudaError_t launch_single(const MainArgs &a, int curve, long long n_points, cudaStream_t s);

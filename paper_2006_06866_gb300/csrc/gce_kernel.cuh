@@ -886,8 +886,9 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
             cur_tile = tile;
             bool any_pdot = false, all_k0 = true;
             margin = 0u;
-            // trial indices (n_trials marks a slot past the grid): a run of B x TPT
-            // flat indices, or B periods x TPT Pdot values (period-major tiles)
+            // trial indices (n_trials marks a slot past the grid): the warp's lists (one
+            // trial per thread: a run of B flat indices), or B periods x TPT Pdot values
+            // (period-major tiles)
             long long p_idx = 0;
             int q_base = 0;
             if (pdm) {
@@ -900,8 +901,11 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                     tt[s] = (p_idx < a.n_periods && q_base + s < a.n_pdots)
                                 ? (long long)(q_base + s) * a.n_periods + p_idx
                                 : a.n_trials;
+                else if (TPT == 1)
+                    tt[s] = (long long)tile * B + tid;
                 else
-                    tt[s] = (long long)tile * (B * TPT) + (long long)s * B + tid;
+                    tt[s] = flat_list_trial(((long long)tile * (B / 32) + warp) * (TPT / 2) + s / 2) +
+                            (s % 2) * 256 + lane;
                 trial_t tr{};
                 if (tt[s] < a.n_trials) {
                     tr = g_tr[tt[s]];
@@ -1066,36 +1070,40 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
             }
         }
 
-        // each warp writes its own candidate list and moments (list index: curve,
-        // tile, warp), so the tile needs no barrier; the merge kernels take B / 32
-        // lists per tile
+        // each warp writes its own candidate list (index: curve, tile, warp) and the
+        // moments of its trial lists, so the tile needs no barrier; the merge kernels
+        // take B / 32 candidate lists per tile
         const long long list = ((long long)c * a.n_tiles + tile) * (B >> 5) + warp;
         if (a.stats) {
-            // moments of the warp's H for the significance of Eq. 5: sums of H - shift
-            // in FP32 (shift = lane 0's first value, so the sums stay small), then
-            // (count, mean, M2) in FP64
-            const float shift = __shfl_sync(0xffffffffu, hv[0], 0);
-            float s1 = 0.f, s2 = 0.f, cnt = 0.f;
+            // moments of a list's H for the significance of Eq. 5: sums of H - shift in
+            // FP32 (shift = lane 0's first value, so the sums stay small), then (count,
+            // mean, M2) in FP64
+            constexpr int PER = TPT >= 2 ? 2 : 1;
 #pragma unroll
-            for (int s = 0; s < TPT; ++s)
-                if (tt[s] < a.n_trials) {
-                    const float dd = hv[s] - shift;
-                    s1 += dd;
-                    s2 = __fmaf_rn(dd, dd, s2);
-                    cnt += 1.f;
+            for (int l = 0; l < TPT / PER; ++l) {
+                const float shift = __shfl_sync(0xffffffffu, hv[l * PER], 0);
+                float s1 = 0.f, s2 = 0.f, cnt = 0.f;
+#pragma unroll
+                for (int s = l * PER; s < (l + 1) * PER; ++s)
+                    if (tt[s] < a.n_trials) {
+                        const float dd = hv[s] - shift;
+                        s1 += dd;
+                        s2 = __fmaf_rn(dd, dd, s2);
+                        cnt += 1.f;
+                    }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                    s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+                    cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
                 }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-                s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-                cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-            }
-            if (lane == 0) {
-                const double nw = cnt;
-                TileStats *t = a.stats + list;
-                t->n = nw;
-                t->mean = nw > 0 ? (double)shift + (double)s1 / nw : 0.0;
-                t->m2 = nw > 0 ? fmax((double)s2 - (double)s1 * (double)s1 / nw, 0.0) : 0.0;
+                if (lane == 0) {
+                    const double nw = cnt;
+                    TileStats *t = a.stats + list * (TPT / PER) + l;
+                    t->n = nw;
+                    t->mean = nw > 0 ? (double)shift + (double)s1 / nw : 0.0;
+                    t->m2 = nw > 0 ? fmax((double)s2 - (double)s1 * (double)s1 / nw, 0.0) : 0.0;
+                }
             }
         }
 

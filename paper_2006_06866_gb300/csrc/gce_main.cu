@@ -11,7 +11,7 @@ namespace {
 // Per-curve merge of the tiles' candidates: k rounds of "smallest key above the
 // previous one" (keys are unique: H bits in the high word, trial index low).
 __global__ void k_topk_merge(const unsigned long long *__restrict__ cand, int n_tiles, int k,
-                             float *topk_H, long long *topk_idx, const TileStats *stats,
+                             int stats_per, float *topk_H, long long *topk_idx, const TileStats *stats,
                              double *mean_out, double *std_out, float *rho_out, const JobState *st) {
     __shared__ unsigned long long sh[32];
     __shared__ double shs[3 * 32];
@@ -47,8 +47,9 @@ __global__ void k_topk_merge(const unsigned long long *__restrict__ cand, int n_
     // moments merged in a fixed order (each thread a strided run of tiles, then
     // a fixed tree), so the result is deterministic
     double nn = 0.0, mu = 0.0, m2 = 0.0;
-    const TileStats *ts = stats + (long long)c * n_tiles;
-    for (int i = threadIdx.x; i < n_tiles; i += blockDim.x) chan_merge(nn, mu, m2, ts[i].n, ts[i].mean, ts[i].m2);
+    const int n_stats = n_tiles * stats_per;
+    const TileStats *ts = stats + (long long)c * n_stats;
+    for (int i = threadIdx.x; i < n_stats; i += blockDim.x) chan_merge(nn, mu, m2, ts[i].n, ts[i].mean, ts[i].m2);
     for (int o = 1; o < 32; o <<= 1) {
         const double nb = __shfl_down_sync(0xffffffffu, nn, o);
         const double mb = __shfl_down_sync(0xffffffffu, mu, o);
@@ -200,11 +201,11 @@ cudaError_t launch_main(int mode, int tpt, int block, int grid, size_t smem, con
 }
 
 cudaError_t launch_topk_merge(const unsigned long long *cand, int n_curves, int n_tiles, int k,
-                              float *topk_H, long long *topk_idx, const TileStats *stats,
-                              double *mean, double *std_dev, float *rho, const JobState *st,
-                              cudaStream_t s) {
+                              int stats_per, float *topk_H, long long *topk_idx,
+                              const TileStats *stats, double *mean, double *std_dev, float *rho,
+                              const JobState *st, cudaStream_t s) {
     if (n_curves <= 0) return cudaSuccess;
-    k_topk_merge<<<n_curves, 256, 0, s>>>(cand, n_tiles, k, topk_H, topk_idx, stats, mean,
+    k_topk_merge<<<n_curves, 256, 0, s>>>(cand, n_tiles, k, stats_per, topk_H, topk_idx, stats, mean,
                                           std_dev, rho, st);
     return cudaGetLastError();
 }

@@ -177,7 +177,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     const int kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
     if (smem > main_dynamic_smem_limit(kmode, tpt, block, kv, (size_t)d->smem_optin))
         return fail(GCE_ERR_UNSUPPORTED, "bin counts too large for this entry point");
-    const TileGrid tg = tile_grid(n_periods, n_pdots, block, tpt);
+    const TileGrid tg = job_tiles(n_periods, n_pdots, block, tpt);
     const long long n_tiles = tg.n_tiles;
     const long long n_lists = n_tiles * (block / 32);  // one candidate list per warp and tile
     // the certified payload and its tau take 24 bytes per point; where they don't
@@ -272,7 +272,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     ma.state = state;
     if ((e = launch_main(kmode, tpt, block, (int)grid, smem, ma, s)) != cudaSuccess)
         return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
-    e = launch_topk_merge(ma.cand, n_curves, (int)n_lists, k, topk_H, (long long *)topk_idx,
+    e = launch_topk_merge(ma.cand, n_curves, (int)n_lists, k, 1, topk_H, (long long *)topk_idx,
                           nullptr, nullptr, nullptr, nullptr, state, s);
     if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     // device-side input checks: read the flags into host stack memory and wait

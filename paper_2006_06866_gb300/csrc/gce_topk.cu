@@ -45,7 +45,8 @@ __device__ __forceinline__ void merge_moments(double &n, double &mean, double &m
 
 __global__ void __launch_bounds__(kReduceBlock)
     k_topk_reduce(const unsigned long long *__restrict__ cand, int n_tiles, int k,
-                  int tiles_per_group, int n_groups, const TileStats *__restrict__ stats,
+                  int tiles_per_group, int n_groups, int stats_per,
+                  const TileStats *__restrict__ stats,
                   unsigned long long *__restrict__ cand2, TileStats *__restrict__ stats2,
                   const JobState *st) {
     __shared__ unsigned long long s_keys[kReduceKeys];
@@ -84,8 +85,8 @@ __global__ void __launch_bounds__(kReduceBlock)
     // the group's tile moments, merged in a fixed order (a strided run of tiles
     // per thread, a fixed tree within each warp, then the warps in order)
     double nn = 0.0, mu = 0.0, m2 = 0.0;
-    const TileStats *ts = stats + (long long)c * n_tiles + t0;
-    for (int i = threadIdx.x; i < nt; i += kReduceBlock) merge_moments(nn, mu, m2, ts[i].n, ts[i].mean, ts[i].m2);
+    const TileStats *ts = stats + ((long long)c * n_tiles + t0) * stats_per;
+    for (int i = threadIdx.x; i < nt * stats_per; i += kReduceBlock) merge_moments(nn, mu, m2, ts[i].n, ts[i].mean, ts[i].m2);
     for (int o = 1; o < 32; o <<= 1) {
         const double nb = __shfl_down_sync(0xffffffffu, nn, o);
         const double mb = __shfl_down_sync(0xffffffffu, mu, o);
@@ -110,7 +111,8 @@ __global__ void __launch_bounds__(kReduceBlock)
 }  // namespace
 
 cudaError_t launch_topk_reduce(const unsigned long long *cand, int n_curves, int n_tiles, int k,
-                               int tiles_per_group, int n_groups, const TileStats *stats,
+                               int tiles_per_group, int n_groups, int stats_per,
+                               const TileStats *stats,
                                unsigned long long *cand2, TileStats *stats2, const JobState *st,
                                cudaStream_t s) {
     if (n_curves <= 0 || n_groups <= 0) return cudaSuccess;
@@ -118,7 +120,7 @@ cudaError_t launch_topk_reduce(const unsigned long long *cand, int n_curves, int
     const long long blocks = (long long)n_curves * n_groups;
     if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
     k_topk_reduce<<<(unsigned int)blocks, kReduceBlock, 0, s>>>(cand, n_tiles, k, tiles_per_group,
-                                                               n_groups, stats, cand2, stats2, st);
+                                                               n_groups, stats_per, stats, cand2, stats2, st);
     return cudaGetLastError();
 }
 

@@ -206,17 +206,37 @@ static gce_tuning default_tuning(const gce_config *cfg, int pd_axis) {
 // w = 16 10.5 / 9.2.
 // Jobs with the significance keep at least two wherever 256 threads x 2 trials have
 // always fitted (100 slots): its moments are summed per list of 64 trials.
-static void fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_trials,
-                       int n_curves, int n_sm, bool stats) {
+// Returns whether the CTA's warps should share one trial set: their points are then
+// counted 4 or 8 at a time, which pays while a curve's points, walked by a single
+// warp, outlast the barriers.  Against the shapes above, at w = 0.05 / 0.26 / 1.0 /
+// 2.6 / 4.1: 2000 points 286 -> 114, 57 -> 24, 16.9 -> 10.4, 7.8 -> 6.4, 7.6 -> 5.8
+// (FIXED32); 811 points 385 -> 207, 77 -> 47, 22.6 -> 15.5, 10.1 -> 9.1, 9.2 -> 7.9;
+// 300 points 670 -> 532, 139 -> 98, 37 -> 31, 16.7 -> 16.7, 13.8 -> 14.4; 100 points
+// 1600 -> 1400, 320 -> 281, 84 -> 80, 36 -> 38, 29 -> 35.
+static bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_trials,
+                       int n_curves, long long n_points, int n_sm, bool stats) {
     const int mode = cfg->phase_mode;
     const long long warps = (n_trials + 31) / 32 * n_curves, schedulers = 4ll * n_sm;
     const bool few = warps <= (mode == GCE_PHASE_FP64 ? 9 : 3) * schedulers;
+    const bool keep2 =
+        stats && slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, n_pdots, 0)) <= 100;
+    if (!(cfg->flags & GCE_FLAG_OVERLAP)) {
+        const bool very_few = 10 * warps <= 3 * schedulers;
+        // mean points per curve >= 200 w
+        if (very_few || (warps <= 6 * schedulers &&
+                         n_points / n_curves * schedulers >= 200 * warps)) {
+            t.block = very_few ? 256 : 128;
+            t.tpt = very_few && !keep2 ? 1 : 2;
+            return true;
+        }
+    }
     if (warps <= 20 * schedulers) t.tpt = std::min(t.tpt, 2);
     if (few && !stats) t.tpt = 1;
-    if (stats && slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, n_pdots, 0)) <= 100) {
+    if (keep2) {
         t.tpt = std::max(t.tpt, 2);
         if (few) t.block = 64;
     }
+    return false;
 }
 
 static bool tuning_ok(const gce_tuning &t, int mode) {
@@ -386,16 +406,17 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     pl.n_max = (int)nmax;
     bool tuned = true;
     gce_tuning t = j.force ? *j.force : lookup_tuning(h, cfg, pl.n_max, j.n_pdots > 1 ? 1 : 0, &tuned);
-    if (!tuned)
-        fit_to_job(t, cfg, j.n_pdots, pl.n_trials, j.n_curves, h->n_sm, j.rho != nullptr);
+    const bool shared_set = !tuned && fit_to_job(t, cfg, j.n_pdots, pl.n_trials, j.n_curves,
+                                                 pl.n_points, h->n_sm, j.rho != nullptr);
     const int kk = j.kind == JOB_TOPK ? j.k : 0;
     pl.range = split_range(cfg->phase_mode, j.n_pdots, t.slot_range);
     // one Pdot value: the staging holds 8-byte half points
     pl.half = j.n_pdots == 1 ? 1 : 0;
     const int kmode = kernel_mode(cfg->phase_mode);
     pl.prep_mode = (j.kind == JOB_GRID || j.kind == JOB_TOPK) ? kmode : cfg->phase_mode;
-    // the kernel instantiation: overlapping bins or not
+    // the kernel instantiation: overlapping bins, a shared trial set, or neither
     pl.kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
+    if (shared_set && pl.kv == KV_SNAP) pl.kv = KV_SHARED;
     const int kv = pl.kv;
     const ShapeKey skey(cfg->phase_mode, cfg->n_phase_bins, cfg->n_mag_bins, pl.n_max, kk,
                         pl.range * 8 + pl.half * 4 + kv, t.block, t.tpt, t.chunk,
@@ -421,7 +442,7 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
         // shrink the staged chunk, then the table, then trials per thread, then the
         // block, until the CTA fits in shared memory
         auto size = [&]() {
-            return main_smem_bytes(kmode, pl.block, pl.tpt, pl.chunk, cfg->n_phase_bins,
+            return main_smem_bytes(kmode, trial_threads(kv, pl.block), pl.tpt, pl.chunk, cfg->n_phase_bins,
                                    cfg->n_mag_bins, pl.table_smem, pl.range, pl.half);
         };
         auto limit = [&]() {
@@ -469,7 +490,7 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
         }
         h->shapes[skey] = LaunchShape{pl.block, pl.tpt, pl.chunk, pl.table_smem, occ, pl.smem};
     }
-    const TileGrid tg = job_tiles(j.n_periods, j.n_pdots, pl.block, pl.tpt);
+    const TileGrid tg = job_tiles(j.n_periods, j.n_pdots, trial_threads(kv, pl.block), pl.tpt);
     pl.n_tiles = (int)tg.n_tiles;
     pl.n_ptiles = tg.n_ptiles;
     pl.pd_major = tg.pd_major;
@@ -482,7 +503,7 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     pl.n_long = j.n_curves - pl.n_short;
     pl.n_long_items = (long long)pl.n_long * pl.n_tiles;
     // each warp of a tile writes its own candidate list and its trial lists' moments
-    pl.n_lists = (long long)pl.n_tiles * (pl.block / 32);
+    pl.n_lists = (long long)pl.n_tiles * (trial_threads(kv, pl.block) / 32);
     pl.stats_per = pl.tpt == 4 ? 2 : 1;
     pl.n_groups = j.kind == JOB_TOPK ? topk_groups(pl.n_lists, j.k, &pl.tiles_per_group) : 0;
     if (j.kind != JOB_TOPK) pl.tiles_per_group = 0;

@@ -590,10 +590,13 @@ struct MainArgs {
 };
 
 // Instantiations of the CE kernel: without overlapping bins (snapshot counters),
-// and with them (packed two-segment counters for curves of at most 1023 points,
-// snapshot counters for longer ones).
-enum { KV_SNAP = 0, KV_OVL = 1 };
+// with them (packed two-segment counters for curves of at most 1023 points, snapshot
+// counters for longer ones), and for small jobs without them (a CTA's warps share
+// one set of 32 x tpt trials).
+enum { KV_SNAP = 0, KV_OVL = 1, KV_SHARED = 2 };
 inline int kernel_variant(bool overlap) { return overlap ? KV_OVL : KV_SNAP; }
+// threads of a CTA with trials (and counters) of their own
+inline int trial_threads(int kv, int block) { return kv == KV_SHARED ? 32 : block; }
 
 // Kernel launchers (defined in the .cu files).
 cudaError_t launch_init(JobState *st, cudaStream_t s);

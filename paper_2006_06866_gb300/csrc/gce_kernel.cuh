@@ -636,11 +636,13 @@ struct Sweep {
     }
 
     // w0[s]: word offset (from cnt) of trial s's first window slot; e: extra
-    // slots, merged first
-    __device__ __forceinline__ void run(const int (&w0)[TPT], int n, int e,
+    // slots, merged first.  The bins [j, end) are swept (all n of them, but for the
+    // warps of a shared trial set).
+    __device__ __forceinline__ void run(const int (&w0)[TPT], int n, int e, int j, int end,
                                         unsigned long long (&acc)[TPT]) {
         {
             for (int i = 0, b = 0; i < e; ++i, b = (b + 1 == n) ? 0 : b + 1) {
+                if (b < j || b >= end) continue;
 #pragma unroll
                 for (int s = 0; s < TPT; ++s) {
                     unsigned int *q = cnt + w0[s] + (n + i) * STRIDE;
@@ -653,25 +655,24 @@ struct Sweep {
         }
         int w[TPT];
 #pragma unroll
-        for (int s = 0; s < TPT; ++s) w[s] = w0[s];
+        for (int s = 0; s < TPT; ++s) w[s] = w0[s] + j * STRIDE;
         // bins per step: four to eight words in flight, eight bins with one trial
         // per thread (+1 % over four at 50 overlapping bins)
         constexpr int G = TPT * NF >= 4 ? 2 : (TPT == 1 ? 8 : 4);
-        int j = 0;
         if (OVL) {
             step<1, true>(w, acc);
             j = 1;
         }
-        for (; j + G <= n; j += G) step<G, false>(w, acc);
-        if (G > 4 && (n - j) >= 4) {
+        for (; j + G <= end; j += G) step<G, false>(w, acc);
+        if (G > 4 && (end - j) >= 4) {
             step<4, false>(w, acc);
             j += 4;
         }
-        if (G > 2 && (n - j) >= 2) {
+        if (G > 2 && (end - j) >= 2) {
             step<2, false>(w, acc);
             j += 2;
         }
-        if (j < n) step<1, false>(w, acc);
+        if (j < end) step<1, false>(w, acc);
         if constexpr (OVL && F::kPairWords) {
 #pragma unroll
             for (int s = 0; s < TPT; ++s) {
@@ -700,12 +701,13 @@ struct Sweeper {
     int table_smem;
     const unsigned long long *g_tab;
     int n;  // phase bins
+    int j0, j1;  // the warp's share of them
 
     template <int FMT, int KIND>
     __device__ __forceinline__ void run(bool tab_all, const int (&w0)[TPT], int e,
                                         unsigned long long (&acc)[TPT]) const {
-        if (tab_all) Sweep<TPT, FMT, KIND, true, OVL, STRIDE>{cnt, s_tab, table_smem, g_tab}.run(w0, n, e, acc);
-        else Sweep<TPT, FMT, KIND, false, OVL, STRIDE>{cnt, s_tab, table_smem, g_tab}.run(w0, n, e, acc);
+        if (tab_all) Sweep<TPT, FMT, KIND, true, OVL, STRIDE>{cnt, s_tab, table_smem, g_tab}.run(w0, n, e, j0, j1, acc);
+        else Sweep<TPT, FMT, KIND, false, OVL, STRIDE>{cnt, s_tab, table_smem, g_tab}.run(w0, n, e, j0, j1, acc);
     }
 };
 
@@ -762,6 +764,8 @@ __device__ __forceinline__ void chan_merge(double &n, double &mean, double &m2, 
 // the 128-thread kernel with overlapping bins, whose counters in the mid slot
 // range fit five CTAs per SM: 96 registers there (measured 3.6 % faster at 50
 // overlapping bins than four CTAs at 121 registers).
+// the shapes that small jobs are given (fit_to_job)
+constexpr bool shared_set_built(int tpt, int log2b) { return tpt <= 2 && (log2b == 7 || log2b == 8); }
 constexpr int main_min_blocks(int tpt, int log2b, int kv) {
     return (kv == KV_OVL && tpt == 1 && log2b == 7) ? 5 :
            tpt == 2 ? (log2b >= 9 ? 2 : (log2b == 8 ? 3 : (log2b == 7 ? 6 : 8)))
@@ -781,8 +785,16 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     extern __shared__ __align__(16) unsigned char smem[];
 
     constexpr int B = 1 << LOG2B;
-    constexpr int SH = LOG2B + 2;  // log2 of the byte stride between a thread's slots
+    // SHARED_SET: the CTA's warps share one set of 32 x TPT trials, whose counters all
+    // of them increment: each counts a share of a segment's points and sweeps a share
+    // of its bins, between barriers.  TB: threads with trials (and counters) of their
+    // own.
+    constexpr bool SHARED_SET = KV == KV_SHARED;
+    constexpr int WARPS = B / 32, TB = SHARED_SET ? 32 : B;
+    constexpr int SH = (SHARED_SET ? 5 : LOG2B) + 2;  // log2 of the byte stride between a thread's slots
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tb = SHARED_SET ? lane : tid;        // thread and warp within the trial set
+    const int tw = SHARED_SET ? 0 : warp;
     const int n_phase = a.n_phase, n_mag = a.n_mag;
     constexpr bool SPLIT = MODE == GCE_PHASE_SPLIT32;
     constexpr bool CERT = MODE == kFoldCertified;
@@ -791,11 +803,11 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     const SlotRange zr = slot_range(MODE, n_phase, range);
     const int n_slots = slots_per_trial(MODE, n_phase, range);
     const int slot_off = -zr.zmin;  // physical index of logical slot l: l + slot_off
-    const int stride_j = B, stride_s = n_slots * B;
+    const int stride_j = TB, stride_s = n_slots * TB;
 
     // the regions at the offsets the host sized the launch with (the table first,
     // so that its address is a constant)
-    const MainSmemLayout lay = main_smem_layout(LAYMODE, B, TPT, a.chunk, n_phase, n_mag, a.table_smem,
+    const MainSmemLayout lay = main_smem_layout(LAYMODE, TB, TPT, a.chunk, n_phase, n_mag, a.table_smem,
                                                 range, a.half);
     unsigned long long *s_tab = reinterpret_cast<unsigned long long *>(smem);
     point_t *s_pts = reinterpret_cast<point_t *>(smem + lay.pts);
@@ -807,10 +819,10 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     // (the binary64 fold of an FP64 job beyond the certified range reads tau)
     const point_t *g_pts = reinterpret_cast<const point_t *>(MODE == LAYMODE ? a.payload : a.tau);
     const trial_t *g_tr = reinterpret_cast<const trial_t *>(a.trialc);
-    unsigned int *my_cnt = s_cnt + tid;
+    unsigned int *my_cnt = s_cnt + tb;
     // counters start at zero; every work item's final sweep clears the words it
     // used, so later items start from zero as well
-    for (int i = 0; i < TPT * n_slots; ++i) my_cnt[i * B] = 0u;
+    for (int i = SHARED_SET ? warp : 0; i < TPT * n_slots; i += SHARED_SET ? WARPS : 1) my_cnt[i * TB] = 0u;
 #if defined(GCE_CHECK_SLOTS)
     FoldConst fk = fold_const(n_phase);
     fk.zmin = zr.zmin;
@@ -892,7 +904,7 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
             long long p_idx = 0;
             int q_base = 0;
             if (pdm) {
-                p_idx = (long long)(tile % a.n_ptiles) * B + tid;
+                p_idx = (long long)(tile % a.n_ptiles) * TB + tb;
                 q_base = (tile / a.n_ptiles) * TPT;
             }
 #pragma unroll
@@ -902,9 +914,9 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                                 ? (long long)(q_base + s) * a.n_periods + p_idx
                                 : a.n_trials;
                 else if (TPT == 1)
-                    tt[s] = (long long)tile * B + tid;
+                    tt[s] = (long long)tile * TB + tb;
                 else
-                    tt[s] = flat_list_trial(((long long)tile * (B / 32) + warp) * (TPT / 2) + s / 2) +
+                    tt[s] = flat_list_trial(((long long)tile * (TB / 32) + tw) * (TPT / 2) + s / 2) +
                             (s % 2) * 256 + lane;
                 trial_t tr{};
                 if (tt[s] < a.n_trials) {
@@ -970,7 +982,9 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
         // of every other sweep, which pays with overlapping bins and costs more
         // field arithmetic than it saves without them.
         const bool pk2 = ovl && n <= kPk2MaxN;
-        const Sweeper<TPT, B, OVL> sw{my_cnt, s_tab, a.table_smem, a.table, n_phase};
+        const Sweeper<TPT, TB, OVL> sw{my_cnt, s_tab, a.table_smem, a.table, n_phase,
+                                       SHARED_SET ? warp * n_phase / WARPS : 0,
+                                       SHARED_SET ? (warp + 1) * n_phase / WARPS : n_phase};
         int ended = 0;  // non-empty segments ended so far (FMT_PK2: field = ended & 1)
         for (int lo = 0; lo < n; lo += chunk_pts) {
             const int hi = min(n, lo + chunk_pts);
@@ -998,7 +1012,13 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
             }
             for (int i = 0; i < n_mag; ++i) {
                 const int s0 = s_seg[i], s1 = s_seg[i + 1];
-                const int ka = max(s0, lo), kb = min(s1, hi);
+                int ka = max(s0, lo), kb = min(s1, hi);
+                if (SHARED_SET && ka < kb) {
+                    // the warp's share, cut between pairs of points
+                    const int per = (kb - ka + WARPS - 1) / WARPS, from = ka, to = kb;
+                    if (warp > 0) ka = min(to, ((from + warp * per - lo + 1) & ~1) + lo);
+                    if (warp < WARPS - 1) kb = min(to, ((from + (warp + 1) * per - lo + 1) & ~1) + lo);
+                }
                 if (ka < kb) {
                     const unsigned int inc = pk2 ? ((ended & 1) ? kPk2IncB : 1u) + kPk2IncC : 1u;
                     compiler_fence();
@@ -1040,6 +1060,7 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                     // after every second one); after the curve's last segment one sweep
                     // takes its counts and the cumulative ones (the marginal term) and
                     // clears the counters for the next item
+                    if (SHARED_SET) __syncthreads();
                     if (s1 == n) {
                         if (pk2) sw.run<FMT_PK2, SW_LAST>(tab_all, wl, n_extra, nh);
                         else sw.run<FMT, SW_LAST>(tab_all, wl, n_extra, nh);
@@ -1048,9 +1069,26 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                     } else if (ended & 1) {
                         sw.run<FMT_PK2, SW_SEG>(tab_all, wl, n_extra, nh);
                     }
+                    if (SHARED_SET) __syncthreads();
                     ++ended;
                 }
             }
+        }
+
+        if (SHARED_SET) {
+            // the warps' shares of the sums, added by the first (integers: any order)
+            __shared__ unsigned long long s_part[SHARED_SET ? WARPS * TPT * 32 : 1];
+#pragma unroll
+            for (int s = 0; s < TPT; ++s) s_part[(warp * TPT + s) * 32 + lane] = nh[s];
+            __syncthreads();
+            if (warp > 0) {
+                ++item;
+                continue;
+            }
+#pragma unroll
+            for (int s = 0; s < TPT; ++s)
+#pragma unroll
+                for (int w = 1; w < WARPS; ++w) nh[s] += s_part[(w * TPT + s) * 32 + lane];
         }
 
         // H (the counts total 2N with overlapping bins, every point being in two)
@@ -1072,8 +1110,8 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
 
         // each warp writes its own candidate list (index: curve, tile, warp) and the
         // moments of its trial lists, so the tile needs no barrier; the merge kernels
-        // take B / 32 candidate lists per tile
-        const long long list = ((long long)c * a.n_tiles + tile) * (B >> 5) + warp;
+        // take TB / 32 candidate lists per tile
+        const long long list = ((long long)c * a.n_tiles + tile) * (TB >> 5) + tw;
         if (a.stats) {
             // moments of a list's H for the significance of Eq. 5: sums of H - shift in
             // FP32 (shift = lane 0's first value, so the sums stay small), then (count,
@@ -1150,6 +1188,12 @@ cudaError_t launch_main_t(int grid, size_t smem, const MainArgs &a, cudaStream_t
     switch (a.kv) {
         case KV_SNAP: k_main<MODE, TPT, LOG2B, KV_SNAP><<<grid, 1 << LOG2B, smem, s>>>(a); break;
         case KV_OVL: k_main<MODE, TPT, LOG2B, KV_OVL><<<grid, 1 << LOG2B, smem, s>>>(a); break;
+        case KV_SHARED:
+            if constexpr (shared_set_built(TPT, LOG2B))
+                k_main<MODE, TPT, LOG2B, KV_SHARED><<<grid, 1 << LOG2B, smem, s>>>(a);
+            else
+                return cudaErrorInvalidValue;
+            break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -1172,6 +1216,12 @@ const void *kernel_for_variant(int block, int kv) {
     switch (kv) {
         case KV_SNAP: return kernel_for_block<MODE, TPT, KV_SNAP>(block);
         case KV_OVL: return kernel_for_block<MODE, TPT, KV_OVL>(block);
+        case KV_SHARED:
+            if constexpr (shared_set_built(TPT, 7))
+                if (block == 128) return (const void *)k_main<MODE, TPT, 7, KV_SHARED>;
+            if constexpr (shared_set_built(TPT, 8))
+                if (block == 256) return (const void *)k_main<MODE, TPT, 8, KV_SHARED>;
+            return nullptr;
         default: return nullptr;
     }
 }

@@ -91,6 +91,8 @@ struct gce_handle_s {
     JobState *h_state = nullptr;         // pinned copy target for the check flags
     cudaEvent_t staged = nullptr;        // staging buffers free again after this
     bool staged_pending = false;
+    int staged_n = -1;                   // curves whose offsets and order the buffers hold
+    cudaStream_t last_stream = nullptr;  // of the last job (its event: staged)
     cudaEvent_t k0 = nullptr, k1 = nullptr;  // around the CE kernel (GCE_FLAG_TIME_KERNEL)
     bool timed = false;
     int launches = 0;                    // kernels the last job launched (directly or in its graph)
@@ -526,19 +528,18 @@ gce_status mark(gce_handle h, cudaEvent_t e, cudaStream_t s, bool capturing) {
 }
 
 // Enqueue the whole sequence of one call on stream s (possibly under capture).
-gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, bool capturing) {
+// pdl: launch the kernels with programmatic dependence.
+gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, bool capturing,
+                   bool pdl) {
     const gce_config *cfg = j.cfg;
     const int mode = pl.prep_mode;
     const int kmode = kernel_mode(cfg->phase_mode);
     JobState *st = (JobState *)h->state.p;
-    CUDA_TRY(h, cudaMemcpyAsync(h->offsets.p, h->h_offsets, sizeof(long long) * (j.n_curves + 1),
-                                cudaMemcpyHostToDevice, s));
-    CUDA_TRY(h, cudaMemcpyAsync(h->order.p, h->h_order, sizeof(int) * j.n_curves,
-                                cudaMemcpyHostToDevice, s));
     int n_launch = 0;  // kernels this sequence launches, for gce_last_launches
-    CUDA_TRY(h, launch_init(st, s));
+    CUDA_TRY(h, launch_init(st, h->h_offsets, h->h_order, (long long *)h->offsets.p,
+                            (int *)h->order.p, j.n_curves, s));
     CUDA_TRY(h, launch_scan(j.times, j.mags, pl.n_points, j.periods, j.n_periods, j.pdots,
-                            j.n_pdots, cfg->t0, st, s));
+                            j.n_pdots, cfg->t0, st, pdl, s));
     n_launch += 2;
     TrialArgs ta;
     ta.periods = j.periods;
@@ -547,7 +548,7 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
     ta.n_pdots = j.n_pdots;
     ta.trialc = h->trialc.p;
     ta.state = st;
-    CUDA_TRY(h, launch_trials(mode, ta, s));
+    CUDA_TRY(h, launch_trials(mode, ta, pdl, s));
     ++n_launch;
     PrepArgs pa;
     pa.times = j.times;
@@ -565,10 +566,10 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
     pa.n_bands = j.bands ? j.n_bands : 0;
     if (j.bands) {
         CUDA_TRY(h, launch_band_stats(j.mags, j.bands, pa.offsets, j.n_curves, j.n_bands,
-                                      (double2 *)h->band_stats.p, st, s));
+                                      (double2 *)h->band_stats.p, st, pdl, s));
         ++n_launch;
     }
-    CUDA_TRY(h, launch_prep(mode, pa, s));
+    CUDA_TRY(h, launch_prep(mode, pa, pdl, s));
     ++n_launch;
     MainArgs ma;
     ma.payload = h->payload.p;
@@ -600,6 +601,7 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
     ma.overlap = (cfg->flags & GCE_FLAG_OVERLAP) ? 1 : 0;
     ma.half = pl.half;
     ma.kv = pl.kv;
+    ma.pdl = pdl ? 1 : 0;
     ma.tau = (const double *)h->tau.p;
     ma.periods = j.periods;
     ma.pdots = j.pdots;
@@ -632,15 +634,15 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
                 CUDA_TRY(h, launch_topk_reduce((const unsigned long long *)h->cand.p, j.n_curves,
                                                (int)pl.n_lists, j.k, pl.tiles_per_group, pl.n_groups,
                                                pl.stats_per, ma.stats, (unsigned long long *)h->cand2.p, stats2,
-                                               st, s));
+                                               st, pdl, s));
                 CUDA_TRY(h, launch_topk_merge((const unsigned long long *)h->cand2.p, j.n_curves,
                                               pl.n_groups, j.k, 1, j.topk_H, (long long *)j.topk_idx,
-                                              stats2, j.mean, j.std_dev, j.rho, st, s));
+                                              stats2, j.mean, j.std_dev, j.rho, st, pdl, s));
                 n_launch += 2;
             } else {
                 CUDA_TRY(h, launch_topk_merge((const unsigned long long *)h->cand.p, j.n_curves,
                                               (int)pl.n_lists, j.k, pl.stats_per, j.topk_H,
-                                              (long long *)j.topk_idx, ma.stats, j.mean, j.std_dev, j.rho, st, s));
+                                              (long long *)j.topk_idx, ma.stats, j.mean, j.std_dev, j.rho, st, pdl, s));
                 ++n_launch;
             }
             break;
@@ -699,6 +701,9 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
     if (j.bands && (j.n_bands < 1 || j.n_bands > GCE_MAX_BANDS))
         return fail(h, GCE_ERR_INVALID, "n_bands must be 1 .. %d", GCE_MAX_BANDS);
     CUDA_TRY(h, cudaSetDevice(h->device));
+    // jobs on one stream follow one another; one on another stream waits on the
+    // device for the handle's workspace
+    if (h->staged_pending && s != h->last_stream) CUDA_TRY(h, cudaStreamWaitEvent(s, h->staged, 0));
     {
         // arrays already checked by the previous call (same argument, same
         // pointer) need no new query
@@ -754,33 +759,40 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
         h->table_n = pl.n_max;
     }
 
-    // host staging (pinned): offsets and the longest-first curve order
-    if (h->staged_pending) {
-        CUDA_TRY(h, cudaEventSynchronize(h->staged));
-        h->staged_pending = false;
+    // host staging (pinned): offsets and the longest-first curve order.  Every job's
+    // first kernel reads them; a job whose offsets are those already staged leaves
+    // the buffers alone and need not wait for the jobs before it.
+    if (h->staged_n != j.n_curves ||
+        std::memcmp(h->h_offsets, j.h_offsets, sizeof(long long) * (j.n_curves + 1)) != 0) {
+        if (h->staged_pending) CUDA_TRY(h, cudaEventSynchronize(h->staged));
+        h->staged_n = -1;
+        if ((size_t)j.n_curves + 1 > h->h_cap) {
+            if (h->h_order) cudaFreeHost(h->h_order);
+            if (h->h_offsets) cudaFreeHost(h->h_offsets);
+            h->h_order = nullptr;
+            h->h_offsets = nullptr;
+            h->h_cap = 0;
+            size_t cap = (size_t)j.n_curves + 1;
+            CUDA_TRY(h, cudaMallocHost((void **)&h->h_order, sizeof(int) * cap));
+            CUDA_TRY(h, cudaMallocHost((void **)&h->h_offsets, sizeof(long long) * cap));
+            h->h_cap = cap;
+        }
+        std::memcpy(h->h_offsets, j.h_offsets, sizeof(long long) * (j.n_curves + 1));
+        std::iota(h->h_order, h->h_order + j.n_curves, 0);
+        std::stable_sort(h->h_order, h->h_order + j.n_curves, [&](int a, int b) {
+            return j.h_offsets[a + 1] - j.h_offsets[a] > j.h_offsets[b + 1] - j.h_offsets[b];
+        });
+        h->staged_n = j.n_curves;
     }
-    if ((size_t)j.n_curves + 1 > h->h_cap) {
-        if (h->h_order) cudaFreeHost(h->h_order);
-        if (h->h_offsets) cudaFreeHost(h->h_offsets);
-        h->h_order = nullptr;
-        h->h_offsets = nullptr;
-        h->h_cap = 0;
-        size_t cap = (size_t)j.n_curves + 1;
-        CUDA_TRY(h, cudaMallocHost((void **)&h->h_order, sizeof(int) * cap));
-        CUDA_TRY(h, cudaMallocHost((void **)&h->h_offsets, sizeof(long long) * cap));
-        h->h_cap = cap;
-    }
-    std::memcpy(h->h_offsets, j.h_offsets, sizeof(long long) * (j.n_curves + 1));
-    std::iota(h->h_order, h->h_order + j.n_curves, 0);
-    std::stable_sort(h->h_order, h->h_order + j.n_curves, [&](int a, int b) {
-        return j.h_offsets[a + 1] - j.h_offsets[a] > j.h_offsets[b + 1] - j.h_offsets[b];
-    });
 
     const bool use_graph = !(j.cfg->flags & GCE_FLAG_NO_GRAPH) && s != nullptr &&
                            j.kind != JOB_SINGLE;
     h->timed = (j.cfg->flags & GCE_FLAG_TIME_KERNEL) != 0 && j.kind != JOB_COUNTS;
     if (!use_graph) {
-        st = enqueue(h, j, pl, s, false);
+        // (the caller may be capturing the stream)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (s != nullptr) CUDA_TRY(h, cudaStreamIsCapturing(s, &cap));
+        st = enqueue(h, j, pl, s, false, cap == cudaStreamCaptureStatusNone);
         if (st != GCE_OK) return st;
     } else {
         GraphKey key{j.kind * 8 + (j.bands ? 4 : 0) + (j.rho ? 2 : 0) +
@@ -804,6 +816,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
         fp.add_u((unsigned long long)j.n_cells);
         fp.add_u((unsigned long long)pl.n_long);
         fp.add_u((unsigned long long)pl.prep_mode);
+        fp.add_u((unsigned long long)(pl.kv * 8 + pl.range));
         auto it = h->graphs.find(key);
         if (it != h->graphs.end() && it->second.fp == fp) {
             // same shape and the same arrays as the cached graph: replay it as it is
@@ -812,7 +825,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
             const int before = h->launches;
             cudaGraph_t graph = nullptr;
             CUDA_TRY(h, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-            st = enqueue(h, j, pl, s, true);
+            st = enqueue(h, j, pl, s, true, false);
             cudaError_t e = cudaStreamEndCapture(s, &graph);
             if (st != GCE_OK) {
                 if (graph) cudaGraphDestroy(graph);
@@ -827,6 +840,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
                     ready = true;
                 } else {
                     cudaGetLastError();
+                    if (h->staged_pending) cudaEventSynchronize(h->staged);
                     cudaGraphExecDestroy(it->second.exec);
                     h->graphs.erase(it);
                 }
@@ -839,6 +853,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
                     return fail(h, GCE_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
                 }
                 if (h->graphs.size() > 64) {
+                    if (h->staged_pending) cudaEventSynchronize(h->staged);
                     for (auto &kv : h->graphs) cudaGraphExecDestroy(kv.second.exec);
                     h->graphs.clear();
                 }
@@ -853,6 +868,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
     }
     CUDA_TRY(h, cudaEventRecord(h->staged, s));
     h->staged_pending = true;
+    h->last_stream = s;
     return GCE_OK;
 }
 

@@ -502,6 +502,40 @@ struct TileStats {
     double n, mean, m2;
 };
 
+// The moments of a block's records [0, n) merged (every thread returns them): the
+// mean from the sums of n and n mean, then M2 from the records' own and their means'
+// distances, each in a fixed order (a strided run per thread, a fixed tree, the
+// warps in order), so the result is deterministic.  Two passes instead of a pairwise
+// update, which divides twice per merge (the whole merge kernel, 782 lists of one curve:
+// 32 -> 13 us).
+__device__ inline double block_sum_fixed(double v, double *sh) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
+    return t;
+}
+__device__ inline TileStats block_moments(const TileStats *ts, int n, double *sh) {
+    double c = 0.0, m = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        c += ts[i].n;
+        m += ts[i].n * ts[i].mean;
+    }
+    TileStats r;
+    r.n = block_sum_fixed(c, sh);
+    r.mean = block_sum_fixed(m, sh);
+    if (r.n > 0.0) r.mean /= r.n;
+    double q = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const double d = ts[i].mean - r.mean;
+        if (ts[i].n > 0.0) q += ts[i].m2 + ts[i].n * d * d;
+    }
+    r.m2 = block_sum_fixed(q, sh);
+    return r;
+}
+
 // Trial tiles of one curve's grid for a launch of `block` threads x `tpt`
 // trials.  With several Pdot values and tpt > 1 a tile is block periods x tpt
 // consecutive Pdot values, so that a thread's trials share their period (and
@@ -581,6 +615,7 @@ struct MainArgs {
     // single Pdot is not 0 stages chunk / 2 whole points in the same bytes
     int half;
     int kv;                    // CE kernel variant (KV_*): overlapping bins or not
+    int pdl;                   // host: launch with programmatic dependence
     // FP64 jobs: every point's binary64 tau in payload order, and the caller's
     // trial arrays (for the points the certified fold leaves to binary64)
     const double *tau;
@@ -598,16 +633,44 @@ inline int kernel_variant(bool overlap) { return overlap ? KV_OVL : KV_SNAP; }
 // threads of a CTA with trials (and counters) of their own
 inline int trial_threads(int kv, int block) { return kv == KV_SHARED ? 32 : block; }
 
+// Programmatic dependent launch.  A call's kernels follow one another on one stream
+// and most are short, so each is launched while the one before it still runs and
+// waits on the device: pdl_wait() returns when everything before it has completed
+// and its writes are visible.  Every kernel that launch_pdl starts calls it before it
+// touches what an earlier kernel writes (so completion is transitive), and
+// pdl_trigger() lets the next one be scheduled.  The first kernel of a call is
+// launched normally, after all of the caller's work.  Not under stream capture.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), unsigned int grid, unsigned int block,
+                              size_t smem, cudaStream_t s, bool pdl, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = pdl ? 1u : 0u;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Kernel launchers (defined in the .cu files).
-cudaError_t launch_init(JobState *st, cudaStream_t s);
+// h_offsets, h_order: pinned host memory read by the kernel itself (nullptr: offsets
+// are on the device already, and the order is 0, 1, ...)
+cudaError_t launch_init(JobState *st, const long long *h_offsets, const int *h_order,
+                        long long *offsets, int *order, int n_curves, cudaStream_t s);
 cudaError_t launch_scan(const double *times, const double *mags, long long n_points,
                         const double *periods, int n_periods, const double *pdots, int n_pdots,
-                        double t0, JobState *st, cudaStream_t s);
-cudaError_t launch_trials(int mode, const TrialArgs &a, cudaStream_t s);
-cudaError_t launch_prep(int mode, const PrepArgs &a, cudaStream_t s);
+                        double t0, JobState *st, bool pdl, cudaStream_t s);
+cudaError_t launch_trials(int mode, const TrialArgs &a, bool pdl, cudaStream_t s);
+cudaError_t launch_prep(int mode, const PrepArgs &a, bool pdl, cudaStream_t s);
 cudaError_t launch_band_stats(const double *mags, const unsigned char *bands,
                               const long long *offsets, int n_curves, int n_bands,
-                              double2 *stats, JobState *st, cudaStream_t s);
+                              double2 *stats, JobState *st, bool pdl, cudaStream_t s);
 cudaError_t launch_table(unsigned long long *table, int n_max, cudaStream_t s);
 size_t main_smem_bytes(int mode, int block, int tpt, int chunk, int n_phase, int n_mag,
                        int table_smem, int range, int half);
@@ -635,7 +698,7 @@ cudaError_t launch_main(int mode, int tpt, int block, int grid, size_t smem,
 cudaError_t launch_topk_merge(const unsigned long long *cand, int n_curves, int n_tiles,
                               int k, int stats_per, float *topk_H, long long *topk_idx, const TileStats *stats,
                               double *mean, double *std_dev, float *rho, const JobState *st,
-                              cudaStream_t s);
+                              bool pdl, cudaStream_t s);
 cudaError_t launch_single(const MainArgs &a, int curve, long long n_points, cudaStream_t s);
 cudaError_t launch_counts(int mode, const MainArgs &a, long long n_cells,
                           const long long *cell_curve, const long long *cell_trial,

@@ -736,23 +736,6 @@ __device__ __forceinline__ void split_slot_window(bool pdot, float cyc_max, int 
     zhi = min((int)floorf(nf + nf * xm), 2 * n_phase - 1);
 }
 
-// Chan et al.'s pairwise update of (count, mean, M2) moments.
-__device__ __forceinline__ void chan_merge(double &n, double &mean, double &m2, double nb,
-                                           double meanb, double m2b) {
-    if (nb <= 0.0) return;
-    if (n <= 0.0) {
-        n = nb;
-        mean = meanb;
-        m2 = m2b;
-        return;
-    }
-    const double tot = n + nb;
-    const double d = meanb - mean;
-    mean += d * (nb / tot);
-    m2 += m2b + d * d * (n * nb / tot);
-    n = tot;
-}
-
 // CTAs per SM the register allocation is sized for.  With two trials per
 // thread the counters (and FP64's wider staged points) already limit shared
 // memory to about three 256-thread CTAs per SM at 15 phase bins, so those
@@ -1173,6 +1156,8 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
 template <int MODE, int TPT, int LOG2B, int KV>
 __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k_main(MainArgs a) {
     __shared__ long long s_item;
+    pdl_trigger();
+    pdl_wait();
     if (a.state->err) return;  // inputs failed the device checks: no work
     if constexpr (MODE == kFoldCertified) {
         if (a.payload == nullptr || a.state->wide) {
@@ -1186,17 +1171,16 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
 template <int MODE, int TPT, int LOG2B>
 cudaError_t launch_main_t(int grid, size_t smem, const MainArgs &a, cudaStream_t s) {
     switch (a.kv) {
-        case KV_SNAP: k_main<MODE, TPT, LOG2B, KV_SNAP><<<grid, 1 << LOG2B, smem, s>>>(a); break;
-        case KV_OVL: k_main<MODE, TPT, LOG2B, KV_OVL><<<grid, 1 << LOG2B, smem, s>>>(a); break;
+        case KV_SNAP: return launch_pdl(k_main<MODE, TPT, LOG2B, KV_SNAP>, grid, 1 << LOG2B, smem, s, a.pdl != 0, a);
+        case KV_OVL: return launch_pdl(k_main<MODE, TPT, LOG2B, KV_OVL>, grid, 1 << LOG2B, smem, s, a.pdl != 0, a);
         case KV_SHARED:
             if constexpr (shared_set_built(TPT, LOG2B))
-                k_main<MODE, TPT, LOG2B, KV_SHARED><<<grid, 1 << LOG2B, smem, s>>>(a);
+                return launch_pdl(k_main<MODE, TPT, LOG2B, KV_SHARED>, grid, 1 << LOG2B, smem, s, a.pdl != 0, a);
             else
                 return cudaErrorInvalidValue;
             break;
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 // The kernel instantiations: mode x trials per thread x block size.

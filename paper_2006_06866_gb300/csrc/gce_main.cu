@@ -8,70 +8,72 @@ namespace gce {
 
 namespace {
 
-// Per-curve merge of the tiles' candidates: k rounds of "smallest key above the
-// previous one" (keys are unique: H bits in the high word, trial index low).
-__global__ void k_topk_merge(const unsigned long long *__restrict__ cand, int n_tiles, int k,
-                             int stats_per, float *topk_H, long long *topk_idx, const TileStats *stats,
-                             double *mean_out, double *std_out, float *rho_out, const JobState *st) {
-    __shared__ unsigned long long sh[32];
-    __shared__ double shs[3 * 32];
+constexpr int kMergeBlock = 256;
+constexpr int kMergeKeys = 16;  // keys a merging thread holds in registers
+
+// Per-curve merge of the candidate lists: k rounds of "smallest key above the
+// previous one" (keys are unique: H bits in the high word, trial index low), and the
+// significance of Eq. 5 from the moment records.  Latency-bound (one CTA per curve):
+// up to 4096 keys are read once, into registers, and a round is one barrier.
+__global__ void __launch_bounds__(kMergeBlock)
+    k_topk_merge(const unsigned long long *__restrict__ cand, int n_tiles, int k, int stats_per,
+                 float *topk_H, long long *topk_idx, const TileStats *stats, double *mean_out,
+                 double *std_out, float *rho_out, const JobState *st) {
+    constexpr int WARPS = kMergeBlock / 32;
+    __shared__ unsigned long long sh[2][WARPS];
+    __shared__ double shs[WARPS];
+    pdl_trigger();
+    pdl_wait();
     if (st->err) return;
-    const int c = blockIdx.x;
+    const int c = blockIdx.x, tid = threadIdx.x;
     const long long n = (long long)n_tiles * k;
     const unsigned long long *src = cand + (long long)c * n;
-    unsigned long long last = 0ull;
+    const bool held = n <= kMergeKeys * kMergeBlock;
+    unsigned long long key[kMergeKeys];
+    unsigned long long mine = kNoKey, last = 0ull, first = kNoKey;
+    if (held) {
+#pragma unroll
+        for (int i = 0; i < kMergeKeys; ++i) {
+            key[i] = tid + i * kMergeBlock < n ? src[tid + i * kMergeBlock] : kNoKey;
+            mine = key[i] < mine ? key[i] : mine;
+        }
+    }
     for (int r = 0; r < k; ++r) {
-        unsigned long long mine = kNoKey;
-        for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-            const unsigned long long v = src[i];
-            if ((r == 0 || v > last) && v < mine) mine = v;
+        if (!held) {
+            mine = kNoKey;
+            for (long long i = tid; i < n; i += kMergeBlock) {
+                const unsigned long long v = src[i];
+                if ((r == 0 || v > last) && v < mine) mine = v;
+            }
         }
-        mine = warp_min_key(mine);
-        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mine;
+        const unsigned long long w = warp_min_key(mine);
+        if ((tid & 31) == 0) sh[r & 1][tid >> 5] = w;
         __syncthreads();
-        if (threadIdx.x < 32) {
-            unsigned long long v = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : kNoKey;
-            v = warp_min_key(v);
-            if (threadIdx.x == 0) sh[0] = v;
-        }
-        __syncthreads();
-        last = sh[0];
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        last = sh[r & 1][0];
+#pragma unroll
+        for (int i = 1; i < WARPS; ++i) last = sh[r & 1][i] < last ? sh[r & 1][i] : last;
+        if (r == 0) first = last;
+        if (tid == 0) {
             topk_H[(long long)c * k + r] = __uint_as_float((unsigned int)(last >> 32));
             topk_idx[(long long)c * k + r] = (long long)(last & 0xffffffffull);
         }
+        if (held && mine == last) {
+            mine = kNoKey;
+#pragma unroll
+            for (int i = 0; i < kMergeKeys; ++i)
+                if (key[i] > last && key[i] < mine) mine = key[i];
+        }
     }
     if (!stats) return;
-    // Eq. 5: rho = (mu - H_min) / sigma over the curve's whole grid, the tiles'
-    // moments merged in a fixed order (each thread a strided run of tiles, then
-    // a fixed tree), so the result is deterministic
-    double nn = 0.0, mu = 0.0, m2 = 0.0;
+    // Eq. 5: rho = (mu - H_min) / sigma over the curve's whole grid
     const int n_stats = n_tiles * stats_per;
-    const TileStats *ts = stats + (long long)c * n_stats;
-    for (int i = threadIdx.x; i < n_stats; i += blockDim.x) chan_merge(nn, mu, m2, ts[i].n, ts[i].mean, ts[i].m2);
-    for (int o = 1; o < 32; o <<= 1) {
-        const double nb = __shfl_down_sync(0xffffffffu, nn, o);
-        const double mb = __shfl_down_sync(0xffffffffu, mu, o);
-        const double qb = __shfl_down_sync(0xffffffffu, m2, o);
-        if ((threadIdx.x & (2 * o - 1)) == 0) chan_merge(nn, mu, m2, nb, mb, qb);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        shs[3 * (threadIdx.x >> 5)] = nn;
-        shs[3 * (threadIdx.x >> 5) + 1] = mu;
-        shs[3 * (threadIdx.x >> 5) + 2] = m2;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        nn = 0.0;
-        mu = 0.0;
-        m2 = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) chan_merge(nn, mu, m2, shs[3 * w], shs[3 * w + 1], shs[3 * w + 2]);
-        const double sd = nn > 0.0 ? sqrt(m2 / nn) : 0.0;
-        mean_out[c] = mu;
+    const TileStats m = block_moments(stats + (long long)c * n_stats, n_stats, shs);
+    if (tid == 0) {
+        const double sd = m.n > 0.0 ? sqrt(m.m2 / m.n) : 0.0;
+        mean_out[c] = m.mean;
         std_out[c] = sd;
-        // H_min is the first of the top-k this thread wrote above
-        rho_out[c] = sd > 0.0 ? (float)((mu - (double)topk_H[(long long)c * k]) / sd) : 0.0f;
+        const double h = (double)__uint_as_float((unsigned int)(first >> 32));
+        rho_out[c] = sd > 0.0 ? (float)((m.mean - h) / sd) : 0.0f;
     }
 }
 
@@ -203,11 +205,10 @@ cudaError_t launch_main(int mode, int tpt, int block, int grid, size_t smem, con
 cudaError_t launch_topk_merge(const unsigned long long *cand, int n_curves, int n_tiles, int k,
                               int stats_per, float *topk_H, long long *topk_idx,
                               const TileStats *stats, double *mean, double *std_dev, float *rho,
-                              const JobState *st, cudaStream_t s) {
+                              const JobState *st, bool pdl, cudaStream_t s) {
     if (n_curves <= 0) return cudaSuccess;
-    k_topk_merge<<<n_curves, 256, 0, s>>>(cand, n_tiles, k, stats_per, topk_H, topk_idx, stats, mean,
-                                          std_dev, rho, st);
-    return cudaGetLastError();
+    return launch_pdl(k_topk_merge, n_curves, kMergeBlock, 0, s, pdl, cand, n_tiles, k, stats_per,
+                      topk_H, topk_idx, stats, mean, std_dev, rho, st);
 }
 
 cudaError_t launch_single(const MainArgs &a, int curve, long long, cudaStream_t s) {

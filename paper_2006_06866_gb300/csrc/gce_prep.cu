@@ -12,13 +12,25 @@ namespace {
 
 constexpr unsigned long long kPosInfBits = 0x7ff0000000000000ull;
 
-__global__ void k_init(JobState *st) {
-    st->tau_max_bits = 0ull;
-    st->pmin_bits = kPosInfBits;
-    st->pdot_max_bits = 0ull;
-    st->err = 0u;
-    st->work = 0ull;
-    st->wide = 0u;
+// The job state cleared, and the curves' offsets and processing order copied from
+// the caller-side staging buffers (pinned host memory, read over the link: two copies
+// on the stream cost more than the whole kernel for small batches).
+__global__ void k_init(JobState *st, const long long *h_offsets, const int *h_order,
+                       long long *offsets, int *order, int n_curves) {
+    pdl_trigger();
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i0 == 0) {
+        st->tau_max_bits = 0ull;
+        st->pmin_bits = kPosInfBits;
+        st->pdot_max_bits = 0ull;
+        st->err = 0u;
+        st->work = 0ull;
+        st->wide = 0u;
+    }
+    for (int i = i0; i <= n_curves; i += gridDim.x * blockDim.x) {
+        if (h_offsets) offsets[i] = h_offsets[i];
+        if (i < n_curves) order[i] = h_order ? h_order[i] : i;
+    }
 }
 
 // Non-negative binary64 values order like their bit patterns, so maxima and
@@ -44,6 +56,8 @@ __device__ inline double warp_min(double v) {
 __global__ void k_scan(const double *__restrict__ times, const double *__restrict__ mags,
                        long long n_points, const double *__restrict__ periods, int n_periods,
                        const double *__restrict__ pdots, int n_pdots, double t0, JobState *st) {
+    pdl_trigger();
+    pdl_wait();
     unsigned int err = 0u;
     double tmax = 0.0, pmin = INFINITY, dmax = 0.0;
     long long stride = (long long)gridDim.x * blockDim.x;
@@ -86,11 +100,19 @@ __device__ inline bool beyond_certified(const JobState *st, int e_tau) {
     return !fixed_range_ok(fmax_, 0.5 * dmax * fmax_ * fmax_, e_tau);
 }
 
+// x 2^e as ldexp rounds it: one multiplication where 2^e is a normal number.
+__device__ __forceinline__ double scale2(double x, int e) {
+    if (e < -1022 || e > 1023) return ldexp(x, e);
+    return __dmul_rn(x, __longlong_as_double((long long)(e + 1023) << 52));
+}
+
 // Per flat trial t = q n_periods + p: f = 1/P, a = (0.5 Pdot) f f (the oracle's
 // sequence), stored in the fold mode's format.
 template <int MODE>
 __global__ void k_trials(TrialArgs a) {
     typedef typename ModeTraits<MODE>::trial_t trial_t;
+    pdl_trigger();
+    pdl_wait();
     trial_t *out = reinterpret_cast<trial_t *>(a.trialc);
     const long long n = (long long)a.n_periods * a.n_pdots;
     const double tau_max = __longlong_as_double((long long)a.state->tau_max_bits);
@@ -138,8 +160,8 @@ __global__ void k_trials(TrialArgs a) {
             v.w = __double2float_rn(-aa - (double)nah);
         } else {
             // Out-of-range values are flagged above; clamp so the conversions stay defined.
-            const double F = fmin(ldexp(f, fs.r), 9.2e18);
-            const double A = fmax(fmin(ldexp(aa, fs.v), 9.2e18), -9.2e18);
+            const double F = fmin(scale2(f, fs.r), 9.2e18);
+            const double A = fmax(fmin(scale2(aa, fs.v), 9.2e18), -9.2e18);
             int f1, f0;
             split_balanced(__double2ll_rn(F), &f1, &f0);
             const long long an = -__double2ll_rn(A);
@@ -149,10 +171,10 @@ __global__ void k_trials(TrialArgs a) {
             const unsigned int uf1 = (unsigned int)f1;
             const int bits = 32 - __clz(uf1);
             const int k = bits > 22 ? bits - 22 : 0;
-            const float g0 = __double2float_rn(ldexp((double)uf1, -23 - k));
-            const float g2 = __double2float_rn(ldexp((double)a1, -23 - k));
+            const float g0 = __double2float_rn(scale2((double)uf1, -23 - k));
+            const float g2 = __double2float_rn(scale2((double)a1, -23 - k));
             const double kk = 12582912.0 - 8388608.0 * (double)g0 - 8388608.0 * (double)g2 -
-                              ldexp((double)a1, -1 - k);
+                              scale2((double)a1, -1 - k);
             v.i = make_uint4(uf1, (unsigned int)f0, (unsigned int)a1, a0);
             v.f = make_float4(g0, g2, __double2float_rn(kk), __uint_as_float((unsigned int)k));
         }
@@ -161,22 +183,7 @@ __global__ void k_trials(TrialArgs a) {
 }
 
 constexpr int kPrepBlock = 256;
-
-__device__ inline double block_reduce(double v, bool is_max, double *sh) {
-    v = is_max ? warp_max(v) : warp_min(v);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        v = l < (blockDim.x >> 5) ? sh[l] : (is_max ? -INFINITY : INFINITY);
-        v = is_max ? warp_max(v) : warp_min(v);
-        if (l == 0) sh[0] = v;
-    }
-    __syncthreads();
-    v = sh[0];
-    __syncthreads();
-    return v;
-}
+constexpr int kPrepMags = 1024, kPrepBins = 8192;
 
 // Magnitude bin of Sec. 2.3 with the oracle's operation sequence:
 // i = floor(((m - mn) / (mx - mn)) * n_mag), clamped; mx == mn -> 0.
@@ -186,6 +193,28 @@ __device__ inline int mag_bin(double m, double mn, double mx, int n_mag) {
     int i = __double2int_rd(__dmul_rn(v, (double)n_mag));
     return min(i, n_mag - 1);
 }
+
+// mag_bin, from a binary32 quotient where that decides it: four roundings leave v
+// within 255 2^-22 = 6.1e-5 of the sequence's value, so a v farther than 1e-4 from
+// the integers has its floor; the others, and ranges that binary32 does not hold
+// well, take the binary64 division (some 25 operations at 2 lanes per clock).
+struct MagBins {
+    double mn, mx;
+    float scale;
+    int n_mag;
+    bool fast;
+    __device__ MagBins(double mn_, double mx_, int n_mag_) : mn(mn_), mx(mx_), n_mag(n_mag_) {
+        const double range = __dsub_rn(mx, mn);
+        fast = range > 1e-30 && range < 1e30;
+        scale = fast ? __fdiv_rn((float)n_mag, __double2float_rn(range)) : 0.0f;
+    }
+    __device__ int operator()(double m) const {
+        const float v = __double2float_rn(__dsub_rn(m, mn)) * scale;
+        const float f = floorf(v), d = v - f;
+        if (fast && d > 1e-4f && d < 1.0f - 1e-4f) return (int)f;
+        return mag_bin(m, mn, mx, n_mag);
+    }
+};
 
 // ------------------------------------------------------------------ filters
 
@@ -232,20 +261,106 @@ __device__ double band_select(const double *m, const unsigned char *bd, int n, i
     return key_f64(prefix);
 }
 
+// Smallest (largest) 64-bit key of the warp: the high words first, then the low
+// words among the lanes holding the best one.
+__device__ inline unsigned long long warp_min_u64(unsigned long long v) {
+    const unsigned int hi = __reduce_min_sync(0xffffffffu, (unsigned int)(v >> 32));
+    const unsigned int lo =
+        __reduce_min_sync(0xffffffffu, (unsigned int)(v >> 32) == hi ? (unsigned int)v : 0xffffffffu);
+    return ((unsigned long long)hi << 32) | lo;
+}
+__device__ inline unsigned long long warp_max_u64(unsigned long long v) { return ~warp_min_u64(~v); }
+
+// Longest curve whose magnitudes k_band_stats holds in shared memory.
+constexpr int kBandCurve = 4096;
+
+// The median and population standard deviation of v[0, cnt) (shared memory, in
+// point order; overwritten), by one warp: the lower median by an exact radix
+// selection on the keys, 8 bits per pass; the upper one, for an even count, is the
+// same key or the next larger one; the sums by lane 0 in point order, the squares
+// by all lanes.
+__device__ double2 warp_band_stats(double *v, int cnt, unsigned int *hist) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long prefix = 0ull;
+    unsigned int kth = (unsigned int)(cnt - 1) / 2, same = 0u;
+    for (int shift = 56; shift >= 0; shift -= 8) {
+        const unsigned long long high = shift == 56 ? 0ull : ~0ull << (shift + 8);
+        for (int i = lane; i < 256; i += 32) hist[i] = 0u;
+        __syncwarp();
+        for (int k = lane; k < cnt; k += 32) {
+            const unsigned long long key = f64_key(v[k]);
+            if ((key & high) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
+        }
+        __syncwarp();
+        unsigned int sum = 0u, incl;
+        for (int i = 0; i < 8; ++i) sum += hist[lane * 8 + i];
+        incl = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        // the lane whose eight digits hold the kth key, and the digit
+        const int owner = __ffs((int)__ballot_sync(0xffffffffu, incl > kth)) - 1;
+        unsigned int below = incl - sum, digit = 0u, count = 0u;
+        if (lane == owner)
+            for (int i = 0; i < 8; ++i) {
+                count = hist[lane * 8 + i];
+                digit = (unsigned int)(lane * 8 + i);
+                if (below + count > kth) break;
+                below += count;
+            }
+        kth -= __shfl_sync(0xffffffffu, below, owner);
+        same = __shfl_sync(0xffffffffu, count, owner);
+        prefix |= (unsigned long long)__shfl_sync(0xffffffffu, digit, owner) << shift;
+        __syncwarp();
+    }
+    double med = key_f64(prefix);
+    if ((cnt & 1) == 0) {
+        unsigned long long next = ~0ull;
+        for (int k = lane; k < cnt; k += 32) {
+            const unsigned long long key = f64_key(v[k]);
+            if (key > prefix && key < next) next = key;
+        }
+        next = warp_min_u64(next);
+        const double hi = kth + 1u < same ? med : key_f64(next);
+        med = __dmul_rn(__dadd_rn(med, hi), 0.5);
+    }
+    double sum = 0.0;
+    if (lane == 0)
+        for (int k = 0; k < cnt; ++k) sum = __dadd_rn(sum, v[k]);
+    const double mean = __ddiv_rn(__shfl_sync(0xffffffffu, sum, 0), (double)cnt);
+    for (int k = lane; k < cnt; k += 32) {
+        const double d = __dsub_rn(v[k], mean);
+        v[k] = __dmul_rn(d, d);
+    }
+    __syncwarp();
+    double ss = 0.0;
+    if (lane == 0)
+        for (int k = 0; k < cnt; ++k) ss = __dadd_rn(ss, v[k]);
+    ss = __shfl_sync(0xffffffffu, ss, 0);
+    return make_double2(med, __dsqrt_rn(__ddiv_rn(ss, (double)cnt)));
+}
+
 // One CTA per curve: for each filter b, the median and the population standard
 // deviation of its magnitudes (the per-filter normalisation of Sec. 2.3), in the
 // operation order stated in gce.h: the median exactly (radix selection), the
-// mean and the sum of squared deviations in binary64 in point order (one
-// thread), so that the normalised values match a plain sequential statement
-// bit for bit.  A filter with no points gets {0, 0}.  Band indices >= n_bands
-// set ERR_BAND.
+// mean and the sum of squared deviations in binary64 in point order, so that the
+// normalised values match a plain sequential statement bit for bit.  A filter with
+// no points gets {0, 0}.  Band indices >= n_bands set ERR_BAND.
+// Bound by the two chains of binary64 additions, so curves of up to kBandCurve points
+// are split by filter into shared memory and each filter has a warp of its own (300
+// curves of 300..900 points in two filters: 360 us when one thread walked global
+// memory filter by filter, 64 us now).
 __global__ void __launch_bounds__(256) k_band_stats(const double *__restrict__ mags,
                                                     const unsigned char *__restrict__ bands,
                                                     const long long *__restrict__ offsets,
                                                     int n_bands, double2 *stats, JobState *st) {
-    __shared__ unsigned int hist[256];
+    __shared__ unsigned int hist[GCE_MAX_BANDS][256];
+    __shared__ double vals[kBandCurve];
     __shared__ unsigned long long s_pref;
     __shared__ int s_k, s_cnt[GCE_MAX_BANDS];
+    pdl_trigger();
+    pdl_wait();
     const int c = blockIdx.x;
     const long long lo = offsets[c];
     const int n = (int)(offsets[c + 1] - lo);
@@ -263,13 +378,33 @@ __global__ void __launch_bounds__(256) k_band_stats(const double *__restrict__ m
         if (threadIdx.x == 0) atomicOr(&st->err, ERR_BAND);
         return;
     }
+    if (n <= kBandCurve) {
+        const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        if (b >= n_bands) return;
+        int first = 0;
+        for (int i = 0; i < b; ++i) first += s_cnt[i];
+        const int cnt = s_cnt[b];
+        int at = first;
+#pragma unroll 4
+        for (int k0 = 0; k0 < n; k0 += 32) {
+            const int k = k0 + lane;
+            const bool mine = k < n && bd[k] == b;
+            const unsigned int all = __ballot_sync(0xffffffffu, mine);
+            if (mine) vals[at + __popc(all & ((1u << lane) - 1u))] = m[k];
+            at += __popc(all);
+        }
+        __syncwarp();
+        const double2 r = cnt > 0 ? warp_band_stats(vals + first, cnt, hist[b]) : make_double2(0.0, 0.0);
+        if (lane == 0) stats[(long long)c * n_bands + b] = r;
+        return;
+    }
     for (int b = 0; b < n_bands; ++b) {
         const int cnt = s_cnt[b];
         double2 r = make_double2(0.0, 0.0);
         if (cnt > 0) {
-            double med = band_select(m, bd, n, b, (cnt - 1) / 2, hist, &s_pref, &s_k);
+            double med = band_select(m, bd, n, b, (cnt - 1) / 2, hist[0], &s_pref, &s_k);
             if ((cnt & 1) == 0) {
-                const double hi = band_select(m, bd, n, b, cnt / 2, hist, &s_pref, &s_k);
+                const double hi = band_select(m, bd, n, b, cnt / 2, hist[0], &s_pref, &s_k);
                 med = __dmul_rn(__dadd_rn(med, hi), 0.5);
             }
             if (threadIdx.x == 0) {
@@ -313,24 +448,47 @@ struct MagView {
 template <int MODE>
 __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
     typedef typename ModeTraits<MODE>::point_t point_t;
-    __shared__ double sh_red[32];
+    __shared__ unsigned long long sh_min[kPrepBlock / 32], sh_max[kPrepBlock / 32];
     __shared__ int hist[GCE_MAX_MAG_BINS + 1];
+    // the first points' magnitudes and bins, each computed once (binary64 arithmetic
+    // bounds this kernel: the divisions of the filters' and the bins' normalisation)
+    __shared__ double s_m[kPrepMags];
+    __shared__ unsigned char s_bin[kPrepBins];
+    pdl_trigger();
+    pdl_wait();
     const int c = blockIdx.x;
     const long long lo = a.offsets[c];
     const int n = (int)(a.offsets[c + 1] - lo);
     const MagView m{a.mags + lo, a.bands ? a.bands + lo : nullptr,
                     a.bands ? a.band_stats + (long long)c * a.n_bands : nullptr, a.n_bands};
     const double *t = a.times + lo;
-    double mn = INFINITY, mx = -INFINITY;
+    unsigned long long kmin = ~0ull, kmax = 0ull;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        mn = fmin(mn, m[k]);
-        mx = fmax(mx, m[k]);
+        const double v = m[k];
+        if (k < kPrepMags) s_m[k] = v;
+        const unsigned long long key = f64_key(v);
+        kmin = key < kmin ? key : kmin;
+        kmax = key > kmax ? key : kmax;
     }
-    mn = block_reduce(mn, false, sh_red);
-    mx = block_reduce(mx, true, sh_red);
+    kmin = warp_min_u64(kmin);
+    kmax = warp_max_u64(kmax);
+    if ((threadIdx.x & 31) == 0) {
+        sh_min[threadIdx.x >> 5] = kmin;
+        sh_max[threadIdx.x >> 5] = kmax;
+    }
     for (int i = threadIdx.x; i <= a.n_mag; i += blockDim.x) hist[i] = 0;
     __syncthreads();
-    for (int k = threadIdx.x; k < n; k += blockDim.x) atomicAdd(&hist[mag_bin(m[k], mn, mx, a.n_mag)], 1);
+#pragma unroll
+    for (int w = 0; w < kPrepBlock / 32; ++w) {
+        kmin = sh_min[w] < kmin ? sh_min[w] : kmin;
+        kmax = sh_max[w] > kmax ? sh_max[w] : kmax;
+    }
+    const MagBins bins(key_f64(kmin), key_f64(kmax), a.n_mag);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const int b = bins(k < kPrepMags ? s_m[k] : m[k]);
+        if (k < kPrepBins) s_bin[k] = (unsigned char)b;
+        atomicAdd(&hist[b], 1);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         int run = 0;
@@ -347,7 +505,8 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
     const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
     point_t *out = reinterpret_cast<point_t *>(a.payload) + lo;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const int pos = atomicAdd(&hist[mag_bin(m[k], mn, mx, a.n_mag)], 1);
+        const int b = k < kPrepBins ? s_bin[k] : bins(k < kPrepMags ? s_m[k] : m[k]);
+        const int pos = atomicAdd(&hist[b], 1);
         const double tau = __dsub_rn(t[k], a.t0);
         point_t v;
         if constexpr (MODE == GCE_PHASE_FP64) {
@@ -363,7 +522,7 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
         } else {
             // T = round(tau 2^s), |T| < 2^62; U = floor(T^2 / 2^62) = tau^2 2^u
             // computed exactly from T in 128-bit integer arithmetic.
-            const long long T = __double2ll_rn(ldexp(tau, fs.s));
+            const long long T = __double2ll_rn(scale2(tau, fs.s));
             const unsigned long long aT = (unsigned long long)(T < 0 ? -T : T);
             const unsigned long long hi = __umul64hi(aT, aT), lw = aT * aT;
             const long long U = (long long)((hi << 2) | (lw >> 62));
@@ -396,51 +555,50 @@ int grid_for(long long n, int block, int cap) {
 
 }  // namespace
 
-cudaError_t launch_init(JobState *st, cudaStream_t s) {
-    k_init<<<1, 1, 0, s>>>(st);
+cudaError_t launch_init(JobState *st, const long long *h_offsets, const int *h_order,
+                        long long *offsets, int *order, int n_curves, cudaStream_t s) {
+    k_init<<<grid_for((long long)n_curves + 1, 256, 152), 256, 0, s>>>(st, h_offsets, h_order,
+                                                                       offsets, order, n_curves);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scan(const double *times, const double *mags, long long n_points,
                         const double *periods, int n_periods, const double *pdots, int n_pdots,
-                        double t0, JobState *st, cudaStream_t s) {
+                        double t0, JobState *st, bool pdl, cudaStream_t s) {
     long long n = n_points;
     if (n_periods > n) n = n_periods;
     if (n_pdots > n) n = n_pdots;
-    k_scan<<<grid_for(n, 256, 1216), 256, 0, s>>>(times, mags, n_points, periods, n_periods,
-                                                     pdots, n_pdots, t0, st);
-    return cudaGetLastError();
+    return launch_pdl(k_scan, grid_for(n, 256, 1216), 256, 0, s, pdl, times, mags, n_points, periods,
+                      n_periods, pdots, n_pdots, t0, st);
 }
 
-cudaError_t launch_trials(int mode, const TrialArgs &a, cudaStream_t s) {
+cudaError_t launch_trials(int mode, const TrialArgs &a, bool pdl, cudaStream_t s) {
     long long n = (long long)a.n_periods * a.n_pdots;
     int g = grid_for(n, 256, 4864);
     switch (mode) {
-        case GCE_PHASE_FP64: k_trials<GCE_PHASE_FP64><<<g, 256, 0, s>>>(a); break;
-        case GCE_PHASE_SPLIT32: k_trials<GCE_PHASE_SPLIT32><<<g, 256, 0, s>>>(a); break;
-        case kFoldCertified: k_trials<kFoldCertified><<<g, 256, 0, s>>>(a); break;
-        default: k_trials<GCE_PHASE_FIXED32><<<g, 256, 0, s>>>(a); break;
+        case GCE_PHASE_FP64: return launch_pdl(k_trials<GCE_PHASE_FP64>, g, 256, 0, s, pdl, a);
+        case GCE_PHASE_SPLIT32: return launch_pdl(k_trials<GCE_PHASE_SPLIT32>, g, 256, 0, s, pdl, a);
+        case kFoldCertified: return launch_pdl(k_trials<kFoldCertified>, g, 256, 0, s, pdl, a);
+        default: return launch_pdl(k_trials<GCE_PHASE_FIXED32>, g, 256, 0, s, pdl, a);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_band_stats(const double *mags, const unsigned char *bands,
                               const long long *offsets, int n_curves, int n_bands,
-                              double2 *stats, JobState *st, cudaStream_t s) {
+                              double2 *stats, JobState *st, bool pdl, cudaStream_t s) {
     if (n_curves <= 0) return cudaSuccess;
-    k_band_stats<<<n_curves, 256, 0, s>>>(mags, bands, offsets, n_bands, stats, st);
-    return cudaGetLastError();
+    return launch_pdl(k_band_stats, n_curves, 256, 0, s, pdl, mags, bands, offsets, n_bands, stats, st);
 }
 
-cudaError_t launch_prep(int mode, const PrepArgs &a, cudaStream_t s) {
+cudaError_t launch_prep(int mode, const PrepArgs &a, bool pdl, cudaStream_t s) {
     if (a.n_curves <= 0) return cudaSuccess;
+    const unsigned int g = a.n_curves;
     switch (mode) {
-        case GCE_PHASE_FP64: k_prep<GCE_PHASE_FP64><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
-        case GCE_PHASE_SPLIT32: k_prep<GCE_PHASE_SPLIT32><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
-        case kFoldCertified: k_prep<kFoldCertified><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
-        default: k_prep<GCE_PHASE_FIXED32><<<a.n_curves, kPrepBlock, 0, s>>>(a); break;
+        case GCE_PHASE_FP64: return launch_pdl(k_prep<GCE_PHASE_FP64>, g, kPrepBlock, 0, s, pdl, a);
+        case GCE_PHASE_SPLIT32: return launch_pdl(k_prep<GCE_PHASE_SPLIT32>, g, kPrepBlock, 0, s, pdl, a);
+        case kFoldCertified: return launch_pdl(k_prep<kFoldCertified>, g, kPrepBlock, 0, s, pdl, a);
+        default: return launch_pdl(k_prep<GCE_PHASE_FIXED32>, g, kPrepBlock, 0, s, pdl, a);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_table(unsigned long long *table, int n_max, cudaStream_t s) {

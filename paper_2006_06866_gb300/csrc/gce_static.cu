@@ -92,11 +92,6 @@ Layout layout(long long n_points, int n_curves, long long n_trials, int n_mag, i
     return L;
 }
 
-__global__ void k_iota(int *order, int n) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        order[i] = i;
-}
-
 gce_status setup(int dev, DeviceSetup *&out) {
     std::lock_guard<std::mutex> lock(g_mutex);
     if (dev < 0 || dev >= kMaxDevices) return fail(GCE_ERR_UNSUPPORTED, "device index too large");
@@ -201,6 +196,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     long long grid = (long long)d->n_sm * occ;
     if (grid > n_items) grid = n_items;
 
+    const bool pdl = true;  // (the call waits for its result, so never under capture)
     unsigned char *b = d->base;
     JobState *state = reinterpret_cast<JobState *>(b + L.state);
     long long *offsets = reinterpret_cast<long long *>(b + L.offsets);
@@ -208,10 +204,9 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     // offsets from the caller's host array (pageable: the copy is staged by the driver)
     e = cudaMemcpyAsync(offsets, h_offsets, 8 * (size_t)(n_curves + 1), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
-    k_iota<<<(n_curves + 255) / 256 < 1024 ? (n_curves + 255) / 256 : 1024, 256, 0, s>>>(order, n_curves);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
-    if ((e = launch_init(state, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
-    e = launch_scan(times, mags, n_points, periods, n_periods, pdots, n_pdots, cfg->t0, state, s);
+    e = launch_init(state, nullptr, nullptr, offsets, order, n_curves, s);
+    if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
+    e = launch_scan(times, mags, n_points, periods, n_periods, pdots, n_pdots, cfg->t0, state, pdl, s);
     if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     TrialArgs ta;
     ta.periods = periods;
@@ -220,7 +215,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     ta.n_pdots = n_pdots;
     ta.trialc = b + L.trialc;
     ta.state = state;
-    if ((e = launch_trials(mode, ta, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
+    if ((e = launch_trials(mode, ta, pdl, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     PrepArgs pa;
     pa.times = times;
     pa.mags = mags;
@@ -235,7 +230,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     pa.bands = nullptr;
     pa.band_stats = nullptr;
     pa.n_bands = 0;
-    if ((e = launch_prep(mode, pa, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
+    if ((e = launch_prep(mode, pa, pdl, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     MainArgs ma;
     ma.payload = mode == GCE_PHASE_FP64 ? nullptr : b + L.payload;
     ma.tau = reinterpret_cast<const double *>(b + (mode == GCE_PHASE_FP64 ? L.payload : L.tau));
@@ -269,11 +264,12 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     ma.overlap = (cfg->flags & GCE_FLAG_OVERLAP) ? 1 : 0;
     ma.half = half;
     ma.kv = kv;
+    ma.pdl = pdl ? 1 : 0;
     ma.state = state;
     if ((e = launch_main(kmode, tpt, block, (int)grid, smem, ma, s)) != cudaSuccess)
         return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     e = launch_topk_merge(ma.cand, n_curves, (int)n_lists, k, 1, topk_H, (long long *)topk_idx,
-                          nullptr, nullptr, nullptr, nullptr, state, s);
+                          nullptr, nullptr, nullptr, nullptr, state, pdl, s);
     if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     // device-side input checks: read the flags into host stack memory and wait
     unsigned int err = 0;

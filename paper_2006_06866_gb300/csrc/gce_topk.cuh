@@ -34,6 +34,6 @@ cudaError_t launch_topk_reduce(const unsigned long long *cand, int n_curves, int
                                int tiles_per_group, int n_groups, int stats_per,
                                const TileStats *stats,
                                unsigned long long *cand2, TileStats *stats2, const JobState *st,
-                               cudaStream_t s);
+                               bool pdl, cudaStream_t s);
 
 }  // namespace gce

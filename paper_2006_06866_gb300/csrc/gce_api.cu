@@ -20,6 +20,97 @@
 
 using namespace gce;
 
+namespace gce {
+
+int most_tpt(int mode) { return mode == GCE_PHASE_FP64 ? 2 : 4; }
+
+// The counter range of a job's SPLIT32 fold: narrow with a Pdot axis (every fold
+// re-reduced), else the shape's (mid: warps with many cycles re-reduce).
+int split_range(int mode, int n_pdots, int slot_range) {
+    if (mode != GCE_PHASE_SPLIT32) return RANGE_WIDE;
+    return n_pdots > 1 ? RANGE_NARROW : slot_range == 1 ? RANGE_MID : RANGE_WIDE;
+}
+
+// The launch shape of a job that was not tuned: 128 threads, and as many trials per
+// thread as leave about 16 warps of counters on an SM.  More trials share a point's
+// loads (and with a Pdot axis its period part) and give the fold independent chains;
+// more warps hide the sweeps.  SM cycles per warp and point-trial, 40 curves x 600
+// points x 1e5 trials, SPLIT32 / FIXED32, against the shape used before (256 x 2):
+//   15 bins 128 x 4 3.53 / 4.53 (3.80 / 4.78), 20 bins 3.89 / 4.75 (4.11 / 5.08), 24
+//   bins 4.41 / 5.02 and 128 x 2 4.29 / 5.08; 16 Pdot values: 15 bins 128 x 4 4.59 /
+//   5.13 (5.51 / 6.02), 31 bins 5.78 / 6.47 (6.29 / 6.87), 40 bins 7.27 / 8.23 and
+//   128 x 2 6.93 / 7.46; 50 bins 128 x 2 6.67 / 7.50 (8.84 / 7.18), 50 overlapping
+//   bins 128 x 1 6.12 / 7.03 (9.15 / 7.22) and with Pdot 128 x 2 8.01 / 9.08 (8.01 /
+//   8.77); 100 bins 128 x 1 11.2 / 11.6 (29.2 / 13.8).
+// (A plan takes 256 threads where 128 leave fewer warps on an SM.)  With a Pdot axis
+// a thread's trials are consecutive Pdot values, so few values leave some of its
+// trials empty: the trials per thread also minimise the padded axis times the cost of
+// a trial (1, 1.18, 1.7 at 4, 2, 1, from the figures above).
+gce_tuning default_tuning(const gce_config *cfg, int n_pdots) {
+    const int mode = cfg->phase_mode;
+    const bool overlap = (cfg->flags & GCE_FLAG_OVERLAP) != 0;
+    gce_tuning t;
+    t.block = 128;
+    t.ctas_per_sm = 0;
+    t.chunk = 2048;
+    t.slot_range = 1;
+    const bool pd_axis = n_pdots > 1;
+    const int slots = slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, n_pdots, 1));
+    t.tpt = slots <= (pd_axis ? 33 : 26) ? 4 : slots <= (overlap && !pd_axis ? 48 : 64) ? 2 : 1;
+    t.tpt = std::min(t.tpt, most_tpt(mode));
+    if (pd_axis) {
+        auto cost = [&](int tpt) {
+            return (double)((n_pdots + tpt - 1) / tpt * tpt) * (tpt == 4 ? 1.0 : tpt == 2 ? 1.18 : 1.7);
+        };
+        for (int tpt = t.tpt / 2; tpt >= 1; tpt /= 2)
+            if (cost(tpt) < cost(t.tpt)) t.tpt = tpt;
+    }
+    return t;
+}
+
+// Fewer trials per thread where the job's trials would not fill the device
+// otherwise.  w: warps per scheduler with one trial per thread.  SM cycles per warp
+// and point-trial of 300-point curves, SPLIT32 at 1 / 2 / 4 trials per thread: w =
+// 2.6 16.3 / 18.9 / -, w = 5.1 13.6 / 10.8 / 13.1, w = 8.2 - / 8.9 / 9.8, w = 16 - /
+// 6.9 / 7.5, w = 41 - / 5.8 / 5.7; FP64, whose warps wait longer, w = 8.2 12.8 / 13.8,
+// w = 16 10.5 / 9.2.
+// Jobs with the significance keep at least two wherever 256 threads x 2 trials have
+// always fitted (100 slots): its moments are summed per list of 64 trials.
+// Returns whether the CTA's warps should share one trial set: their points are then
+// counted 4 or 8 at a time, which pays while a curve's points, walked by a single
+// warp, outlast the barriers.  Against the shapes above, at w = 0.05 / 0.26 / 1.0 /
+// 2.6 / 4.1: 2000 points 286 -> 114, 57 -> 24, 16.9 -> 10.4, 7.8 -> 6.4, 7.6 -> 5.8
+// (FIXED32); 811 points 385 -> 207, 77 -> 47, 22.6 -> 15.5, 10.1 -> 9.1, 9.2 -> 7.9;
+// 300 points 670 -> 532, 139 -> 98, 37 -> 31, 16.7 -> 16.7, 13.8 -> 14.4; 100 points
+// 1600 -> 1400, 320 -> 281, 84 -> 80, 36 -> 38, 29 -> 35.
+bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_trials,
+                       int n_curves, long long n_points, int n_sm, bool stats) {
+    const int mode = cfg->phase_mode;
+    const long long warps = (n_trials + 31) / 32 * n_curves, schedulers = 4ll * n_sm;
+    const bool few = warps <= (mode == GCE_PHASE_FP64 ? 9 : 3) * schedulers;
+    const bool keep2 =
+        stats && slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, n_pdots, 0)) <= 100;
+    if (!(cfg->flags & GCE_FLAG_OVERLAP)) {
+        const bool very_few = 10 * warps <= 3 * schedulers;
+        // mean points per curve >= 200 w
+        if (very_few || (warps <= 6 * schedulers &&
+                         n_points / n_curves * schedulers >= 200 * warps)) {
+            t.block = very_few ? 256 : 128;
+            t.tpt = very_few && !keep2 ? 1 : 2;
+            return true;
+        }
+    }
+    if (warps <= 20 * schedulers) t.tpt = std::min(t.tpt, 2);
+    if (few && !stats) t.tpt = 1;
+    if (keep2) {
+        t.tpt = std::max(t.tpt, 2);
+        if (few) t.block = 64;
+    }
+    return false;
+}
+
+}  // namespace gce
+
 namespace {
 
 struct DevBuf {
@@ -58,10 +149,10 @@ struct Fingerprint {
     }
 };
 
-// The inputs of a launch shape's fitting (mode, bins, longest curve, top-k,
+// The inputs of a launch shape's fitting (mode, bins, longest curve,
 // slot range, the tuning's block / tpt / chunk / CTA cap) and its result, so
 // that repeated calls skip the driver queries of the fitting.
-typedef std::tuple<int, int, int, int, int, int, int, int, int, int> ShapeKey;
+typedef std::tuple<int, int, int, int, int, int, int, int, int> ShapeKey;
 struct LaunchShape {
     int block, tpt, chunk, table_smem, occ;
     size_t smem;
@@ -147,9 +238,6 @@ static gce_status ensure(gce_handle h, DevBuf &b, size_t bytes) {
     return GCE_OK;
 }
 
-// The CE kernel's fold for a job's phase mode: FP64 jobs run the certified one.
-static int kernel_mode(int mode) { return mode == GCE_PHASE_FP64 ? kFoldCertified : mode; }
-
 static int point_bytes(int mode) { return mode == GCE_PHASE_FP64 ? 8 : 16; }
 
 static size_t trial_bytes(int mode) {
@@ -164,81 +252,6 @@ static int ilog2_ceil(long long v) {
     int e = 0;
     while ((1ll << e) < v) ++e;
     return e;
-}
-
-static int most_tpt(int mode) { return mode == GCE_PHASE_FP64 ? 2 : 4; }
-
-// The counter range of a job's SPLIT32 fold: narrow with a Pdot axis (every fold
-// re-reduced), else the shape's (mid: warps with many cycles re-reduce).
-static int split_range(int mode, int n_pdots, int slot_range) {
-    if (mode != GCE_PHASE_SPLIT32) return RANGE_WIDE;
-    return n_pdots > 1 ? RANGE_NARROW : slot_range == 1 ? RANGE_MID : RANGE_WIDE;
-}
-
-// The launch shape of a job that was not tuned: 128 threads, and as many trials per
-// thread as leave about 16 warps of counters on an SM.  More trials share a point's
-// loads (and with a Pdot axis its period part) and give the fold independent chains;
-// more warps hide the sweeps.  SM cycles per warp and point-trial, 40 curves x 600
-// points x 1e5 trials, SPLIT32 / FIXED32, against the shape used before (256 x 2):
-//   15 bins 128 x 4 3.53 / 4.53 (3.80 / 4.78), 20 bins 3.89 / 4.75 (4.11 / 5.08), 24
-//   bins 4.41 / 5.02 and 128 x 2 4.29 / 5.08; 16 Pdot values: 15 bins 128 x 4 4.59 /
-//   5.13 (5.51 / 6.02), 31 bins 5.78 / 6.47 (6.29 / 6.87), 40 bins 7.27 / 8.23 and
-//   128 x 2 6.93 / 7.46; 50 bins 128 x 2 6.67 / 7.50 (8.84 / 7.18), 50 overlapping
-//   bins 128 x 1 6.12 / 7.03 (9.15 / 7.22) and with Pdot 128 x 2 8.01 / 9.08 (8.01 /
-//   8.77); 100 bins 128 x 1 11.2 / 11.6 (29.2 / 13.8).
-static gce_tuning default_tuning(const gce_config *cfg, int pd_axis) {
-    const int mode = cfg->phase_mode;
-    const bool overlap = (cfg->flags & GCE_FLAG_OVERLAP) != 0;
-    gce_tuning t;
-    t.block = 128;
-    t.ctas_per_sm = 0;
-    t.chunk = 2048;
-    t.slot_range = 1;
-    const int slots = slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, pd_axis ? 2 : 1, 1));
-    t.tpt = slots <= (pd_axis ? 33 : 26) ? 4 : slots <= (overlap && !pd_axis ? 48 : 64) ? 2 : 1;
-    t.tpt = std::min(t.tpt, most_tpt(mode));
-    return t;
-}
-
-// Fewer trials per thread where the job's trials would not fill the device
-// otherwise.  w: warps per scheduler with one trial per thread.  SM cycles per warp
-// and point-trial of 300-point curves, SPLIT32 at 1 / 2 / 4 trials per thread: w =
-// 2.6 16.3 / 18.9 / -, w = 5.1 13.6 / 10.8 / 13.1, w = 8.2 - / 8.9 / 9.8, w = 16 - /
-// 6.9 / 7.5, w = 41 - / 5.8 / 5.7; FP64, whose warps wait longer, w = 8.2 12.8 / 13.8,
-// w = 16 10.5 / 9.2.
-// Jobs with the significance keep at least two wherever 256 threads x 2 trials have
-// always fitted (100 slots): its moments are summed per list of 64 trials.
-// Returns whether the CTA's warps should share one trial set: their points are then
-// counted 4 or 8 at a time, which pays while a curve's points, walked by a single
-// warp, outlast the barriers.  Against the shapes above, at w = 0.05 / 0.26 / 1.0 /
-// 2.6 / 4.1: 2000 points 286 -> 114, 57 -> 24, 16.9 -> 10.4, 7.8 -> 6.4, 7.6 -> 5.8
-// (FIXED32); 811 points 385 -> 207, 77 -> 47, 22.6 -> 15.5, 10.1 -> 9.1, 9.2 -> 7.9;
-// 300 points 670 -> 532, 139 -> 98, 37 -> 31, 16.7 -> 16.7, 13.8 -> 14.4; 100 points
-// 1600 -> 1400, 320 -> 281, 84 -> 80, 36 -> 38, 29 -> 35.
-static bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_trials,
-                       int n_curves, long long n_points, int n_sm, bool stats) {
-    const int mode = cfg->phase_mode;
-    const long long warps = (n_trials + 31) / 32 * n_curves, schedulers = 4ll * n_sm;
-    const bool few = warps <= (mode == GCE_PHASE_FP64 ? 9 : 3) * schedulers;
-    const bool keep2 =
-        stats && slots_per_trial(mode, cfg->n_phase_bins, split_range(mode, n_pdots, 0)) <= 100;
-    if (!(cfg->flags & GCE_FLAG_OVERLAP)) {
-        const bool very_few = 10 * warps <= 3 * schedulers;
-        // mean points per curve >= 200 w
-        if (very_few || (warps <= 6 * schedulers &&
-                         n_points / n_curves * schedulers >= 200 * warps)) {
-            t.block = very_few ? 256 : 128;
-            t.tpt = very_few && !keep2 ? 1 : 2;
-            return true;
-        }
-    }
-    if (warps <= 20 * schedulers) t.tpt = std::min(t.tpt, 2);
-    if (few && !stats) t.tpt = 1;
-    if (keep2) {
-        t.tpt = std::max(t.tpt, 2);
-        if (few) t.block = 64;
-    }
-    return false;
 }
 
 static bool tuning_ok(const gce_tuning &t, int mode) {
@@ -256,14 +269,15 @@ static TuneKey tune_key(const gce_config *cfg, int n_obs, int pd_axis) {
 
 // The cached shape for the key (a Pdot-axis job without its own entry uses the
 // plain one), or the default one (*tuned = false).
-static gce_tuning lookup_tuning(gce_handle h, const gce_config *cfg, int n_max, int pd_axis,
+static gce_tuning lookup_tuning(gce_handle h, const gce_config *cfg, int n_max, int n_pdots,
                                 bool *tuned = nullptr) {
+    const int pd_axis = n_pdots > 1 ? 1 : 0;
     if (tuned) *tuned = true;
     auto it = h->tune.find(tune_key(cfg, n_max, pd_axis));
     if (it == h->tune.end() && pd_axis) it = h->tune.find(tune_key(cfg, n_max, 0));
     if (it != h->tune.end()) return it->second;
     if (tuned) *tuned = false;
-    return default_tuning(cfg, pd_axis);
+    return default_tuning(cfg, n_pdots);
 }
 
 extern "C" const char *gce_status_string(gce_status s) {
@@ -396,6 +410,75 @@ struct Plan {
     size_t smem;
 };
 
+// A launch shape fitted to the device for the plan's fold, slots and longest curve
+// (cached per handle).
+gce_status fit_shape(gce_handle h, const gce_config *cfg, const Plan &pl, const gce_tuning &t,
+                     LaunchShape &ls) {
+    const int kmode = kernel_mode(cfg->phase_mode), kv = pl.kv;
+    const ShapeKey skey(cfg->phase_mode, cfg->n_phase_bins, cfg->n_mag_bins, pl.n_max,
+                        pl.range * 8 + pl.half * 4 + kv, t.block, t.tpt, t.chunk, t.ctas_per_sm);
+    auto sit = h->shapes.find(skey);
+    if (sit != h->shapes.end()) {
+        ls = sit->second;
+        return GCE_OK;
+    }
+    ls.block = t.block;
+    ls.tpt = t.tpt;
+    ls.chunk = std::min(t.chunk, ((pl.n_max + 31) / 32) * 32);
+    // the c ln c table in shared memory: the whole table when it has at most
+    // 2048 entries (16 KB), so that lookups need no bounds test; longer curves
+    // read counts above it from global memory
+    ls.table_smem = std::min(pl.n_max + 1, 2048);
+    // shrink the staged chunk, then the table, then trials per thread, then the
+    // block, until the CTA fits in shared memory
+    auto size = [&]() {
+        return main_smem_bytes(kmode, trial_threads(kv, ls.block), ls.tpt, ls.chunk, cfg->n_phase_bins,
+                               cfg->n_mag_bins, ls.table_smem, pl.range, pl.half);
+    };
+    auto limit = [&]() {
+        return main_dynamic_smem_limit(kmode, ls.tpt, ls.block, kv, (size_t)h->smem_optin);
+    };
+    ls.smem = size();
+    while (ls.smem > limit()) {
+        if (ls.chunk > 512) ls.chunk /= 2;
+        else if (ls.table_smem > 256) ls.table_smem /= 2;
+        else if (ls.tpt > 1) ls.tpt /= 2;
+        else if (ls.block > 64) ls.block /= 2;
+        else if (ls.chunk > 64) ls.chunk /= 2;
+        else break;
+        ls.smem = size();
+    }
+    if (ls.smem > limit())
+        return fail(h, GCE_ERR_UNSUPPORTED, "launch shape needs %zu bytes of shared memory", ls.smem);
+    CUDA_TRY(h, main_kernel_attrs(kmode, ls.tpt, ls.block, kv, (size_t)h->smem_optin));
+    const void *kern = main_kernel_ptr(kmode, ls.tpt, ls.block, kv);
+    CUDA_TRY(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ls.occ, kern, ls.block, ls.smem));
+    if (ls.occ < 1) return fail(h, GCE_ERR_UNSUPPORTED, "launch shape does not fit on an SM");
+    // A smaller staged chunk costs only more staging passes: take it whenever it
+    // admits more CTAs per SM (the counters leave little room at many phase bins, so
+    // the tuned chunk can sit just past an occupancy step).
+    // Every halving down to 256 points is tried; the largest chunk that reaches
+    // the best occupancy is kept.
+    int best_chunk = ls.chunk;
+    size_t best_smem = ls.smem;
+    for (int c = ls.chunk; c > 256;) {
+        c = std::max(256, (c / 2 + 31) / 32 * 32);
+        ls.chunk = c;
+        const size_t sm2 = size();
+        int occ2 = 0;
+        CUDA_TRY(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, kern, ls.block, sm2));
+        if (occ2 > ls.occ) {
+            ls.occ = occ2;
+            best_chunk = c;
+            best_smem = sm2;
+        }
+    }
+    ls.chunk = best_chunk;
+    ls.smem = best_smem;
+    h->shapes[skey] = ls;
+    return GCE_OK;
+}
+
 // Curves of at most this many points are scheduled tile-major (Plan).
 constexpr long long kShortCurve = 256;
 
@@ -407,10 +490,9 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     for (int c = 0; c < j.n_curves; ++c) nmax = std::max<long long>(nmax, j.h_offsets[c + 1] - j.h_offsets[c]);
     pl.n_max = (int)nmax;
     bool tuned = true;
-    gce_tuning t = j.force ? *j.force : lookup_tuning(h, cfg, pl.n_max, j.n_pdots > 1 ? 1 : 0, &tuned);
+    gce_tuning t = j.force ? *j.force : lookup_tuning(h, cfg, pl.n_max, j.n_pdots, &tuned);
     const bool shared_set = !tuned && fit_to_job(t, cfg, j.n_pdots, pl.n_trials, j.n_curves,
                                                  pl.n_points, h->n_sm, j.rho != nullptr);
-    const int kk = j.kind == JOB_TOPK ? j.k : 0;
     pl.range = split_range(cfg->phase_mode, j.n_pdots, t.slot_range);
     // one Pdot value: the staging holds 8-byte half points
     pl.half = j.n_pdots == 1 ? 1 : 0;
@@ -420,78 +502,22 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     pl.kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
     if (shared_set && pl.kv == KV_SNAP) pl.kv = KV_SHARED;
     const int kv = pl.kv;
-    const ShapeKey skey(cfg->phase_mode, cfg->n_phase_bins, cfg->n_mag_bins, pl.n_max, kk,
-                        pl.range * 8 + pl.half * 4 + kv, t.block, t.tpt, t.chunk,
-                        t.ctas_per_sm);
-    int occ = 0;
-    auto sit = h->shapes.find(skey);
-    if (sit != h->shapes.end()) {
-        const LaunchShape &ls = sit->second;
-        pl.block = ls.block;
-        pl.tpt = ls.tpt;
-        pl.chunk = ls.chunk;
-        pl.table_smem = ls.table_smem;
-        pl.smem = ls.smem;
-        occ = ls.occ;
-    } else {
-        pl.block = t.block;
-        pl.tpt = t.tpt;
-        pl.chunk = std::min(t.chunk, ((pl.n_max + 31) / 32) * 32);
-        // the c ln c table in shared memory: the whole table when it has at most
-        // 2048 entries (16 KB), so that lookups need no bounds test; longer curves
-        // read counts above it from global memory
-        pl.table_smem = std::min(pl.n_max + 1, 2048);
-        // shrink the staged chunk, then the table, then trials per thread, then the
-        // block, until the CTA fits in shared memory
-        auto size = [&]() {
-            return main_smem_bytes(kmode, trial_threads(kv, pl.block), pl.tpt, pl.chunk, cfg->n_phase_bins,
-                                   cfg->n_mag_bins, pl.table_smem, pl.range, pl.half);
-        };
-        auto limit = [&]() {
-            return main_dynamic_smem_limit(kmode, pl.tpt, pl.block, kv, (size_t)h->smem_optin);
-        };
-        pl.smem = size();
-        while (pl.smem > limit()) {
-            if (pl.chunk > 512) pl.chunk /= 2;
-            else if (pl.table_smem > 256) pl.table_smem /= 2;
-            else if (pl.tpt > 1) pl.tpt /= 2;
-            else if (pl.block > 64) pl.block /= 2;
-            else if (pl.chunk > 64) pl.chunk /= 2;
-            else break;
-            pl.smem = size();
-        }
-        if (pl.smem > limit())
-            return fail(h, GCE_ERR_UNSUPPORTED, "launch shape needs %zu bytes of shared memory", pl.smem);
-        CUDA_TRY(h, main_kernel_attrs(kmode, pl.tpt, pl.block, kv, (size_t)h->smem_optin));
-        const void *kern = main_kernel_ptr(kmode, pl.tpt, pl.block, kv);
-        CUDA_TRY(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, pl.block, pl.smem));
-        if (occ < 1) return fail(h, GCE_ERR_UNSUPPORTED, "launch shape does not fit on an SM");
-        // A smaller staged chunk costs only more staging passes: take it whenever it
-        // admits more CTAs per SM (the counters leave little room at many phase bins,
-        // and the top-k buffer grows with k, so the tuned chunk can sit just past an
-        // occupancy step for another k).
-        // Every halving down to 256 points is tried; the largest chunk that reaches
-        // the best occupancy is kept.
-        {
-            int best_chunk = pl.chunk;
-            size_t best_smem = pl.smem;
-            for (int c = pl.chunk; c > 256;) {
-                c = std::max(256, (c / 2 + 31) / 32 * 32);
-                pl.chunk = c;
-                const size_t sm2 = size();
-                int occ2 = 0;
-                CUDA_TRY(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, kern, pl.block, sm2));
-                if (occ2 > occ) {
-                    occ = occ2;
-                    best_chunk = c;
-                    best_smem = sm2;
-                }
-            }
-            pl.chunk = best_chunk;
-            pl.smem = best_smem;
-        }
-        h->shapes[skey] = LaunchShape{pl.block, pl.tpt, pl.chunk, pl.table_smem, occ, pl.smem};
+    LaunchShape ls;
+    if (gce_status st = fit_shape(h, cfg, pl, t, ls)) return st;
+    if (!tuned && pl.kv != KV_SHARED && ls.block == 128 && ls.occ * ls.block < 512) {
+        gce_tuning wide = t;
+        wide.block = 256;
+        LaunchShape lw;
+        const std::string last = h->last_error;
+        if (fit_shape(h, cfg, pl, wide, lw) != GCE_OK) h->last_error = last;
+        else if (lw.tpt == ls.tpt && lw.occ * lw.block > ls.occ * ls.block) ls = lw;
     }
+    pl.block = ls.block;
+    pl.tpt = ls.tpt;
+    pl.chunk = ls.chunk;
+    pl.table_smem = ls.table_smem;
+    pl.smem = ls.smem;
+    int occ = ls.occ;
     const TileGrid tg = job_tiles(j.n_periods, j.n_pdots, trial_threads(kv, pl.block), pl.tpt);
     pl.n_tiles = (int)tg.n_tiles;
     pl.n_ptiles = tg.n_ptiles;
@@ -1063,7 +1089,7 @@ extern "C" gce_status gce_last_launches(gce_handle h, int32_t *n) {
 extern "C" gce_status gce_get_tuning(gce_handle h, const gce_config *cfg, int32_t n_obs_hint,
                                      int32_t n_pdots_hint, gce_tuning *t) {
     if (!h || !cfg || !t || n_pdots_hint < 1) return GCE_ERR_INVALID;
-    *t = lookup_tuning(h, cfg, std::max(1, n_obs_hint), n_pdots_hint > 1 ? 1 : 0);
+    *t = lookup_tuning(h, cfg, std::max(1, n_obs_hint), n_pdots_hint);
     return GCE_OK;
 }
 
@@ -1174,7 +1200,7 @@ extern "C" gce_status gce_autotune_job(gce_handle h, const double *times, const 
     cudaStream_t s = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     gce_status result = GCE_OK;
-    gce_tuning best = default_tuning(cfg, n_pdots > 1 ? 1 : 0);
+    gce_tuning best = default_tuning(cfg, n_pdots);
     gce_config c2cfg = *cfg;
     c2cfg.flags = (c2cfg.flags | GCE_FLAG_NO_GRAPH) & ~GCE_FLAG_TIME_KERNEL;
     do {
@@ -1249,7 +1275,7 @@ extern "C" gce_status gce_autotune(gce_handle h, const gce_config *cfg, int32_t 
     cudaStream_t s = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     gce_status result = GCE_OK;
-    gce_tuning best[2] = {default_tuning(cfg, 0), default_tuning(cfg, 1)};
+    gce_tuning best[2] = {default_tuning(cfg, 1), default_tuning(cfg, 8)};
     gce_config c2 = *cfg;
     c2.flags |= GCE_FLAG_NO_GRAPH;
     do {

@@ -633,6 +633,15 @@ inline int kernel_variant(bool overlap) { return overlap ? KV_OVL : KV_SNAP; }
 // threads of a CTA with trials (and counters) of their own
 inline int trial_threads(int kv, int block) { return kv == KV_SHARED ? 32 : block; }
 
+// The CE kernel's fold for a job's phase mode: FP64 jobs run the certified one.
+inline int kernel_mode(int mode) { return mode == GCE_PHASE_FP64 ? (int)kFoldCertified : mode; }
+// The launch shape of a job that was not tuned (gce_api.cu).
+int most_tpt(int mode);
+int split_range(int mode, int n_pdots, int slot_range);
+gce_tuning default_tuning(const gce_config *cfg, int n_pdots);
+bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_trials,
+                int n_curves, long long n_points, int n_sm, bool stats);
+
 // Programmatic dependent launch.  A call's kernels follow one another on one stream
 // and most are short, so each is launched while the one before it still runs and
 // waits on the device: pdl_wait() returns when everything before it has completed
@@ -660,7 +669,11 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), unsigned int grid, unsigned 
 
 // Kernel launchers (defined in the .cu files).
 // h_offsets, h_order: pinned host memory read by the kernel itself (nullptr: offsets
-// are on the device already, and the order is 0, 1, ...)
+// are on the device already, and the order is 0, 1, ...); launch_init_few takes the
+// offsets of at most kFewCurves curves from any host memory, as a kernel argument
+constexpr int kFewCurves = 255;
+cudaError_t launch_init_few(JobState *st, const int64_t *h_offsets, long long *offsets, int *order,
+                            int n_curves, cudaStream_t s);
 cudaError_t launch_init(JobState *st, const long long *h_offsets, const int *h_order,
                         long long *offsets, int *order, int n_curves, cudaStream_t s);
 cudaError_t launch_scan(const double *times, const double *mags, long long n_points,

@@ -15,22 +15,35 @@ constexpr unsigned long long kPosInfBits = 0x7ff0000000000000ull;
 // The job state cleared, and the curves' offsets and processing order copied from
 // the caller-side staging buffers (pinned host memory, read over the link: two copies
 // on the stream cost more than the whole kernel for small batches).
+__device__ __forceinline__ void clear_state(JobState *st) {
+    st->tau_max_bits = 0ull;
+    st->pmin_bits = kPosInfBits;
+    st->pdot_max_bits = 0ull;
+    st->err = 0u;
+    st->work = 0ull;
+    st->wide = 0u;
+}
 __global__ void k_init(JobState *st, const long long *h_offsets, const int *h_order,
                        long long *offsets, int *order, int n_curves) {
     pdl_trigger();
     const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i0 == 0) {
-        st->tau_max_bits = 0ull;
-        st->pmin_bits = kPosInfBits;
-        st->pdot_max_bits = 0ull;
-        st->err = 0u;
-        st->work = 0ull;
-        st->wide = 0u;
-    }
+    if (i0 == 0) clear_state(st);
     for (int i = i0; i <= n_curves; i += gridDim.x * blockDim.x) {
         if (h_offsets) offsets[i] = h_offsets[i];
         if (i < n_curves) order[i] = h_order ? h_order[i] : i;
     }
+}
+
+struct FewOffsets {
+    int64_t v[kFewCurves + 1];
+};
+__global__ void k_init_few(JobState *st, const __grid_constant__ FewOffsets few, long long *offsets,
+                           int *order, int n_curves) {
+    pdl_trigger();
+    const int i = threadIdx.x;
+    if (i == 0) clear_state(st);
+    if (i <= n_curves) offsets[i] = few.v[i];
+    if (i < n_curves) order[i] = i;
 }
 
 // Non-negative binary64 values order like their bit patterns, so maxima and
@@ -559,6 +572,15 @@ cudaError_t launch_init(JobState *st, const long long *h_offsets, const int *h_o
                         long long *offsets, int *order, int n_curves, cudaStream_t s) {
     k_init<<<grid_for((long long)n_curves + 1, 256, 152), 256, 0, s>>>(st, h_offsets, h_order,
                                                                        offsets, order, n_curves);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init_few(JobState *st, const int64_t *h_offsets, long long *offsets, int *order,
+                            int n_curves, cudaStream_t s) {
+    if (n_curves > kFewCurves) return cudaErrorInvalidValue;
+    FewOffsets few;
+    for (int i = 0; i <= kFewCurves; ++i) few.v[i] = h_offsets[i <= n_curves ? i : n_curves];
+    k_init_few<<<1, kFewCurves + 1, 0, s>>>(st, few, offsets, order, n_curves);
     return cudaGetLastError();
 }
 

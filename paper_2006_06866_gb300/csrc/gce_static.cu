@@ -30,9 +30,12 @@
 // The call runs on the current device.  Every device array it is given must
 // live on that device (checked with cudaPointerGetAttributes; memory of another
 // device is GCE_ERR_INVALID).
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <map>
 #include <mutex>
+#include <utility>
 
 #include "gce_internal.cuh"
 
@@ -48,6 +51,8 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 struct DeviceSetup {
     bool done = false;
+    // CTAs per SM of the launch shapes used so far (0: does not fit)
+    std::map<std::pair<const void *, size_t>, int> occ;
     unsigned char *base = nullptr;  // device address of g_scratch
     int n_sm = 0;
     int smem_optin = 0;
@@ -103,6 +108,7 @@ gce_status setup(int dev, DeviceSetup *&out) {
         // first use on this device, or the module was loaded anew (the array moved
         // and its table is gone): fill the c ln c table again
         d.done = false;
+        d.occ.clear();
         e = cudaDeviceGetAttribute(&d.n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
         e = cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -115,6 +121,24 @@ gce_status setup(int dev, DeviceSetup *&out) {
     }
     out = &d;
     return GCE_OK;
+}
+
+// CTAs per SM of a kernel with smem bytes of dynamic shared memory (0: none), from
+// the driver the first time.
+int fitted(DeviceSetup *d, const void *kern, int kmode, int tpt, int block, int kv, size_t smem) {
+    std::lock_guard<std::mutex> lock(g_mutex);
+    const auto key = std::make_pair(kern, smem);
+    const auto it = d->occ.find(key);
+    if (it != d->occ.end()) return it->second;
+    int occ = 0;
+    if (!kern || smem > main_dynamic_smem_limit(kmode, tpt, block, kv, (size_t)d->smem_optin) ||
+        main_kernel_attrs(kmode, tpt, block, kv, (size_t)d->smem_optin) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess) {
+        cudaGetLastError();
+        occ = 0;
+    }
+    if (d->occ.size() >= 256) d->occ.clear();
+    return d->occ[key] = occ;
 }
 
 // A device array of the call must be on the current device: memory that the
@@ -153,45 +177,72 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
         if (!on_device(a, dev)) return fail(GCE_ERR_INVALID, "an array is on another device");
     cudaStream_t s = (cudaStream_t)stream;
     // FP64 jobs run the CE kernel's certified fold
-    const int kmode = cfg->phase_mode == GCE_PHASE_FP64 ? (int)kFoldCertified : cfg->phase_mode;
-
-    // launch shape: block 256, 2 trials per thread, the curve staged in chunks
+    const int kmode = kernel_mode(cfg->phase_mode);
+    const bool overlap = (cfg->flags & GCE_FLAG_OVERLAP) != 0;
     long long n_max = 1;
     for (int c = 0; c < n_curves; ++c)
         n_max = h_offsets[c + 1] - h_offsets[c] > n_max ? h_offsets[c + 1] - h_offsets[c] : n_max;
     const long long n_points = h_offsets[n_curves];
     const long long n_trials = (long long)n_periods * n_pdots;
-    const int block = 256, tpt = 2;
-    int chunk = (int)((n_max + 31) / 32 * 32);
-    if (chunk > 1024) chunk = 1024;
-    int table_smem = (int)(n_max + 1 < 1024 ? n_max + 1 : 1024);
-    const int range = (kmode == GCE_PHASE_SPLIT32 && n_pdots > 1) ? RANGE_NARROW : RANGE_WIDE;
+    const int table_smem = (int)(n_max + 1 < 1024 ? n_max + 1 : 1024);
+    const int chunk_max = (int)std::min<long long>(1024, (n_max + 31) / 32 * 32);
     const int half = n_pdots == 1 ? 1 : 0;
-    const size_t smem = main_smem_bytes(kmode, block, tpt, chunk, cfg->n_phase_bins,
-                                        cfg->n_mag_bins, table_smem, range, half);
-    const int kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
-    if (smem > main_dynamic_smem_limit(kmode, tpt, block, kv, (size_t)d->smem_optin))
+
+    // what this entry point takes: jobs whose counters (all slots), candidates and own
+    // payload fit with 256 threads x 2 trials
+    const int all_slots = split_range(cfg->phase_mode, n_pdots, 0);
+    if (main_smem_bytes(cfg->phase_mode, 256, 2, chunk_max, cfg->n_phase_bins, cfg->n_mag_bins,
+                        table_smem, all_slots, half) >
+        main_dynamic_smem_limit(kmode, 2, 256, kernel_variant(overlap), (size_t)d->smem_optin))
         return fail(GCE_ERR_UNSUPPORTED, "bin counts too large for this entry point");
-    const TileGrid tg = job_tiles(n_periods, n_pdots, block, tpt);
-    const long long n_tiles = tg.n_tiles;
-    const long long n_lists = n_tiles * (block / 32);  // one candidate list per warp and tile
-    // the certified payload and its tau take 24 bytes per point; where they don't
-    // fit, the binary64 payload's 8 may
-    int mode = kmode;
-    Layout L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 16,
-                      kmode == kFoldCertified ? 8 : 0, n_lists, k);
-    if (L.end > kScratchBytes && kmode == kFoldCertified) {
-        mode = GCE_PHASE_FP64;
-        L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 8, 0, n_lists, k);
-    }
-    if (L.end > kScratchBytes)
+    const long long lists256 = job_tiles(n_periods, n_pdots, 256, 2).n_tiles * 8;
+    if (layout(n_points, n_curves, n_trials, cfg->n_mag_bins, cfg->phase_mode == GCE_PHASE_FP64 ? 8 : 16,
+               0, lists256, k).end > kScratchBytes)
         return fail(GCE_ERR_NOMEM, "job needs more than the 32 MiB of built-in scratch");
 
-    e = main_kernel_attrs(kmode, tpt, block, kv, (size_t)d->smem_optin);
-    if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
+    // the launch shape: the job's own, or where that needs more scratch or shared
+    // memory, 256 threads x 2 trials
+    gce_tuning t = default_tuning(cfg, n_pdots);
+    int kv = kernel_variant(overlap);
+    if (fit_to_job(t, cfg, n_pdots, n_trials, n_curves, n_points, d->n_sm, false) && !overlap)
+        kv = KV_SHARED;
+    int chunk = chunk_max, range = split_range(cfg->phase_mode, n_pdots, t.slot_range), mode = kmode;
+    size_t smem = 0;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, main_kernel_ptr(kmode, tpt, block, kv), block, smem);
-    if (e != cudaSuccess || occ < 1) return fail(GCE_ERR_CUDA, "occupancy query failed");
+    long long n_lists = 0, n_tiles = 0;
+    TileGrid tg{};
+    Layout L{};
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if (attempt == 1) {
+            t.block = 256;
+            t.tpt = 2;
+            kv = kernel_variant(overlap);
+            range = all_slots;
+            // (16-byte certified points in the bytes of FP64's 8)
+            if (kmode == kFoldCertified && !half) chunk = chunk_max / 2;
+        }
+        const int tb = trial_threads(kv, t.block);
+        smem = main_smem_bytes(kmode, tb, t.tpt, chunk, cfg->n_phase_bins, cfg->n_mag_bins, table_smem,
+                               range, half);
+        occ = fitted(d, main_kernel_ptr(kmode, t.tpt, t.block, kv), kmode, t.tpt, t.block, kv, smem);
+        if (occ < 1) continue;
+        tg = job_tiles(n_periods, n_pdots, tb, t.tpt);
+        n_tiles = tg.n_tiles;
+        n_lists = n_tiles * (tb / 32);  // one candidate list per warp and tile
+        // the certified payload and its tau take 24 bytes per point; where they don't
+        // fit, the binary64 payload's 8 may
+        mode = kmode;
+        L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 16, kmode == kFoldCertified ? 8 : 0,
+                   n_lists, k);
+        if (L.end > kScratchBytes && kmode == kFoldCertified) {
+            mode = GCE_PHASE_FP64;
+            L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 8, 0, n_lists, k);
+        }
+        if (L.end <= kScratchBytes) break;
+        occ = 0;
+    }
+    if (occ < 1) return fail(GCE_ERR_CUDA, "occupancy query failed");
+    const int block = t.block, tpt = t.tpt;
     const long long n_items = (long long)n_curves * n_tiles;
     long long grid = (long long)d->n_sm * occ;
     if (grid > n_items) grid = n_items;
@@ -201,10 +252,14 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     JobState *state = reinterpret_cast<JobState *>(b + L.state);
     long long *offsets = reinterpret_cast<long long *>(b + L.offsets);
     int *order = reinterpret_cast<int *>(b + L.order);
-    // offsets from the caller's host array (pageable: the copy is staged by the driver)
-    e = cudaMemcpyAsync(offsets, h_offsets, 8 * (size_t)(n_curves + 1), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
-    e = launch_init(state, nullptr, nullptr, offsets, order, n_curves, s);
+    // offsets from the caller's host array: few of them as a kernel argument, else a
+    // copy (pageable, staged by the driver)
+    if (n_curves <= kFewCurves) {
+        e = launch_init_few(state, h_offsets, offsets, order, n_curves, s);
+    } else {
+        e = cudaMemcpyAsync(offsets, h_offsets, 8 * (size_t)(n_curves + 1), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = launch_init(state, nullptr, nullptr, offsets, order, n_curves, s);
+    }
     if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     e = launch_scan(times, mags, n_points, periods, n_periods, pdots, n_pdots, cfg->t0, state, pdl, s);
     if (e != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));

@@ -1,8 +1,10 @@
 // Trial-independent preparation (O(sum N + n_trials)): input checks and
 // maxima, per-trial fold constants, per-curve magnitude binning with the
 // points regrouped by magnitude bin, and the c ln c fixed-point table.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <numeric>
 
 #include "gce_internal.cuh"
 
@@ -36,6 +38,7 @@ __global__ void k_init(JobState *st, const long long *h_offsets, const int *h_or
 
 struct FewOffsets {
     int64_t v[kFewCurves + 1];
+    unsigned char order[kFewCurves + 1];  // longest curve first
 };
 __global__ void k_init_few(JobState *st, const __grid_constant__ FewOffsets few, long long *offsets,
                            int *order, int n_curves) {
@@ -43,7 +46,7 @@ __global__ void k_init_few(JobState *st, const __grid_constant__ FewOffsets few,
     const int i = threadIdx.x;
     if (i == 0) clear_state(st);
     if (i <= n_curves) offsets[i] = few.v[i];
-    if (i < n_curves) order[i] = i;
+    if (i < n_curves) order[i] = few.order[i];
 }
 
 // Non-negative binary64 values order like their bit patterns, so maxima and
@@ -580,6 +583,10 @@ cudaError_t launch_init_few(JobState *st, const int64_t *h_offsets, long long *o
     if (n_curves > kFewCurves) return cudaErrorInvalidValue;
     FewOffsets few;
     for (int i = 0; i <= kFewCurves; ++i) few.v[i] = h_offsets[i <= n_curves ? i : n_curves];
+    std::iota(few.order, few.order + n_curves, (unsigned char)0);
+    std::stable_sort(few.order, few.order + n_curves, [&](int a, int b) {
+        return h_offsets[a + 1] - h_offsets[a] > h_offsets[b + 1] - h_offsets[b];
+    });
     k_init_few<<<1, kFewCurves + 1, 0, s>>>(st, few, offsets, order, n_curves);
     return cudaGetLastError();
 }

@@ -58,9 +58,10 @@ typedef enum {
     /* binary64 with the operation sequence s = tau*f, b = a*tau,
      * x = fma(-b, tau, s), phi = x - floor(x), j = floor(phi*n_phase) (clamped),
      * f = 1/P, a = (0.5*Pdot)*f*f.  Counts are bit-identical to a CPU binary64
-     * evaluation of that sequence.  (Within FIXED32's range the search evaluates
-     * the sequence itself only for points whose fixed-point phase lies so close
-     * to a phase-bin edge that the two folds could disagree.) */
+     * evaluation of that sequence.  (Up to 2^21 cycles and 2^18 Pdot cycles the
+     * search evaluates the sequence itself only for points whose phase, from a
+     * coarser fixed-point fold, lies so close to a phase-bin edge that the two
+     * could disagree; beyond them, for all, at the speed of binary64.) */
     GCE_PHASE_FP64 = 0,
     /* FP32 double-float: tau, tau^2, f and a split into (hi, lo) float pairs,
      * error-free products via fmaf, integer cycles removed with a rounding
@@ -72,7 +73,8 @@ typedef enum {
      * away).  The large partial products are integer multiplies, the small
      * cross terms FP32 multiply-adds.  Phase error a few 2^-32 cycles up to
      * about 2^22 cycles, growing to ~6e-8 cycles at the limit; needs |tau|/P <
-     * 2^28 and |Pdot| tau^2/P^2 < 2^16 cycles. */
+     * 2^28 and |Pdot| tau^2/P^2 < 2^16 cycles.  (Like FP64's, its sequence is
+     * evaluated only near the edges up to 2^21 cycles.) */
     GCE_PHASE_FIXED32 = 2
 } gce_phase_mode;
 
@@ -123,9 +125,9 @@ typedef struct gce_handle_s *gce_handle;
  * thread).  The handle owns the device workspace, the autotune cache and the
  * captured CUDA graphs.  *h is NULL on failure.
  * The workspace grows to the largest job seen and is kept until gce_destroy:
- * 16 bytes per point (FP64: 24), 16 (SPLIT32) or 32 (FIXED32, FP64) bytes per
- * (P, Pdot) trial (where FP64's do not fit, 8 per point and 16 per trial, at
- * the speed of binary64 arithmetic), 8 k bytes per (curve, warp of a trial tile) for top-k (24 more with
+ * 16 bytes per point (FP64 and FIXED32: 32), 16 (SPLIT32) or 32 (FIXED32, FP64)
+ * bytes per (P, Pdot) trial (where those of FP64 or FIXED32 do not fit, 8 or 16
+ * per point and 16 or 32 per trial, at the speed of their own folds), 8 k bytes per (curve, warp of a trial tile) for top-k (24 more with
  * the significance), and 8 bytes per entry of the c ln c table (longest curve
  * + 1).  A grid of 5,183,995 periods x 512 Pdot values thus holds 42 GB of
  * trial constants in SPLIT32.  Growing a buffer waits for the device. */

@@ -238,7 +238,9 @@ static gce_status ensure(gce_handle h, DevBuf &b, size_t bytes) {
     return GCE_OK;
 }
 
-static int point_bytes(int mode) { return mode == GCE_PHASE_FP64 ? 8 : 16; }
+static int point_bytes(int mode) {
+    return coarse_mode(mode) ? (int)sizeof(CoarsePoint) : mode == GCE_PHASE_FP64 ? 8 : 16;
+}
 
 static size_t trial_bytes(int mode) {
     switch (mode) {
@@ -403,9 +405,9 @@ struct Plan {
     int n_max, n_tiles, n_ptiles, pd_major, range, half, kv, block, tpt, grid, chunk, table_smem,
         grab;
     int n_groups, tiles_per_group;  // top-k: first merge level (0 groups: none)
-    // the payload's fold mode: kernel_mode(), or GCE_PHASE_FP64 for the diagnostic
-    // jobs and for an FP64 job whose certified payload (24 bytes per point and 32
-    // per trial instead of 8 and 16) does not fit the device
+    // the payload's fold mode: kernel_mode(), or the job's phase mode itself for the
+    // diagnostic jobs and where the coarse payload (32 bytes per point and per trial
+    // instead of FP64's 8 and 16 or FIXED32's 16 and 32) does not fit the device
     int prep_mode;
     size_t smem;
 };
@@ -497,7 +499,9 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     // one Pdot value: the staging holds 8-byte half points
     pl.half = j.n_pdots == 1 ? 1 : 0;
     const int kmode = kernel_mode(cfg->phase_mode);
-    pl.prep_mode = (j.kind == JOB_GRID || j.kind == JOB_TOPK) ? kmode : cfg->phase_mode;
+    pl.prep_mode = (j.kind == JOB_GRID || j.kind == JOB_TOPK)
+                       ? job_prep_mode(cfg, pl.n_trials, j.n_pdots, j.n_curves, h->n_sm)
+                       : cfg->phase_mode;
     // the kernel instantiation: overlapping bins, a shared trial set, or neither
     pl.kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
     if (shared_set && pl.kv == KV_SNAP) pl.kv = KV_SHARED;
@@ -631,10 +635,7 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
     ma.tau = (const double *)h->tau.p;
     ma.periods = j.periods;
     ma.pdots = j.pdots;
-    if ((j.kind == JOB_GRID || j.kind == JOB_TOPK) && mode == GCE_PHASE_FP64) {
-        ma.tau = (const double *)h->payload.p;  // binary64 fold alone
-        ma.payload = nullptr;
-    }
+    ma.plain = mode == kmode ? 0 : 1;
     ma.state = st;
     const bool timed = (cfg->flags & GCE_FLAG_TIME_KERNEL) != 0;
     gce_status ms;
@@ -750,12 +751,12 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
     if (st != GCE_OK) return st;
 
     // workspace
-    if (pl.prep_mode == kFoldCertified &&
+    if (coarse_mode(pl.prep_mode) &&
         (ensure(h, h->tau, 8 * (size_t)pl.n_points) != GCE_OK ||
-         ensure(h, h->payload, (size_t)point_bytes(kFoldCertified) * pl.n_points) != GCE_OK ||
-         ensure(h, h->trialc, trial_bytes(kFoldCertified) * (size_t)pl.n_trials) != GCE_OK)) {
+         ensure(h, h->payload, (size_t)point_bytes(pl.prep_mode) * pl.n_points) != GCE_OK ||
+         ensure(h, h->trialc, trial_bytes(pl.prep_mode) * (size_t)pl.n_trials) != GCE_OK)) {
         h->last_error.clear();
-        pl.prep_mode = GCE_PHASE_FP64;
+        pl.prep_mode = j.cfg->phase_mode;
     }
     const int mode = pl.prep_mode;
     if ((st = ensure(h, h->payload, (size_t)point_bytes(mode) * pl.n_points)) != GCE_OK) return st;

@@ -22,8 +22,8 @@ struct JobState {
     unsigned long long pdot_max_bits;   // max |Pdot| as binary64 bits
     unsigned long long work;            // next work item (persistent kernel)
     unsigned int err;                   // ERR_* bits
-    // FP64 jobs prepared for the certified fold: 1 when the job's range is beyond
-    // it, so that the binary64 fold runs on every point (set by k_trials)
+    // FP64 and FIXED32 jobs prepared for the coarse fold: 1 when the job's range is
+    // beyond it, so that the mode's own fold runs on every point (set by k_trials)
     unsigned int wide;
     unsigned int pad[2];
 };
@@ -37,10 +37,14 @@ enum : unsigned int {
     ERR_SLOT = 32u,     // checked builds only: a counter slot outside the trial's kept range
 };
 
-// The CE kernel's fold of a GCE_PHASE_FP64 job (not part of the ABI): the FIXED32
-// fold with every point's distance to the phase-bin edges checked against the two
-// folds' error bound, and the binary64 fold for the points within it.
-enum { kFoldCertified = 3 };
+// The CE kernel's modes of GCE_PHASE_FP64 and GCE_PHASE_FIXED32 jobs (not part of
+// the ABI): a coarser fixed-point fold with every point's distance to the phase-bin
+// edges checked against the folds' error bounds, and the mode's own fold for the
+// points within them.
+enum { kJobFp64 = 3, kJobFixed32 = 4 };
+__host__ __device__ constexpr bool coarse_mode(int mode) {
+    return mode == kJobFp64 || mode == kJobFixed32;
+}
 
 // Whether a job's maxima lie inside the FIXED32 fold's range: F < 2^63, and the
 // Pdot cross term small enough for its FP32 path.
@@ -112,14 +116,27 @@ template <> struct ModeTraits<GCE_PHASE_FIXED32> {
     __device__ static point_t widen(half_t h) { return make_uint4(h.x, h.y, 0u, 0u); }
 };
 
-// FP64 jobs: FIXED32 points and trials; the binary64 tau of each point is kept
-// beside them (MainArgs::tau) for the points within the error bound of an edge.
-template <> struct ModeTraits<kFoldCertified> {
-    typedef uint4 point_t;
-    typedef uint2 half_t;
-    typedef FixedTrial trial_t;
-    __device__ static point_t widen(half_t h) { return make_uint4(h.x, h.y, 0u, 0u); }
+// The coarse fold's points and trials (see coarse_margin); the binary64 tau of each
+// point is kept beside them (MainArgs::tau) for the points near an edge.
+struct CoarsePoint {
+    unsigned int T1;
+    float T1f, b;
+    unsigned int U1;
+    float U1f, ub;
 };
+struct __align__(16) CoarseTrial {
+    unsigned int F1;
+    float F0, F1f;
+    unsigned int A1;
+    float A0, A1f;
+    unsigned int margin, pad;
+};
+template <> struct ModeTraits<kJobFp64> {
+    typedef CoarsePoint point_t;
+    typedef CoarsePoint half_t;
+    typedef CoarseTrial trial_t;
+};
+template <> struct ModeTraits<kJobFixed32> : ModeTraits<kJobFp64> {};
 
 // Balanced split of a 64-bit value: x = hi 2^32 + lo with lo a signed 32-bit
 // value in [-2^31, 2^31), so that signed multiply-high works on it.
@@ -388,21 +405,115 @@ __device__ __forceinline__ unsigned int fold_fixed_bin_from(unsigned int acc, ui
     return __umulhi(fold_fixed_phase_from<PDOT, K0>(acc, pt, t), n_phase);
 }
 
-// The certified fold's margin, in units of 2^-32 cycles: above the distance
-// between the FIXED32 phase and the phase of the binary64 sequence, which the
-// bounds below add up to, and at least twice their sum.
-//   FIXED32 against tau f - a tau^2: T and F rounded to their limbs (1/4 + 1/8),
-//   the floor of hi32(T1 F0) (1), T0 F0 / 2^64 dropped (1/2), T0 >> 9 (F1 2^-23 <=
-//   2^(k-1)), G0 rounded (2^(k-2)), K and the FMA rounded (2^k); with a Pdot term U
-//   and A rounded (1/8), the floor of hi32(A0 U1) (1), A0 U0 dropped (1/2), U0 >> 9
-//   (1/8), one more FMA rounding (2^(k-1)), and, where the two cross terms carry the
-//   FMA result past 2^24, its coarser grid (|A1| / 4 + 2^k).  The binary64 sequence
-//   against the same: 2^-53 (2 |tau f| + 2 |a tau^2| + 3) cycles <= 2^k + 1, as
-//   |tau f| < F1 / 4 <= 2^(20+k) cycles and |a tau^2| < 2^18.
-// Sum: below 5 + 5 2^k + |A1| / 4.
-__device__ __forceinline__ unsigned int certified_margin(unsigned int k, unsigned int a1) {
-    const int a = (int)a1;
-    return 16u + (10u << k) + (unsigned int)(a < 0 ? -a : a);
+// x 2^e as ldexp rounds it: one multiplication where 2^e is a normal number.
+__device__ __forceinline__ double scale2(double x, int e) {
+    if (e < -1022 || e > 1023) return ldexp(x, e);
+    return __dmul_rn(x, __longlong_as_double((long long)(e + 1023) << 52));
+}
+
+// A point and a trial in the FIXED32 formats (the preparation of plain and
+// out-of-range jobs, and the CE kernel for the points the coarse fold leaves to it).
+__device__ inline uint4 fixed_point(double tau, const FixedScale &fs) {
+    // T = round(tau 2^s), |T| < 2^62; U = floor(T^2 / 2^62) = tau^2 2^u computed
+    // exactly from T in 128-bit integer arithmetic.
+    const long long T = __double2ll_rn(scale2(tau, fs.s));
+    const unsigned long long aT = (unsigned long long)(T < 0 ? -T : T);
+    const unsigned long long hi = __umul64hi(aT, aT), lw = aT * aT;
+    const long long U = (long long)((hi << 2) | (lw >> 62));
+    int u1, u0;
+    split_balanced(U, &u1, &u0);
+    const unsigned int t0 = (unsigned int)(T & 0xffffffffll);
+    return make_uint4((unsigned int)(int)(T >> 32), 0x4B000000u | (t0 >> 9),  // 2^23 + (T0 >> 9)
+                      (unsigned int)u1,
+                      0x4B000000u | (((unsigned int)u0 ^ 0x80000000u) >> 9));  // 2^23 + ((U0+2^31) >> 9)
+}
+__device__ inline FixedTrial fixed_trial(double f, double aa, const FixedScale &fs) {
+    FixedTrial v;
+    // Out-of-range values are flagged by the range check; clamp so the conversions stay defined.
+    const double F = fmin(scale2(f, fs.r), 9.2e18);
+    const double A = fmax(fmin(scale2(aa, fs.v), 9.2e18), -9.2e18);
+    int f1, f0;
+    split_balanced(__double2ll_rn(F), &f1, &f0);
+    const long long an = -__double2ll_rn(A);
+    const int a1 = (int)(an >> 32);
+    const unsigned int a0 = (unsigned int)(an & 0xffffffffll);
+    // k: the smallest shift with F1 < 2^(22+k)
+    const unsigned int uf1 = (unsigned int)f1;
+    const int bits = 32 - __clz(uf1);
+    const int k = bits > 22 ? bits - 22 : 0;
+    const float g0 = __double2float_rn(scale2((double)uf1, -23 - k));
+    const float g2 = __double2float_rn(scale2((double)a1, -23 - k));
+    const double kk = 12582912.0 - 8388608.0 * (double)g0 - 8388608.0 * (double)g2 -
+                      scale2((double)a1, -1 - k);
+    v.i = make_uint4(uf1, (unsigned int)f0, (unsigned int)a1, a0);
+    v.f = make_float4(g0, g2, __double2float_rn(kk), __uint_as_float((unsigned int)k));
+    return v;
+}
+
+// The coarse fold (FP64 and FIXED32 jobs).  FIXED32's construction with fewer integer
+// multiplies: with T = tau 2^(58-e) = T1 2^32 + T0 and F = f 2^(38+e) = F1 2^32 + F0,
+// both balanced, the phase in units of 2^-32 cycles is
+//   lo32(T1 F1) + (T1 F0 + T0 F1) / 2^32   (+ T0 F0 / 2^64),
+// the first an exact integer product, the rest two FP32 FMAs into 1.5 2^29, whose
+// result's bit pattern counts 64 units per step and joins by one shift-add.  -a tau^2
+// is the same with U = tau^2 2^(58-2e) and A = -a 2^(38+2e).  The high-half multiplies
+// that bound FIXED32 (a quarter of the FMA rate) are left only in the bin.
+//   Range: cycles < 2^21 (F1 < 2^28) and Pdot cycles < 2^18 (A1 < 2^26), so that the
+//   FMA results stay within 2^28 of the constant.
+//   Error, in units: T1 and F0 as floats 2, T0 and F1 8, two FMA roundings 64, the
+//   dropped product and the limbs' own rounding 1: 75; with Pdot U1 and A0 2, U0 and
+//   A1 2, two more roundings 64, dropped and rounded 1: 69 more.
+//   The mode's own fold: binary64 2^-53 (2 cycles + 2 Pdot cycles + 3) of a cycle: 3;
+//   FIXED32 5 + 5 2^k (its limbs, floors, truncations and roundings), and |A1| / 4 +
+//   2^k more where its two FP32 terms could carry the sum past 2^24 (its A1).
+// coarse_margin is 5/4 of the sum and 8.  With w = (phase + margin) n_phase, the bin
+// is hi32(w), and it is the own fold's too unless lo32(w) < 2 margin n_phase.
+constexpr float kCoarseRound = 805306368.0f;  // 1.5 2^29
+constexpr unsigned int kCoarseOffset = 0u - (0x4E400000u << 6);  // cancels its bits
+__device__ inline CoarsePoint coarse_point(double tau, int e) {
+    CoarsePoint p;
+    int hi, lo;
+    split_balanced(__double2ll_rn(scale2(tau, 58 - e)), &hi, &lo);
+    p.T1 = (unsigned int)hi;
+    p.T1f = (float)hi;
+    p.b = (float)lo * 2.3283064365386963e-10f;  // 2^-32
+    split_balanced(__double2ll_rn(scale2(__dmul_rn(tau, tau), 58 - 2 * e)), &hi, &lo);
+    p.U1 = (unsigned int)hi;
+    p.U1f = (float)hi;
+    p.ub = (float)lo * 2.3283064365386963e-10f;
+    return p;
+}
+__device__ inline CoarseTrial coarse_trial(double f, double aa, int e, bool own_fixed) {
+    CoarseTrial t;
+    int hi, lo;
+    split_balanced(__double2ll_rn(scale2(f, 38 + e)), &hi, &lo);
+    t.F1 = (unsigned int)hi;
+    t.F1f = (float)hi;
+    t.F0 = (float)lo * 2.3283064365386963e-10f;
+    split_balanced(-__double2ll_rn(scale2(aa, 38 + 2 * e)), &hi, &lo);
+    t.A1 = (unsigned int)hi;
+    t.A1f = (float)hi;
+    t.A0 = (float)lo * 2.3283064365386963e-10f;
+    unsigned int err = 75u + (aa != 0.0 ? 69u : 0u) + 3u;
+    if (own_fixed) {
+        // FIXED32's F1 and A1 are these over 16
+        const unsigned int f1 = (t.F1 >> 4) + 1u;
+        const unsigned int a1 = (unsigned int)((hi < 0 ? -hi : hi) >> 4) + 1u;
+        const int bits = 32 - __clz(f1);
+        const unsigned int k = bits > 22 ? (unsigned int)bits - 22u : 0u;
+        err += 5u + (5u << k);
+        if (f1 + a1 / 2u + (8u << k) >= (1u << (22u + k))) err += a1 / 4u + (1u << k);
+    }
+    t.margin = err + err / 4u + 8u;
+    t.pad = 0u;
+    return t;
+}
+// Whether the coarse fold serves a job (NaN: it does not).
+__device__ inline bool coarse_range_ok(const JobState *st) {
+    const double tau = __longlong_as_double((long long)st->tau_max_bits);
+    const double f = 1.0 / __longlong_as_double((long long)st->pmin_bits);
+    const double a = 0.5 * __longlong_as_double((long long)st->pdot_max_bits) * f * f;
+    return tau * f < 2097152.0 && a * tau * tau < 262144.0;
 }
 
 // ------------------------------------------------------------------ entropy
@@ -443,7 +554,7 @@ __host__ __device__ inline int slots_per_trial(int mode, int n_phase, int range)
 // Byte offsets of the CE kernel's dynamic shared-memory regions, in order: the
 // c ln c table (an even number of 8-byte entries, so the points after it stay
 // 16-byte aligned), the staged points (8 bytes each for FP64 and for half
-// points, else 16; chunk is a multiple of 32), the counters and the segment
+// points, else 16; the coarse fold's 12 and 24; chunk is a multiple of 32), the counters and the segment
 // starts.  The host sizes the launch with `total` and the kernel carves its
 // memory with the same offsets.  (k and block do not enter: each warp writes its
 // top-k keys and moments straight to global memory.)
@@ -454,7 +565,8 @@ __host__ __device__ inline MainSmemLayout main_smem_layout(int mode, int block, 
                                                            int n_phase, int n_mag,
                                                            int table_smem, int range, int half) {
     MainSmemLayout L;
-    const unsigned int pt = (mode == GCE_PHASE_FP64 || half) ? 8u : 16u;
+    const unsigned int pt = coarse_mode(mode) ? (half ? 12u : 24u)
+                            : (mode == GCE_PHASE_FP64 || half) ? 8u : 16u;
     L.pts = 8u * (unsigned int)((table_smem + 1) & ~1);
     L.cnt = L.pts + pt * (unsigned int)chunk;
     L.seg = L.cnt + 4u * (unsigned int)(tpt * slots_per_trial(mode, n_phase, range) * block);
@@ -481,7 +593,7 @@ struct PrepArgs {
     double t0;
     void *payload;             // ModeTraits<MODE>::point_t[sum N], sorted by mag bin per curve
     int *seg;                  // [n_curves][n_mag + 1] segment starts (relative to the curve)
-    double *tau;               // certified FP64 jobs: tau in payload order, else nullptr
+    double *tau;               // coarse modes: tau in payload order, else nullptr
     const JobState *state;
     const unsigned char *bands;  // multi-filter input: filter of each point, or nullptr
     const double2 *band_stats;   // [n_curves][n_bands] {median, standard deviation}
@@ -616,8 +728,10 @@ struct MainArgs {
     int half;
     int kv;                    // CE kernel variant (KV_*): overlapping bins or not
     int pdl;                   // host: launch with programmatic dependence
-    // FP64 jobs: every point's binary64 tau in payload order, and the caller's
-    // trial arrays (for the points the certified fold leaves to binary64)
+    // FP64 and FIXED32 jobs: every point's binary64 tau in payload order, and the
+    // caller's trial arrays (for the points the coarse fold leaves undecided);
+    // plain: payload and trials are in the mode's own format, with no tau
+    int plain;
     const double *tau;
     const double *periods;
     const double *pdots;
@@ -633,8 +747,24 @@ inline int kernel_variant(bool overlap) { return overlap ? KV_OVL : KV_SNAP; }
 // threads of a CTA with trials (and counters) of their own
 inline int trial_threads(int kv, int block) { return kv == KV_SHARED ? 32 : block; }
 
-// The CE kernel's fold for a job's phase mode: FP64 jobs run the certified one.
-inline int kernel_mode(int mode) { return mode == GCE_PHASE_FP64 ? (int)kFoldCertified : mode; }
+// The CE kernel's mode for a job's phase mode.
+inline int kernel_mode(int mode) {
+    return mode == GCE_PHASE_FP64 ? (int)kJobFp64 : mode == GCE_PHASE_FIXED32 ? (int)kJobFixed32 : mode;
+}
+// The preparation's mode: the kernel's, but FIXED32's own where the coarse fold gains
+// nothing over it: an undecided point makes its CTA some 8 us late (mostly fetching
+// code that is not cached), which small kernels and many bins feel more than the saved
+// multiplies (811 points x 50000 periods 70 us a call with FIXED32's own fold, 79 us
+// with the coarse one; 639 x 317 x 2358 periods at 31 bins 491 and 535 us; 1671 x
+// 119..952 x 3003 at 50 overlapping bins 2.34 and 2.43 ms; but 300 x 300..900 x 2e4 at
+// 15 bins 1.69 and 1.59 ms, 294 x 209..627 x 1222 x 131 Pdot at 50 17.3 and 16.7 ms).
+inline int job_prep_mode(const gce_config *cfg, long long n_trials, int n_pdots, int n_curves,
+                         int n_sm) {
+    const bool small = (n_trials + 31) / 32 * n_curves <= 400ll * n_sm;
+    const bool own = small || (n_pdots == 1 && cfg->n_phase_bins > 31);
+    return cfg->phase_mode == GCE_PHASE_FIXED32 && own ? (int)GCE_PHASE_FIXED32
+                                                       : kernel_mode(cfg->phase_mode);
+}
 // The launch shape of a job that was not tuned (gce_api.cu).
 int most_tpt(int mode);
 int split_range(int mode, int n_pdots, int slot_range);

@@ -55,6 +55,7 @@ struct FoldConst {
     float nphi_f;
     float zoff;          // SPLIT32: 1.5 2^23 + n_phase
     int n_phase;
+    unsigned int c0;     // coarse fold: kCoarseOffset and the thread's margin
 #if defined(GCE_CHECK_SLOTS)
     // checked builds: the trial's kept logical slots and where to flag a miss
     int zmin, zmax;
@@ -165,43 +166,17 @@ template <> struct Fold<GCE_PHASE_FIXED32> {
     __device__ __forceinline__ static bool k_zero(const prep_t &t) { return t.k == 0u; }
 };
 
-// FP64 jobs: a FIXED32 trial whose phases come out raised by an error margin (in
-// C; the largest of the thread's trials), so that one comparison bounds the
-// distance to the edges on both sides: with w = (phase + margin) n_phase, the bin
-// is hi32(w), and it is also the binary64 sequence's bin unless lo32(w) < 2 margin
-// n_phase.
-struct CertPrep : FixedPrep {};
-template <> struct Fold<kFoldCertified> {
-    typedef CertPrep prep_t;
+// Coarse jobs.  The margin (the largest of the thread's trials) is in FoldConst::c0.
+template <> struct Fold<kJobFp64> {
+    typedef CoarseTrial prep_t;
     static constexpr int kSlotBias = 0;
-    __device__ __forceinline__ static prep_t prepare(const FixedTrial &t) {
-        prep_t p;
-        static_cast<FixedPrep &>(p) = fixed_prep(t);
-        return p;
+    __device__ __forceinline__ static prep_t prepare(const CoarseTrial &t) { return t; }
+    __device__ __forceinline__ static bool has_pdot(const CoarseTrial &t) {
+        return t.A1 != 0u || t.A0 != 0.0f;
     }
-    __device__ __forceinline__ static unsigned int margin(const prep_t &p) {
-        return certified_margin(p.k, p.A1);
-    }
-    // a trial past the grid's end: every point in the middle of a bin
-    __device__ __forceinline__ static void park(prep_t &p, int n_phase) {
-        p.C += 0x80000000u / (unsigned int)n_phase;
-    }
-    // bin = hi32(w), lo = lo32(w): the two registers of one widening multiply (the
-    // product as a 64-bit C value cost two more instructions per point-trial, 14 %
-    // of the kernel's time at 256 threads x 2 trials)
-    template <bool PDOT, bool K0>
-    __device__ __forceinline__ static void bins(unsigned int fpart, uint4 p, const prep_t &t,
-                                                const FoldConst &k, unsigned int &bin,
-                                                unsigned int &lo) {
-        asm("{.reg .u64 w; mul.wide.u32 w, %2, %3; mov.b64 {%0, %1}, w;}"
-            : "=r"(lo), "=r"(bin)
-            : "r"(fold_fixed_phase_from<PDOT, K0>(fpart, p, t)), "r"((unsigned int)k.n_phase));
-    }
-    __device__ __forceinline__ static bool has_pdot(const FixedTrial &t) {
-        return (t.i.z | t.i.w) != 0u;
-    }
-    __device__ __forceinline__ static bool k_zero(const prep_t &t) { return t.k == 0u; }
+    __device__ __forceinline__ static bool k_zero(const prep_t &) { return true; }
 };
+template <> struct Fold<kJobFixed32> : Fold<kJobFp64> {};
 
 // The increment carries no memory clobber, so the compiler may schedule the
 // next points' shared loads around it; compiler_fence() before and after each
@@ -251,52 +226,184 @@ __device__ __forceinline__ void count_point(const typename ModeTraits<MODE>::poi
                        fk, inc);
 }
 
-// count_point of an FP64 job: the certified fold's bin, and near lowered to the
-// smallest lo32(w) seen (two trials per three-input minimum).
-template <int TPT, int SH, bool PDOT, bool K0, bool SHARED>
-__device__ __forceinline__ void count_point_cert(const uint4 &p, const CertPrep (&tc)[TPT],
-                                                 const unsigned int (&base)[TPT],
-                                                 const FoldConst &fk, unsigned int inc,
-                                                 unsigned int &near) {
-    unsigned int fp = 0u, lo[TPT];
-    if (SHARED) fp = fold_fixed_fpart(p, tc[0]);
-#pragma unroll
-    for (int s = 0; s < TPT; ++s) {
-        unsigned int bin;
-        Fold<kFoldCertified>::bins<PDOT, K0>(SHARED ? fp : fold_fixed_fpart(p, tc[s]), p, tc[s], fk,
-                                             bin, lo[s]);
-        bump<kFoldCertified, SH>(base[s], bin << SH, fk, inc);
+// Staged coarse points, in pairs: {T1, T1', T1f, T1f'}, then (from 8 chunk bytes on)
+// {b, b'}, or with a Pdot term {b, b', ub, ub'} and (from 16 chunk bytes on) {U1, U1',
+// U1f, U1f'}.
+struct CoarseSite {
+    const unsigned char *pts;
+    int chunk;
+};
+template <bool HALF>
+__device__ __forceinline__ void stage_coarse(unsigned int *s, int chunk, int k, const CoarsePoint &q) {
+    const int i = k >> 1, j = k & 1;
+    unsigned int *x = s + 4 * i + j, *y = s + 2 * chunk + (HALF ? 2 : 4) * i + j;
+    x[0] = q.T1;
+    x[2] = __float_as_uint(q.T1f);
+    y[0] = __float_as_uint(q.b);
+    if (!HALF) {
+        unsigned int *z = s + 4 * chunk + 4 * i + j;
+        y[2] = __float_as_uint(q.ub);
+        z[0] = q.U1;
+        z[2] = __float_as_uint(q.U1f);
     }
-    if (TPT == 1) near = min(near, lo[0]);
-#pragma unroll
-    for (int s = 0; s + 1 < TPT; s += 2) near = __vimin3_u32(near, lo[s], lo[s + 1]);
+}
+template <bool HALF, bool PDOT>
+__device__ __forceinline__ void staged_coarse(const CoarseSite &s, int pair, CoarsePoint (&p)[2]) {
+    const uint4 x = reinterpret_cast<const uint4 *>(s.pts)[pair];
+    p[0].T1 = x.x;
+    p[1].T1 = x.y;
+    p[0].T1f = __uint_as_float(x.z);
+    p[1].T1f = __uint_as_float(x.w);
+    if (HALF) {
+        const float2 y = reinterpret_cast<const float2 *>(s.pts + 8 * s.chunk)[pair];
+        p[0].b = y.x;
+        p[1].b = y.y;
+    } else {
+        const float4 y = reinterpret_cast<const float4 *>(s.pts + 8 * s.chunk)[pair];
+        p[0].b = y.x;
+        p[1].b = y.y;
+        p[0].ub = y.z;
+        p[1].ub = y.w;
+    }
+    if (PDOT) {
+        const uint4 z = reinterpret_cast<const uint4 *>(s.pts + 16 * s.chunk)[pair];
+        p[0].U1 = z.x;
+        p[1].U1 = z.y;
+        p[0].U1f = __uint_as_float(z.z);
+        p[1].U1f = __uint_as_float(z.w);
+    }
 }
 
-// The points of [ka, kb) of one trial that the certified fold may have put in the
-// wrong bin are decided by the binary64 sequence, and those that it did put there
-// are moved.  Rare (a point-trial comes here with probability 2 margin n_phase
-// 2^-32, about 3e-7 at 15 bins), so everything is read anew from global memory.
-template <int SH>
-__device__ __noinline__ void recount_near(const FixedTrial *tr, const double *tau, double period,
-                                          double pdot, const void *pts, bool half, int ka, int kb,
-                                          unsigned int base, unsigned int inc, unsigned int margin,
-                                          FoldConst fk) {
-    CertPrep t = Fold<kFoldCertified>::prepare(*tr);
-    t.C += margin;
-    const unsigned int thr = 2u * margin * (unsigned int)fk.n_phase;
-    const double f = 1.0 / period;
-    const double a = (0.5 * pdot) * f * f;
-    for (int k = ka; k < kb; ++k) {
-        typedef ModeTraits<kFoldCertified> MT;
-        const uint4 p = half ? MT::widen(static_cast<const uint2 *>(pts)[k])
-                             : static_cast<const uint4 *>(pts)[k];
-        unsigned int bin, lo;
-        Fold<kFoldCertified>::bins<true, false>(fold_fixed_fpart(p, t), p, t, fk, bin, lo);
-        if (lo >= thr) continue;
-        const unsigned int j = (unsigned int)fold_fp64<true>(tau[k], f, a, fk.nphi_d, fk.n_phase);
-        if (j == bin) continue;
-        bump<kFoldCertified, SH>(base, bin << SH, fk, 0u - inc);
-        bump<kFoldCertified, SH>(base, j << SH, fk, inc);
+// The period part of the coarse fold, and the rest of it: bin = hi32(w) and lo =
+// lo32(w), the two registers of one widening multiply (the product as a 64-bit C
+// value cost two more instructions per point-trial).
+__device__ __forceinline__ void coarse_fpart(const CoarsePoint &p, const CoarseTrial &t,
+                                             unsigned int c0, unsigned int &acc, float &z) {
+    acc = mad_lo_u32(p.T1, t.F1, c0);
+    z = __fmaf_rn(p.b, t.F1f, __fmaf_rn(p.T1f, t.F0, kCoarseRound));
+}
+template <bool PDOT>
+__device__ __forceinline__ void coarse_bins(unsigned int acc, float z, const CoarsePoint &p,
+                                            const CoarseTrial &t, const FoldConst &k,
+                                            unsigned int &bin, unsigned int &lo) {
+    if (PDOT) {
+        acc = mad_lo_u32(p.U1, t.A1, acc);
+        z = __fmaf_rn(p.ub, t.A1f, __fmaf_rn(p.U1f, t.A0, z));
+    }
+    asm("{.reg .u64 w; mul.wide.u32 w, %2, %3; mov.b64 {%0, %1}, w;}"
+        : "=r"(lo), "=r"(bin)
+        : "r"(acc + (__float_as_uint(z) << 6)), "r"((unsigned int)k.n_phase));
+}
+
+// Points [I, N) of a staged pair of a coarse job, counted as count_point does; near is
+// lowered to the smallest lo32(w) seen (two points per three-input minimum).
+template <int I, int N, int MODE, int TPT, int SH, bool PDOT, bool SHARED>
+__device__ __forceinline__ void count_coarse(const CoarsePoint (&p)[2], const CoarseTrial (&tc)[TPT],
+                                             const unsigned int (&base)[TPT], const FoldConst &fk,
+                                             unsigned int inc, unsigned int &near) {
+    unsigned int acc[2] = {0u, 0u};
+    float z[2] = {0.0f, 0.0f};
+    if (SHARED)
+#pragma unroll
+        for (int i = I; i < N; ++i) coarse_fpart(p[i], tc[0], fk.c0, acc[i], z[i]);
+#pragma unroll
+    for (int s = 0; s < TPT; ++s) {
+        unsigned int lo[2] = {0xffffffffu, 0xffffffffu};
+#pragma unroll
+        for (int i = I; i < N; ++i) {
+            unsigned int bin;
+            if (!SHARED) coarse_fpart(p[i], tc[s], fk.c0, acc[i], z[i]);
+            coarse_bins<PDOT>(acc[i], z[i], p[i], tc[s], fk, bin, lo[i]);
+            bump<MODE, SH>(base[s], bin << SH, fk, inc);
+        }
+        near = N - I == 2 ? __vimin3_u32(near, lo[0], lo[1]) : min(near, lo[I]);
+    }
+}
+
+// The mode's own phase bin of point k (payload order) in flat trial t.
+template <int MODE>
+__device__ __forceinline__ unsigned int own_bin(const MainArgs &a, long long k, long long t,
+                                                const FoldConst &fk) {
+    const long long q = t / a.n_periods;
+    const double f = 1.0 / a.periods[t - q * a.n_periods];
+    const double aa = (0.5 * a.pdots[q]) * f * f;
+    const double tau = a.tau[k];
+    // t = t0: phase 0 in both folds (FIXED32's rounds to it exactly without Pdot)
+    if (tau == 0.0 && (MODE == kJobFp64 || aa == 0.0)) return 0u;
+    if (MODE == kJobFp64) return (unsigned int)fold_fp64<true>(tau, f, aa, fk.nphi_d, fk.n_phase);
+    const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
+    return (unsigned int)fold_fixed<true>(fixed_point(tau, fs), fixed_prep(fixed_trial(f, aa, fs)),
+                                          (unsigned int)fk.n_phase);
+}
+
+// What a run of points needs to have its undecided points decided: where the blocks
+// of per pairs that the mask's bits 1, 2, ... stand for begin and end (bit 31: the
+// 31st block and all after it; bit 0: the points of [ka, kb) before and after them).
+struct Undecided {
+    unsigned int mask;
+    int first, blocks, per;
+};
+
+// The undecided points of one trial per lane go where the mode's own fold puts them.
+// Called by the whole warp: lane after lane, all lanes test the points of that lane's
+// blocks with its trial (and the one that finds an undecided point decides it).  Rare
+// (a point-trial is undecided with probability 2 margin n_phase 2^-32, 8e-7 at 15
+// bins), but what matters is its latency, which the CTA's other warps wait for at
+// their next barrier: with each lane walking its own blocks it took 33 us and 12 % of
+// the kernel.
+template <int MODE, int SH>
+__device__ __noinline__ void settle(const MainArgs &a, Undecided u, CoarseTrial tr, long long t,
+                                    long long pt0, CoarseSite site, bool half, int ka, int kb,
+                                    unsigned int base, unsigned int inc, unsigned int thr, FoldConst fk) {
+    const int lane = threadIdx.x & 31;
+    if (t >= a.n_trials) u.mask = 0u;
+    for (unsigned int lanes = __ballot_sync(0xffffffffu, u.mask != 0u); lanes; lanes &= lanes - 1u) {
+        const int l = __ffs((int)lanes) - 1;
+        CoarseTrial x;
+        x.F1 = __shfl_sync(0xffffffffu, tr.F1, l);
+        x.F0 = __shfl_sync(0xffffffffu, tr.F0, l);
+        x.F1f = __shfl_sync(0xffffffffu, tr.F1f, l);
+        x.A1 = __shfl_sync(0xffffffffu, tr.A1, l);
+        x.A0 = __shfl_sync(0xffffffffu, tr.A0, l);
+        x.A1f = __shfl_sync(0xffffffffu, tr.A1f, l);
+        const long long xt = __shfl_sync(0xffffffffu, t, l);
+        const unsigned int xbase = __shfl_sync(0xffffffffu, base, l);
+        const unsigned int xthr = __shfl_sync(0xffffffffu, thr, l);
+        FoldConst xk = fk;
+        xk.c0 = __shfl_sync(0xffffffffu, fk.c0, l);
+        auto range = [&](int from, int to) {
+            for (int k = from + lane; k < to; k += 32) {
+                CoarsePoint p[2];
+                if (half) {
+                    staged_coarse<true, false>(site, k >> 1, p);
+                    p[0].U1 = p[1].U1 = 0u;
+                    p[0].U1f = p[1].U1f = p[0].ub = p[1].ub = 0.0f;
+                } else {
+                    staged_coarse<false, true>(site, k >> 1, p);
+                }
+                const CoarsePoint q = (k & 1) ? p[1] : p[0];
+                unsigned int acc, bin, lo;
+                float z;
+                coarse_fpart(q, x, xk.c0, acc, z);
+                coarse_bins<true>(acc, z, q, x, xk, bin, lo);
+                if (lo >= xthr) continue;
+                const unsigned int j = own_bin<MODE>(a, pt0 + k, xt, xk);
+                if (j == bin) continue;
+                bump<MODE, SH>(xbase, bin << SH, xk, 0u - inc);
+                bump<MODE, SH>(xbase, j << SH, xk, inc);
+            }
+        };
+        for (unsigned int m = __shfl_sync(0xffffffffu, u.mask, l); m; m &= m - 1u) {
+            const int i = __ffs((int)m) - 1;
+            if (i == 0) {
+                range(ka, min(kb, 2 * u.first));
+                range(max(ka, 2 * (u.first + u.blocks * u.per)), kb);
+            } else {
+                const int last = i == 31 ? u.blocks : i;
+                range(2 * (u.first + (i - 1) * u.per), 2 * (u.first + last * u.per));
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -371,20 +478,54 @@ template <int MODE, int TPT, int SH, bool PDOT, bool K0, bool RED, bool SHARED, 
 __device__ __forceinline__ void count_points(
     const void *__restrict__ pts, int ka, int kb,
     const typename Fold<MODE>::prep_t (&tc)[TPT], const unsigned int (&base)[TPT],
-    const FoldConst &fk, unsigned int inc, unsigned int &near) {
+    const FoldConst &fk, unsigned int inc, int chunk, unsigned int thr, Undecided &und) {
     typedef ModeTraits<MODE> MT;
     static_assert(!(HALF && PDOT), "half points carry no tau^2");
     // points unrolled by 16 (8 with the longer Pdot fold): measured faster than 8
     // and 4 on every workload without a Pdot axis, and than 16 with one
     constexpr int UNROLL = PDOT ? 8 : 16;
-    constexpr bool PAIRS = HALF && (MODE == GCE_PHASE_FIXED32 || MODE == kFoldCertified);
-    auto one = [&](const typename MT::point_t &p) {
-        if constexpr (MODE == kFoldCertified)
-            count_point_cert<TPT, SH, PDOT, K0, SHARED>(p, tc, base, fk, inc, near);
-        else
+    constexpr bool PAIRS = HALF && MODE == GCE_PHASE_FIXED32;
+    [[maybe_unused]] auto one = [&](const typename MT::point_t &p) {
+        if constexpr (!coarse_mode(MODE))
             count_point<MODE, TPT, SH, PDOT, K0, RED, SHARED>(p, tc, base, fk, inc);
     };
-    if constexpr (MODE == GCE_PHASE_SPLIT32) {
+    if constexpr (coarse_mode(MODE)) {
+        constexpr int U = UNROLL / 2;
+        const CoarseSite site{static_cast<const unsigned char *>(pts), chunk};
+        CoarsePoint p[2];
+        unsigned int edge = 0xffffffffu;  // smallest lo32(w) outside the blocks
+        int q = ka >> 1;
+        if ((ka & 1) && ka < kb) {
+            staged_coarse<HALF, PDOT>(site, q, p);
+            count_coarse<1, 2, MODE, TPT, SH, PDOT, SHARED>(p, tc, base, fk, inc, edge);
+            ++q;
+        }
+        und.first = q;
+        und.per = U;
+        und.mask = 0u;
+        unsigned int bit = 2u;
+        for (; 2 * (q + U) <= kb; q += U) {
+            unsigned int near = 0xffffffffu;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                staged_coarse<HALF, PDOT>(site, q + u, p);
+                count_coarse<0, 2, MODE, TPT, SH, PDOT, SHARED>(p, tc, base, fk, inc, near);
+            }
+            if (near < thr) und.mask |= bit;
+            bit = bit < 0x80000000u ? bit << 1 : bit;
+        }
+        und.blocks = (q - und.first) / U;
+#pragma unroll 1
+        for (; 2 * q + 1 < kb; ++q) {
+            staged_coarse<HALF, PDOT>(site, q, p);
+            count_coarse<0, 2, MODE, TPT, SH, PDOT, SHARED>(p, tc, base, fk, inc, edge);
+        }
+        if (2 * q < kb) {
+            staged_coarse<HALF, PDOT>(site, q, p);
+            count_coarse<0, 1, MODE, TPT, SH, PDOT, SHARED>(p, tc, base, fk, inc, edge);
+        }
+        if (edge < thr) und.mask |= 1u;
+    } else if constexpr (MODE == GCE_PHASE_SPLIT32) {
         int k = ka;
         if ((k & 1) && k < kb) {
             one(staged_point<HALF>(pts, k));
@@ -430,10 +571,10 @@ template <int MODE, int TPT, int SH, bool PDOT, bool K0, bool RED = false, bool 
 __device__ __forceinline__ void count_points_any(
     bool shared, const void *__restrict__ pts, int ka, int kb,
     const typename Fold<MODE>::prep_t (&tc)[TPT], const unsigned int (&base)[TPT],
-    const FoldConst &fk, unsigned int inc, unsigned int &near) {
+    const FoldConst &fk, unsigned int inc, int chunk, unsigned int thr, Undecided &und) {
     constexpr bool SH_OK = PDOT && TPT > 1;  // sharing pays only with a Pdot term
-    if (SH_OK && shared) count_points<MODE, TPT, SH, PDOT, K0, RED, SH_OK, HALF>(pts, ka, kb, tc, base, fk, inc, near);
-    else count_points<MODE, TPT, SH, PDOT, K0, RED, false, HALF>(pts, ka, kb, tc, base, fk, inc, near);
+    if (SH_OK && shared) count_points<MODE, TPT, SH, PDOT, K0, RED, SH_OK, HALF>(pts, ka, kb, tc, base, fk, inc, chunk, thr, und);
+    else count_points<MODE, TPT, SH, PDOT, K0, RED, false, HALF>(pts, ka, kb, tc, base, fk, inc, chunk, thr, und);
 }
 
 // c_ij of one phase bin at the end of a magnitude segment (low - snapshot), with
@@ -780,7 +921,7 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     const int tw = SHARED_SET ? 0 : warp;
     const int n_phase = a.n_phase, n_mag = a.n_mag;
     constexpr bool SPLIT = MODE == GCE_PHASE_SPLIT32;
-    constexpr bool CERT = MODE == kFoldCertified;
+    constexpr bool COARSE = coarse_mode(MODE);
     constexpr int ovl = OVL ? 1 : 0;  // 50 %-overlapping phase bins
     const int range = SPLIT ? a.range : (int)RANGE_WIDE;
     const SlotRange zr = slot_range(MODE, n_phase, range);
@@ -790,8 +931,8 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
 
     // the regions at the offsets the host sized the launch with (the table first,
     // so that its address is a constant)
-    const MainSmemLayout lay = main_smem_layout(LAYMODE, TB, TPT, a.chunk, n_phase, n_mag, a.table_smem,
-                                                range, a.half);
+    const MainSmemLayout lay = main_smem_layout(a.plain ? MODE : LAYMODE, TB, TPT, a.chunk, n_phase, n_mag, a.table_smem,
+                                                a.range, a.half);
     unsigned long long *s_tab = reinterpret_cast<unsigned long long *>(smem);
     point_t *s_pts = reinterpret_cast<point_t *>(smem + lay.pts);
     unsigned int *s_cnt = reinterpret_cast<unsigned int *>(smem + lay.cnt);
@@ -799,8 +940,9 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
 
     for (int i = tid; i < a.table_smem; i += B) s_tab[i] = a.table[i];
 
-    // (the binary64 fold of an FP64 job beyond the certified range reads tau)
-    const point_t *g_pts = reinterpret_cast<const point_t *>(MODE == LAYMODE ? a.payload : a.tau);
+    // (an FP64 job beyond the coarse fold's range has its points in tau)
+    const point_t *g_pts = reinterpret_cast<const point_t *>(
+        MODE == GCE_PHASE_FP64 && !a.plain ? (const void *)a.tau : a.payload);
     const trial_t *g_tr = reinterpret_cast<const trial_t *>(a.trialc);
     unsigned int *my_cnt = s_cnt + tb;
     // counters start at zero; every work item's final sweep clears the words it
@@ -812,7 +954,7 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     fk.zmax = zr.zmax;
     fk.err = &a.state->err;
 #else
-    const FoldConst fk = fold_const(n_phase);
+    FoldConst fk = fold_const(n_phase);
 #endif
     unsigned int base[TPT];
     unsigned int *wbase[TPT];  // physical slot 0 of trial s
@@ -826,7 +968,7 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     // single Pdot value is not 0 stages whole points, half as many per chunk
     const bool job_pdot = a.state->pdot_max_bits != 0ull;
     const bool half = a.half != 0 && !job_pdot;
-    const int chunk_pts = (a.half != 0 && job_pdot) ? (a.chunk >> 1) : a.chunk;
+    const int chunk_pts = (a.half != 0 && job_pdot) ? (a.chunk >> 1) & ~1 : a.chunk;
     // max |tau| of the job (SPLIT32 slot windows), rounded up to FP32
     const float tau_max_f =
         SPLIT ? __double2float_ru(__longlong_as_double((long long)a.state->tau_max_bits)) : 0.0f;
@@ -838,7 +980,7 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     typename Fold<MODE>::prep_t tc[TPT];
     long long tt[TPT];
     bool pdot = false, k0 = true;
-    unsigned int margin = 0u;  // FP64: the certified fold's margin (0: no trial in the grid)
+    unsigned int margin = 0u;  // coarse fold: the thread's margin
     bool red = false;  // SPLIT32: this warp's folds re-reduce the residual (narrow window)
     const bool pdm = a.pd_major != 0;
     int wl[TPT];           // word offset (from my_cnt) of each trial's first window slot
@@ -901,32 +1043,24 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                 else
                     tt[s] = flat_list_trial(((long long)tile * (TB / 32) + tw) * (TPT / 2) + s / 2) +
                             (s % 2) * 256 + lane;
-                trial_t tr{};
-                if (tt[s] < a.n_trials) {
-                    tr = g_tr[tt[s]];
-                    any_pdot |= Fold<MODE>::has_pdot(tr);
-                }
+                // (past the grid's end the last trial once more, without output)
+                const trial_t tr = g_tr[min(tt[s], a.n_trials - 1)];
+                any_pdot |= Fold<MODE>::has_pdot(tr);
                 tc[s] = Fold<MODE>::prepare(tr);
-                if constexpr (CERT) {
-                    if (tt[s] < a.n_trials) margin = max(margin, Fold<MODE>::margin(tc[s]));
-                    else Fold<MODE>::park(tc[s], n_phase);
-                }
+                if constexpr (COARSE) margin = max(margin, tr.margin);
                 all_k0 &= Fold<MODE>::k_zero(tc[s]);
             }
-            if constexpr (CERT) {
-#pragma unroll
-                for (int s = 0; s < TPT; ++s) tc[s].C += margin;
-            }
+            if constexpr (COARSE) fk.c0 = kCoarseOffset + margin;
             // the fold variant is chosen per warp (a warp vote, no CTA barrier)
             pdot = __any_sync(0xffffffffu, any_pdot);
-            k0 = (MODE != GCE_PHASE_FIXED32 && !CERT) || __all_sync(0xffffffffu, all_k0);
+            k0 = MODE != GCE_PHASE_FIXED32 || __all_sync(0xffffffffu, all_k0);
             // live logical slots [L, R] of this warp's counters (warp-uniform)
             int L = 0, R = n_phase - 1;
             if (SPLIT) {
                 float fm = 0.0f;
 #pragma unroll
                 for (int s = 0; s < TPT; ++s)
-                    if (tt[s] < a.n_trials) fm = fmaxf(fm, fabsf(split_fh(tc[s])));
+                    fm = fmaxf(fm, fabsf(split_fh(tc[s])));
                 fm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fm)));
                 // folds without a Pdot term re-reduce their residual with the
                 // narrow range, and with the mid one where the warp's cycles
@@ -980,6 +1114,12 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                         for (int k = tid; k < hi - lo; k += B) stage_split<true>(sp, k, src[k]);
                     else
                         for (int k = tid; k < hi - lo; k += B) stage_split<false>(sp, k, src[k]);
+                } else if constexpr (COARSE) {
+                    unsigned int *sp = reinterpret_cast<unsigned int *>(s_pts);
+                    if (half)
+                        for (int k = tid; k < hi - lo; k += B) stage_coarse<true>(sp, chunk_pts, k, src[k]);
+                    else
+                        for (int k = tid; k < hi - lo; k += B) stage_coarse<false>(sp, chunk_pts, k, src[k]);
                 } else if (half) {
                     typedef typename ModeTraits<MODE>::half_t half_t;
                     half_t *s_half = reinterpret_cast<half_t *>(s_pts);
@@ -1006,34 +1146,32 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                     const unsigned int inc = pk2 ? ((ended & 1) ? kPk2IncB : 1u) + kPk2IncC : 1u;
                     compiler_fence();
                     const void *pp = s_pts;
-                    unsigned int near = 0xffffffffu;
+                    Undecided und{};
+                    const unsigned int thr = 2u * margin * (unsigned int)n_phase;
                     constexpr bool HP = MODE != GCE_PHASE_FP64;  // half points exist
                     if (k0) {
-                        if (pdot) count_points_any<MODE, TPT, SH, true, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                        if (pdot) count_points_any<MODE, TPT, SH, true, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
                         // (red: the warp's slot window is the narrow one, so its folds
                         // must re-reduce, with half points as with whole ones)
-                        else if (SPLIT && red && half) count_points_any<MODE, TPT, SH, false, true, SPLIT, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
-                        else if (SPLIT && red) count_points_any<MODE, TPT, SH, false, true, SPLIT>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
-                        else if (HP && half) count_points_any<MODE, TPT, SH, false, true, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
-                        else count_points_any<MODE, TPT, SH, false, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
-                    } else if (MODE == GCE_PHASE_FIXED32 || CERT) {
-                        if (pdot) count_points_any<MODE, TPT, SH, true, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
-                        else if (half) count_points_any<MODE, TPT, SH, false, false, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
-                        else count_points_any<MODE, TPT, SH, false, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, near);
+                        else if (SPLIT && red && half) count_points_any<MODE, TPT, SH, false, true, SPLIT, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
+                        else if (SPLIT && red) count_points_any<MODE, TPT, SH, false, true, SPLIT>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
+                        else if (HP && half) count_points_any<MODE, TPT, SH, false, true, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
+                        else count_points_any<MODE, TPT, SH, false, true>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
+                    } else if (MODE == GCE_PHASE_FIXED32) {
+                        if (pdot) count_points_any<MODE, TPT, SH, true, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
+                        else if (half) count_points_any<MODE, TPT, SH, false, false, false, HP>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
+                        else count_points_any<MODE, TPT, SH, false, false>(pdm, pp, ka - lo, kb - lo, tc, base, fk, inc, chunk_pts, thr, und);
                     }
                     compiler_fence();
-                    if constexpr (CERT) {
-                        if (near < 2u * margin * (unsigned int)n_phase) {
+                    if constexpr (COARSE) {
+                        if (__any_sync(0xffffffffu, und.mask != 0u)) {
                             // undecided points in this run: decide them before the
                             // counts are read
 #pragma unroll
-                            for (int s = 0; s < TPT; ++s) {
-                                if (tt[s] >= a.n_trials) continue;
-                                const long long q = tt[s] / a.n_periods;
-                                recount_near<SH>(reinterpret_cast<const FixedTrial *>(a.trialc) + tt[s],
-                                                 a.tau + off + lo, a.periods[tt[s] - q * a.n_periods],
-                                                 a.pdots[q], pp, half, ka - lo, kb - lo, base[s], inc, margin, fk);
-                            }
+                            for (int s = 0; s < TPT; ++s)
+                                settle<MODE, SH>(a, und, tc[s], tt[s], off + lo,
+                                                 CoarseSite{reinterpret_cast<const unsigned char *>(s_pts), chunk_pts},
+                                                 half, ka - lo, kb - lo, base[s], inc, thr, fk);
                             compiler_fence();
                         }
                     }
@@ -1146,22 +1284,24 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     }
 }
 
-// The CE kernel.  An FP64 job runs the certified fold (MODE kFoldCertified), or,
-// where its range is beyond that fold or the host laid it out for binary64 alone
-// (no payload), the binary64 fold on every point.  Binary64 arithmetic runs at 2
-// lanes per clock and SM and bounds that fold: 19.4 ms on 100 curves x 1000 points
-// x 2e4 periods, 22.5 ms on 23 x 487 x 1e4 x 16 Pdot.  The certified fold, bound
-// like FIXED32 by the integer multiplies of the FMA-heavy pipe and by latency,
-// takes 1.13 and 1.33 ms for the same counts.
+// The CE kernel.  FP64 and FIXED32 jobs run the coarse fold, or, where the job's range
+// is beyond it or the host laid it out plain, the mode's own fold on every point.
+// Binary64 arithmetic runs at 2 lanes per clock and SM and bounds the FP64 fold (100
+// curves x 1000 points x 2e4 periods 19.4 ms, 23 x 487 x 1e4 x 16 Pdot 22.5 ms); the
+// high-half integer multiplies of the FMA-heavy pipe bound FIXED32's, two per
+// point-trial (three with Pdot; 300 curves x 300..900 points x 2e4 periods 1.54 ms, 20
+// x 200..1000 x 5e4 x 16 Pdot 4.49 ms).  The coarse fold has one: 0.85, 1.03, 1.44 and
+// 4.09 ms, of which keeping the distance to the edges takes a tenth.  Bound by issue
+// (nine instructions per point-trial) and latency at 16 to 24 warps per SM.
 template <int MODE, int TPT, int LOG2B, int KV>
-__global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k_main(MainArgs a) {
+__global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k_main(const __grid_constant__ MainArgs a) {
     __shared__ long long s_item;
     pdl_trigger();
     pdl_wait();
     if (a.state->err) return;  // inputs failed the device checks: no work
-    if constexpr (MODE == kFoldCertified) {
-        if (a.payload == nullptr || a.state->wide) {
-            ce_items<GCE_PHASE_FP64, MODE, TPT, LOG2B, KV>(a, s_item);
+    if constexpr (coarse_mode(MODE)) {
+        if (a.plain || a.state->wide) {
+            ce_items<MODE == kJobFp64 ? GCE_PHASE_FP64 : GCE_PHASE_FIXED32, MODE, TPT, LOG2B, KV>(a, s_item);
             return;
         }
     }

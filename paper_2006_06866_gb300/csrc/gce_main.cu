@@ -152,14 +152,14 @@ size_t single_smem_bytes(int n_phase, int block) { return 4 * (size_t)n_phase * 
 
 const void *main_kernel_ptr(int mode, int tpt, int block, int kv) {
     switch (mode * 8 + tpt) {
-        case kFoldCertified * 8 + 1: return main_kernel_ptr_fp64_t1(block, kv);
-        case kFoldCertified * 8 + 2: return main_kernel_ptr_fp64_t2(block, kv);
+        case kJobFp64 * 8 + 1: return main_kernel_ptr_fp64_t1(block, kv);
+        case kJobFp64 * 8 + 2: return main_kernel_ptr_fp64_t2(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 1: return main_kernel_ptr_split32_t1(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 2: return main_kernel_ptr_split32_t2(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 4: return main_kernel_ptr_split32_t4(block, kv);
-        case GCE_PHASE_FIXED32 * 8 + 1: return main_kernel_ptr_fixed32_t1(block, kv);
-        case GCE_PHASE_FIXED32 * 8 + 2: return main_kernel_ptr_fixed32_t2(block, kv);
-        case GCE_PHASE_FIXED32 * 8 + 4: return main_kernel_ptr_fixed32_t4(block, kv);
+        case kJobFixed32 * 8 + 1: return main_kernel_ptr_fixed32_t1(block, kv);
+        case kJobFixed32 * 8 + 2: return main_kernel_ptr_fixed32_t2(block, kv);
+        case kJobFixed32 * 8 + 4: return main_kernel_ptr_fixed32_t4(block, kv);
         default: return nullptr;
     }
 }
@@ -190,14 +190,14 @@ cudaError_t main_kernel_attrs(int mode, int tpt, int block, int kv, size_t smem_
 cudaError_t launch_main(int mode, int tpt, int block, int grid, size_t smem, const MainArgs &a,
                         cudaStream_t s) {
     switch (mode * 8 + tpt) {
-        case kFoldCertified * 8 + 1: return launch_main_fp64_t1(block, grid, smem, a, s);
-        case kFoldCertified * 8 + 2: return launch_main_fp64_t2(block, grid, smem, a, s);
+        case kJobFp64 * 8 + 1: return launch_main_fp64_t1(block, grid, smem, a, s);
+        case kJobFp64 * 8 + 2: return launch_main_fp64_t2(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 1: return launch_main_split32_t1(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 2: return launch_main_split32_t2(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 4: return launch_main_split32_t4(block, grid, smem, a, s);
-        case GCE_PHASE_FIXED32 * 8 + 1: return launch_main_fixed32_t1(block, grid, smem, a, s);
-        case GCE_PHASE_FIXED32 * 8 + 2: return launch_main_fixed32_t2(block, grid, smem, a, s);
-        case GCE_PHASE_FIXED32 * 8 + 4: return launch_main_fixed32_t4(block, grid, smem, a, s);
+        case kJobFixed32 * 8 + 1: return launch_main_fixed32_t1(block, grid, smem, a, s);
+        case kJobFixed32 * 8 + 2: return launch_main_fixed32_t2(block, grid, smem, a, s);
+        case kJobFixed32 * 8 + 4: return launch_main_fixed32_t4(block, grid, smem, a, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,4 +1,4 @@
-// Instantiations of the CE kernel for FP64 jobs (the certified fold and the binary64 one) with 2 trials per
+// Instantiations of the CE kernel for FP64 jobs with 2 trials per
 // thread (one translation unit per fold mode and trials per thread, so that
 // they compile in parallel).
 #include "gce_kernel.cuh"
@@ -6,12 +6,12 @@
 namespace gce {
 
 const void *main_kernel_ptr_fp64_t2(int block, int kv) {
-    return kernel_for_variant<kFoldCertified, 2>(block, kv);
+    return kernel_for_variant<kJobFp64, 2>(block, kv);
 }
 
 cudaError_t launch_main_fp64_t2(int block, int grid, size_t smem, const MainArgs &a,
                                   cudaStream_t s) {
-    return launch_for_block<kFoldCertified, 2>(block, grid, smem, a, s);
+    return launch_for_block<kJobFp64, 2>(block, grid, smem, a, s);
 }
 
 }  // namespace gce

@@ -107,32 +107,17 @@ __global__ void k_scan(const double *__restrict__ times, const double *__restric
     }
 }
 
-// Whether an FP64 job is beyond the certified fold's range (from the job's
-// maxima, so every thread that asks agrees).
-__device__ inline bool beyond_certified(const JobState *st, int e_tau) {
-    const double pmin = __longlong_as_double((long long)st->pmin_bits);
-    const double dmax = __longlong_as_double((long long)st->pdot_max_bits);
-    const double fmax_ = 1.0 / pmin;
-    return !fixed_range_ok(fmax_, 0.5 * dmax * fmax_ * fmax_, e_tau);
-}
-
-// x 2^e as ldexp rounds it: one multiplication where 2^e is a normal number.
-__device__ __forceinline__ double scale2(double x, int e) {
-    if (e < -1022 || e > 1023) return ldexp(x, e);
-    return __dmul_rn(x, __longlong_as_double((long long)(e + 1023) << 52));
-}
-
 // Per flat trial t = q n_periods + p: f = 1/P, a = (0.5 Pdot) f f (the oracle's
 // sequence), stored in the fold mode's format.
 template <int MODE>
 __global__ void k_trials(TrialArgs a) {
-    typedef typename ModeTraits<MODE>::trial_t trial_t;
     pdl_trigger();
     pdl_wait();
-    trial_t *out = reinterpret_cast<trial_t *>(a.trialc);
     const long long n = (long long)a.n_periods * a.n_pdots;
     const double tau_max = __longlong_as_double((long long)a.state->tau_max_bits);
     const FixedScale fs = fixed_scale_from(tau_max);
+    // (of a coarse job: every thread that asks agrees, the maxima being final)
+    const bool wide = coarse_mode(MODE) && !coarse_range_ok(a.state);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         // Range of the fold (checked once, from the maxima).
         const double pmin = __longlong_as_double((long long)a.state->pmin_bits);
@@ -144,57 +129,34 @@ __global__ void k_trials(TrialArgs a) {
             if (MODE == GCE_PHASE_SPLIT32) {
                 // |x| < 1 needs |c| + |c2| < 1/2: cycles < 2^21 and Pdot cycles < 2^19
                 bad = tau_max * fmax_ >= 2097152.0 || amax * tau_max * tau_max >= 524288.0;
-            } else if (MODE == GCE_PHASE_FIXED32) {
+            } else if (MODE == GCE_PHASE_FIXED32 || MODE == kJobFixed32) {
                 bad = !fixed_range_ok(fmax_, amax, fs.e_tau);
             }
             if (bad) atomicOr(&a.state->err, ERR_RANGE);
         }
-        if (MODE == kFoldCertified) a.state->wide = beyond_certified(a.state, fs.e_tau) ? 1u : 0u;
+        if (coarse_mode(MODE)) a.state->wide = wide ? 1u : 0u;
     }
-    const bool wide = MODE == kFoldCertified && beyond_certified(a.state, fs.e_tau);
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (long long)gridDim.x * blockDim.x) {
         const int p = (int)(t % a.n_periods);
         const int q = (int)(t / a.n_periods);
         const double f = 1.0 / a.periods[p];
         const double aa = (0.5 * a.pdots[q]) * f * f;
-        if (MODE == kFoldCertified && wide) {  // {f, a}, read by the binary64 fold
+        if (MODE == GCE_PHASE_FP64 || (MODE == kJobFp64 && wide)) {
             reinterpret_cast<double2 *>(a.trialc)[t] = make_double2(f, aa);
-            continue;
-        }
-        trial_t v;
-        if constexpr (MODE == GCE_PHASE_FP64) {
-            v.x = f;
-            v.y = aa;
-        } else if constexpr (MODE == GCE_PHASE_SPLIT32) {
-            // f split, and -a split (the fold adds -a tau^2)
-            float fh = __double2float_rn(f);
-            float nah = __double2float_rn(-aa);
-            v.x = fh;
-            v.y = __double2float_rn(f - (double)fh);
-            v.z = nah;
-            v.w = __double2float_rn(-aa - (double)nah);
+        } else if (MODE == GCE_PHASE_FIXED32 || (MODE == kJobFixed32 && wide)) {
+            reinterpret_cast<FixedTrial *>(a.trialc)[t] = fixed_trial(f, aa, fs);
+        } else if (coarse_mode(MODE)) {
+            reinterpret_cast<CoarseTrial *>(a.trialc)[t] =
+                coarse_trial(f, aa, fs.e_tau, MODE == kJobFixed32);
         } else {
-            // Out-of-range values are flagged above; clamp so the conversions stay defined.
-            const double F = fmin(scale2(f, fs.r), 9.2e18);
-            const double A = fmax(fmin(scale2(aa, fs.v), 9.2e18), -9.2e18);
-            int f1, f0;
-            split_balanced(__double2ll_rn(F), &f1, &f0);
-            const long long an = -__double2ll_rn(A);
-            const int a1 = (int)(an >> 32);
-            const unsigned int a0 = (unsigned int)(an & 0xffffffffll);
-            // k: the smallest shift with F1 < 2^(22+k)
-            const unsigned int uf1 = (unsigned int)f1;
-            const int bits = 32 - __clz(uf1);
-            const int k = bits > 22 ? bits - 22 : 0;
-            const float g0 = __double2float_rn(scale2((double)uf1, -23 - k));
-            const float g2 = __double2float_rn(scale2((double)a1, -23 - k));
-            const double kk = 12582912.0 - 8388608.0 * (double)g0 - 8388608.0 * (double)g2 -
-                              scale2((double)a1, -1 - k);
-            v.i = make_uint4(uf1, (unsigned int)f0, (unsigned int)a1, a0);
-            v.f = make_float4(g0, g2, __double2float_rn(kk), __uint_as_float((unsigned int)k));
+            // f split, and -a split (the fold adds -a tau^2)
+            const float fh = __double2float_rn(f);
+            const float nah = __double2float_rn(-aa);
+            reinterpret_cast<float4 *>(a.trialc)[t] =
+                make_float4(fh, __double2float_rn(f - (double)fh), nah,
+                            __double2float_rn(-aa - (double)nah));
         }
-        out[t] = v;
     }
 }
 
@@ -463,7 +425,6 @@ struct MagView {
 // a segment is arbitrary; counts do not depend on it.
 template <int MODE>
 __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
-    typedef typename ModeTraits<MODE>::point_t point_t;
     __shared__ unsigned long long sh_min[kPrepBlock / 32], sh_max[kPrepBlock / 32];
     __shared__ int hist[GCE_MAX_MAG_BINS + 1];
     // the first points' magnitudes and bins, each computed once (binary64 arithmetic
@@ -519,39 +480,26 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
     }
     __syncthreads();
     const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
-    point_t *out = reinterpret_cast<point_t *>(a.payload) + lo;
+    const bool wide = coarse_mode(MODE) && !coarse_range_ok(a.state);
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         const int b = k < kPrepBins ? s_bin[k] : bins(k < kPrepMags ? s_m[k] : m[k]);
         const int pos = atomicAdd(&hist[b], 1);
         const double tau = __dsub_rn(t[k], a.t0);
-        point_t v;
-        if constexpr (MODE == GCE_PHASE_FP64) {
-            v = tau;
-        } else if constexpr (MODE == GCE_PHASE_SPLIT32) {
-            const double tau2 = __dmul_rn(tau, tau);
-            float th = __double2float_rn(tau);
-            float t2h = __double2float_rn(tau2);
-            v.x = th;
-            v.y = __double2float_rn(tau - (double)th);
-            v.z = t2h;
-            v.w = __double2float_rn(tau2 - (double)t2h);
+        if (coarse_mode(MODE)) a.tau[lo + pos] = tau;
+        if (MODE == GCE_PHASE_FP64) {
+            reinterpret_cast<double *>(a.payload)[lo + pos] = tau;
+        } else if (MODE == GCE_PHASE_FIXED32 || (MODE == kJobFixed32 && wide)) {
+            reinterpret_cast<uint4 *>(a.payload)[lo + pos] = fixed_point(tau, fs);
+        } else if (coarse_mode(MODE)) {
+            reinterpret_cast<CoarsePoint *>(a.payload)[lo + pos] = coarse_point(tau, fs.e_tau);
         } else {
-            // T = round(tau 2^s), |T| < 2^62; U = floor(T^2 / 2^62) = tau^2 2^u
-            // computed exactly from T in 128-bit integer arithmetic.
-            const long long T = __double2ll_rn(scale2(tau, fs.s));
-            const unsigned long long aT = (unsigned long long)(T < 0 ? -T : T);
-            const unsigned long long hi = __umul64hi(aT, aT), lw = aT * aT;
-            const long long U = (long long)((hi << 2) | (lw >> 62));
-            int u1, u0;
-            split_balanced(U, &u1, &u0);
-            const unsigned int t0 = (unsigned int)(T & 0xffffffffll);
-            v.x = (unsigned int)(int)(T >> 32);
-            v.y = 0x4B000000u | (t0 >> 9);                               // 2^23 + (T0 >> 9)
-            v.z = (unsigned int)u1;
-            v.w = 0x4B000000u | (((unsigned int)u0 ^ 0x80000000u) >> 9);  // 2^23 + ((U0+2^31) >> 9)
-            if (MODE == kFoldCertified) a.tau[lo + pos] = tau;
+            const double tau2 = __dmul_rn(tau, tau);
+            const float th = __double2float_rn(tau);
+            const float t2h = __double2float_rn(tau2);
+            reinterpret_cast<float4 *>(a.payload)[lo + pos] =
+                make_float4(th, __double2float_rn(tau - (double)th), t2h,
+                            __double2float_rn(tau2 - (double)t2h));
         }
-        out[pos] = v;
     }
 }
 
@@ -607,7 +555,8 @@ cudaError_t launch_trials(int mode, const TrialArgs &a, bool pdl, cudaStream_t s
     switch (mode) {
         case GCE_PHASE_FP64: return launch_pdl(k_trials<GCE_PHASE_FP64>, g, 256, 0, s, pdl, a);
         case GCE_PHASE_SPLIT32: return launch_pdl(k_trials<GCE_PHASE_SPLIT32>, g, 256, 0, s, pdl, a);
-        case kFoldCertified: return launch_pdl(k_trials<kFoldCertified>, g, 256, 0, s, pdl, a);
+        case kJobFp64: return launch_pdl(k_trials<kJobFp64>, g, 256, 0, s, pdl, a);
+        case kJobFixed32: return launch_pdl(k_trials<kJobFixed32>, g, 256, 0, s, pdl, a);
         default: return launch_pdl(k_trials<GCE_PHASE_FIXED32>, g, 256, 0, s, pdl, a);
     }
 }
@@ -625,7 +574,8 @@ cudaError_t launch_prep(int mode, const PrepArgs &a, bool pdl, cudaStream_t s) {
     switch (mode) {
         case GCE_PHASE_FP64: return launch_pdl(k_prep<GCE_PHASE_FP64>, g, kPrepBlock, 0, s, pdl, a);
         case GCE_PHASE_SPLIT32: return launch_pdl(k_prep<GCE_PHASE_SPLIT32>, g, kPrepBlock, 0, s, pdl, a);
-        case kFoldCertified: return launch_pdl(k_prep<kFoldCertified>, g, kPrepBlock, 0, s, pdl, a);
+        case kJobFp64: return launch_pdl(k_prep<kJobFp64>, g, kPrepBlock, 0, s, pdl, a);
+        case kJobFixed32: return launch_pdl(k_prep<kJobFixed32>, g, kPrepBlock, 0, s, pdl, a);
         default: return launch_pdl(k_prep<GCE_PHASE_FIXED32>, g, kPrepBlock, 0, s, pdl, a);
     }
 }

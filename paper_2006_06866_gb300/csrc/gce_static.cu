@@ -176,7 +176,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     for (const void *a : arrays)
         if (!on_device(a, dev)) return fail(GCE_ERR_INVALID, "an array is on another device");
     cudaStream_t s = (cudaStream_t)stream;
-    // FP64 jobs run the CE kernel's certified fold
+    // FP64 and FIXED32 jobs run the CE kernel's coarse fold
     const int kmode = kernel_mode(cfg->phase_mode);
     const bool overlap = (cfg->flags & GCE_FLAG_OVERLAP) != 0;
     long long n_max = 1;
@@ -218,8 +218,8 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
             t.tpt = 2;
             kv = kernel_variant(overlap);
             range = all_slots;
-            // (16-byte certified points in the bytes of FP64's 8)
-            if (kmode == kFoldCertified && !half) chunk = chunk_max / 2;
+            // (coarse points in no more bytes than the mode's own)
+            if (coarse_mode(kmode)) chunk = chunk_max / 4;
         }
         const int tb = trial_threads(kv, t.block);
         smem = main_smem_bytes(kmode, tb, t.tpt, chunk, cfg->n_phase_bins, cfg->n_mag_bins, table_smem,
@@ -229,14 +229,16 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
         tg = job_tiles(n_periods, n_pdots, tb, t.tpt);
         n_tiles = tg.n_tiles;
         n_lists = n_tiles * (tb / 32);  // one candidate list per warp and tile
-        // the certified payload and its tau take 24 bytes per point; where they don't
-        // fit, the binary64 payload's 8 may
-        mode = kmode;
-        L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 16, kmode == kFoldCertified ? 8 : 0,
+        // the coarse payload and its tau take 32 bytes per point; where they don't fit,
+        // the mode's own payload may
+        mode = job_prep_mode(cfg, n_trials, n_pdots, n_curves, d->n_sm);
+        L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins,
+                   coarse_mode(mode) ? (int)sizeof(CoarsePoint) : 16, coarse_mode(mode) ? 8 : 0,
                    n_lists, k);
-        if (L.end > kScratchBytes && kmode == kFoldCertified) {
-            mode = GCE_PHASE_FP64;
-            L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, 8, 0, n_lists, k);
+        if (L.end > kScratchBytes && coarse_mode(mode)) {
+            mode = cfg->phase_mode;
+            L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins, mode == GCE_PHASE_FP64 ? 8 : 16,
+                       0, n_lists, k);
         }
         if (L.end <= kScratchBytes) break;
         occ = 0;
@@ -287,8 +289,9 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     pa.n_bands = 0;
     if ((e = launch_prep(mode, pa, pdl, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     MainArgs ma;
-    ma.payload = mode == GCE_PHASE_FP64 ? nullptr : b + L.payload;
-    ma.tau = reinterpret_cast<const double *>(b + (mode == GCE_PHASE_FP64 ? L.payload : L.tau));
+    ma.payload = b + L.payload;
+    ma.plain = mode == kmode ? 0 : 1;
+    ma.tau = reinterpret_cast<const double *>(b + L.tau);
     ma.periods = periods;
     ma.pdots = pdots;
     ma.offsets = offsets;

@@ -690,10 +690,14 @@ template <> struct Fields<FMT_PK2, SW_LAST> {  // A, B and the cumulative C; wor
 // logical slots [L, R] start at word w0[s] (slot L), STRIDE words apart; slot
 // L + i counts bin (L + i) mod n, so the first n slots hold one bin each and
 // the e = R - L + 1 - n extra slots L + n + i more points of the bin of slot
-// L + (i mod n) (SPLIT32's two slots per bin).  Each extra word is first merged
-// into its bin's first word and cleared, so the sweep proper reads one word per
-// bin.  SW_LAST clears every word it reads, so the next work item starts from
-// zero counters without a separate pass.
+// L + (i mod n) (SPLIT32's two slots per bin).  An extra word joins its bin's
+// first word as the bin is read, and is cleared (10 curves of 600..1200 points x 1e5
+// periods x 4 Pdot at 50 overlapping bins 2.52 ms, 3000 curves of 100 points x 5e4
+// periods 14.03 ms; 2.56 and 14.18 ms with a pass before, which read and wrote the
+// bin's first word once more).
+// SW_LAST clears every word it reads, so the next work item starts from zero counters
+// without a separate pass.  Bound by the shared-memory pipe: a read, a write and the
+// table's gather (2..3 wavefronts) per word, 84 % of its rate with curves of 100 points.
 // OVL (50 %-overlapping bins, Sec. 2.3): overlapping bin j holds the fine bins j
 // and j + 1 (mod n), so the sum is over T(c_j + c_(j+1)): the first bin is
 // peeled off, each later bin pairs with the one before it, and the last pairs
@@ -725,14 +729,23 @@ struct Sweep {
     }
 
     // G bins of trial s at words cnt[w[s]], cnt[w[s] + STRIDE], ...; PEEL: the
-    // first bin of an OVL sweep
-    template <int G, bool PEEL>
-    __device__ __forceinline__ void step(int (&w)[TPT], unsigned long long (&acc)[TPT]) {
+    // first bin of an OVL sweep; EXTRA: the bins have extra slots, whose words lie
+    // `extra` words on
+    template <int G, bool PEEL, bool EXTRA>
+    __device__ __forceinline__ void step(int (&w)[TPT], unsigned long long (&acc)[TPT], int extra) {
         unsigned int v[TPT][G];
 #pragma unroll
         for (int s = 0; s < TPT; ++s)
 #pragma unroll
-            for (int g = 0; g < G; ++g) v[s][g] = cnt[w[s] + g * STRIDE];
+            for (int g = 0; g < G; ++g) {
+                v[s][g] = cnt[w[s] + g * STRIDE];
+                if (EXTRA) {
+                    unsigned int *const q = cnt + w[s] + extra + g * STRIDE;
+                    const unsigned int x = *q;
+                    *q = 0u;
+                    v[s][g] = F::merge(v[s][g], x);
+                }
+            }
         unsigned long long t[TPT];
 #pragma unroll
         for (int s = 0; s < TPT; ++s) {
@@ -777,23 +790,11 @@ struct Sweep {
     }
 
     // w0[s]: word offset (from cnt) of trial s's first window slot; e: extra
-    // slots, merged first.  The bins [j, end) are swept (all n of them, but for the
-    // warps of a shared trial set).
+    // slots.  The bins [j, end) are swept (all n of them, but for the warps of a
+    // shared trial set), the ones with extra slots first.
     __device__ __forceinline__ void run(const int (&w0)[TPT], int n, int e, int j, int end,
                                         unsigned long long (&acc)[TPT]) {
-        {
-            for (int i = 0, b = 0; i < e; ++i, b = (b + 1 == n) ? 0 : b + 1) {
-                if (b < j || b >= end) continue;
-#pragma unroll
-                for (int s = 0; s < TPT; ++s) {
-                    unsigned int *q = cnt + w0[s] + (n + i) * STRIDE;
-                    unsigned int *f = cnt + w0[s] + b * STRIDE;
-                    const unsigned int x = *q;
-                    *q = 0u;
-                    *f = F::merge(*f, x);
-                }
-            }
-        }
+        const int extra = n * STRIDE;
         int w[TPT];
 #pragma unroll
         for (int s = 0; s < TPT; ++s) w[s] = w0[s] + j * STRIDE;
@@ -801,19 +802,21 @@ struct Sweep {
         // per thread (+1 % over four at 50 overlapping bins)
         constexpr int G = TPT * NF >= 4 ? 2 : (TPT == 1 ? 8 : 4);
         if (OVL) {
-            step<1, true>(w, acc);
+            if (e > 0) step<1, true, true>(w, acc, extra);
+            else step<1, true, false>(w, acc, extra);
             j = 1;
         }
-        for (; j + G <= end; j += G) step<G, false>(w, acc);
+        for (; j < min(e, end); ++j) step<1, false, true>(w, acc, extra);
+        for (; j + G <= end; j += G) step<G, false, false>(w, acc, extra);
         if (G > 4 && (end - j) >= 4) {
-            step<4, false>(w, acc);
+            step<4, false, false>(w, acc, extra);
             j += 4;
         }
         if (G > 2 && (end - j) >= 2) {
-            step<2, false>(w, acc);
+            step<2, false, false>(w, acc, extra);
             j += 2;
         }
-        if (j < end) step<1, false>(w, acc);
+        if (j < end) step<1, false, false>(w, acc, extra);
         if constexpr (OVL && F::kPairWords) {
 #pragma unroll
             for (int s = 0; s < TPT; ++s) {

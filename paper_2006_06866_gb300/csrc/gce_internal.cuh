@@ -431,22 +431,26 @@ __device__ inline FixedTrial fixed_trial(double f, double aa, const FixedScale &
     FixedTrial v;
     // Out-of-range values are flagged by the range check; clamp so the conversions stay defined.
     const double F = fmin(scale2(f, fs.r), 9.2e18);
-    const double A = fmax(fmin(scale2(aa, fs.v), 9.2e18), -9.2e18);
     int f1, f0;
     split_balanced(__double2ll_rn(F), &f1, &f0);
-    const long long an = -__double2ll_rn(A);
+    long long an = 0;
+    if (aa != 0.0) an = -__double2ll_rn(fmax(fmin(scale2(aa, fs.v), 9.2e18), -9.2e18));
     const int a1 = (int)(an >> 32);
     const unsigned int a0 = (unsigned int)(an & 0xffffffffll);
     // k: the smallest shift with F1 < 2^(22+k)
     const unsigned int uf1 = (unsigned int)f1;
     const int bits = 32 - __clz(uf1);
     const int k = bits > 22 ? bits - 22 : 0;
-    const float g0 = __double2float_rn(scale2((double)uf1, -23 - k));
-    const float g2 = __double2float_rn(scale2((double)a1, -23 - k));
-    const double kk = 12582912.0 - 8388608.0 * (double)g0 - 8388608.0 * (double)g2 -
-                      scale2((double)a1, -1 - k);
+    const float scale = __uint_as_float((unsigned int)(104 - k) << 23);  // 2^(-23-k)
+    const float g0 = __uint2float_rn(uf1) * scale;
+    const float g2 = __int2float_rn(a1) * scale;
+    // rounded once: the binary64 terms are exact, and so is 2^23 g0
+    float kk = __fsub_rn(12582912.0f, 8388608.0f * g0);
+    if (a1 != 0)
+        kk = __double2float_rn(12582912.0 - 8388608.0 * (double)g0 - 8388608.0 * (double)g2 -
+                               scale2((double)a1, -1 - k));
     v.i = make_uint4(uf1, (unsigned int)f0, (unsigned int)a1, a0);
-    v.f = make_float4(g0, g2, __double2float_rn(kk), __uint_as_float((unsigned int)k));
+    v.f = make_float4(g0, g2, kk, __uint_as_float((unsigned int)k));
     return v;
 }
 
@@ -490,7 +494,8 @@ __device__ inline CoarseTrial coarse_trial(double f, double aa, int e, bool own_
     t.F1 = (unsigned int)hi;
     t.F1f = (float)hi;
     t.F0 = (float)lo * 2.3283064365386963e-10f;
-    split_balanced(-__double2ll_rn(scale2(aa, 38 + 2 * e)), &hi, &lo);
+    hi = lo = 0;
+    if (aa != 0.0) split_balanced(-__double2ll_rn(scale2(aa, 38 + 2 * e)), &hi, &lo);
     t.A1 = (unsigned int)hi;
     t.A1f = (float)hi;
     t.A0 = (float)lo * 2.3283064365386963e-10f;
@@ -614,37 +619,57 @@ struct TileStats {
     double n, mean, m2;
 };
 
-// The moments of a block's records [0, n) merged (every thread returns them): the
-// mean from the sums of n and n mean, then M2 from the records' own and their means'
-// distances, each in a fixed order (a strided run per thread, a fixed tree, the
-// warps in order), so the result is deterministic.  Two passes instead of a pairwise
-// update, which divides twice per merge (the whole merge kernel, 782 lists of one curve:
-// 32 -> 13 us).
-__device__ inline double block_sum_fixed(double v, double *sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-    return t;
+// The moments of a block's records [0, n) merged: the mean from the sums of n and
+// n mean, then M2 from the records' own and their means' distances, each in a fixed
+// order (a strided run per thread, then a fixed tree), so the result is deterministic.
+// Two passes instead of a pairwise update, which divides twice per merge.  A warp's
+// binary64 operation holds the SM's unit for 16 cycles, however few lanes it is for,
+// so the block's sums and the division are the first warp's alone (shuffle sums in
+// every warp and the rest in every thread: the whole merge of 300 curves with 313 lists
+// each 14.8 -> 10.2 us).
+// sh: kMomentsBlock (the block's threads) doubles, twice.  Thread 0 returns all three.
+constexpr int kMomentsBlock = 256;
+__device__ inline double block_sum_fixed(const double *sh) {  // first warp; lane 0's result
+    double v[kMomentsBlock / 32];
+#pragma unroll
+    for (int w = 0; w < kMomentsBlock / 32; ++w) v[w] = sh[threadIdx.x + 32 * w];
+#pragma unroll
+    for (int o = kMomentsBlock / 64; o > 0; o >>= 1)
+#pragma unroll
+        for (int w = 0; w < o; ++w) v[w] += v[w + o];
+    for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
 }
 __device__ inline TileStats block_moments(const TileStats *ts, int n, double *sh) {
+    const int tid = threadIdx.x;
     double c = 0.0, m = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+#pragma unroll 4
+    for (int i = tid; i < n; i += kMomentsBlock) {
         c += ts[i].n;
         m += ts[i].n * ts[i].mean;
     }
+    sh[tid] = c;
+    sh[kMomentsBlock + tid] = m;
+    __syncthreads();
     TileStats r;
-    r.n = block_sum_fixed(c, sh);
-    r.mean = block_sum_fixed(m, sh);
-    if (r.n > 0.0) r.mean /= r.n;
+    if (tid < 32) {
+        r.n = block_sum_fixed(sh);
+        r.mean = block_sum_fixed(sh + kMomentsBlock);
+        if (r.n > 0.0) r.mean /= r.n;
+    }
+    __syncthreads();
+    if (tid == 0) sh[0] = r.mean;
+    __syncthreads();
+    const double mean = sh[0];
     double q = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double d = ts[i].mean - r.mean;
+#pragma unroll 4
+    for (int i = tid; i < n; i += kMomentsBlock) {
+        const double d = ts[i].mean - mean;
         if (ts[i].n > 0.0) q += ts[i].m2 + ts[i].n * d * d;
     }
-    r.m2 = block_sum_fixed(q, sh);
+    sh[kMomentsBlock + tid] = q;
+    __syncthreads();
+    if (tid < 32) r.m2 = block_sum_fixed(sh + kMomentsBlock);
     return r;
 }
 

@@ -8,7 +8,7 @@ namespace gce {
 
 namespace {
 
-constexpr int kMergeBlock = 256;
+constexpr int kMergeBlock = kMomentsBlock;
 constexpr int kMergeKeys = 16;  // keys a merging thread holds in registers
 
 // Per-curve merge of the candidate lists: k rounds of "smallest key above the
@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(kMergeBlock)
                  double *std_out, float *rho_out, const JobState *st) {
     constexpr int WARPS = kMergeBlock / 32;
     __shared__ unsigned long long sh[2][WARPS];
-    __shared__ double shs[WARPS];
+    __shared__ double shs[2 * kMomentsBlock];
     pdl_trigger();
     pdl_wait();
     if (st->err) return;

@@ -108,7 +108,9 @@ __global__ void k_scan(const double *__restrict__ times, const double *__restric
 }
 
 // Per flat trial t = q n_periods + p: f = 1/P, a = (0.5 Pdot) f f (the oracle's
-// sequence), stored in the fold mode's format.
+// sequence), stored in the fold mode's format.  Bound by binary64 arithmetic at 2
+// lanes per clock and SM, so what binary32 holds exactly is done there, and nothing
+// for a Pdot of 0 (5e4 FIXED32 trials 8.4 -> 5.9 us).
 template <int MODE>
 __global__ void k_trials(TrialArgs a) {
     pdl_trigger();

@@ -14,7 +14,7 @@ namespace gce {
 namespace {
 
 constexpr unsigned long long kEmptyKey = ~0ull;
-constexpr int kReduceBlock = 256;
+constexpr int kReduceBlock = kMomentsBlock;
 
 // Smallest 64-bit key of the warp: the smallest high word, then the smallest
 // low word among the lanes holding it.
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(kReduceBlock)
                   const JobState *st) {
     __shared__ unsigned long long s_keys[kReduceKeys];
     __shared__ unsigned long long s_warp[kReduceBlock / 32];
-    __shared__ double s_mom[kReduceBlock / 32];
+    __shared__ double s_mom[2 * kMomentsBlock];
     pdl_trigger();
     pdl_wait();
     if (st->err) return;

@@ -100,7 +100,17 @@ bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_t
             return true;
         }
     }
-    if (warps <= 20 * schedulers) t.tpt = std::min(t.tpt, 2);
+    if (mode == GCE_PHASE_FP64) {
+        // As many as a FIXED32 job, which runs the same fold (a caller's own or the
+        // tuner's shape has at most two).  100 curves x 1000 points x 2e4 periods, the
+        // CE kernel: 0.85 ms with two, 0.80 with four; 23 x 487 x 1e4 x 16 Pdot 1.03 /
+        // 0.87; 300 x 50..2000 x 1e4 0.80 / 0.70.  Near 20 w, where four leave one wave
+        // and a bit, 20 x 200 points 0.076 / 0.079, from 25 w on 0.089 / 0.086.
+        gce_config fixed = *cfg;
+        fixed.phase_mode = GCE_PHASE_FIXED32;
+        t.tpt = default_tuning(&fixed, n_pdots).tpt;
+    }
+    if (warps <= (mode == GCE_PHASE_FP64 ? 24 : 20) * schedulers) t.tpt = std::min(t.tpt, 2);
     if (few && !stats) t.tpt = 1;
     if (keep2) {
         t.tpt = std::max(t.tpt, 2);

@@ -853,6 +853,7 @@ const void *main_kernel_ptr(int mode, int tpt, int block, int kv);
                                           cudaStream_t s);
 GCE_MAIN_TU(fp64, 1)
 GCE_MAIN_TU(fp64, 2)
+GCE_MAIN_TU(fp64, 4)
 GCE_MAIN_TU(split32, 1)
 GCE_MAIN_TU(split32, 2)
 GCE_MAIN_TU(split32, 4)

@@ -154,6 +154,7 @@ const void *main_kernel_ptr(int mode, int tpt, int block, int kv) {
     switch (mode * 8 + tpt) {
         case kJobFp64 * 8 + 1: return main_kernel_ptr_fp64_t1(block, kv);
         case kJobFp64 * 8 + 2: return main_kernel_ptr_fp64_t2(block, kv);
+        case kJobFp64 * 8 + 4: return main_kernel_ptr_fp64_t4(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 1: return main_kernel_ptr_split32_t1(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 2: return main_kernel_ptr_split32_t2(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 4: return main_kernel_ptr_split32_t4(block, kv);
@@ -192,6 +193,7 @@ cudaError_t launch_main(int mode, int tpt, int block, int grid, size_t smem, con
     switch (mode * 8 + tpt) {
         case kJobFp64 * 8 + 1: return launch_main_fp64_t1(block, grid, smem, a, s);
         case kJobFp64 * 8 + 2: return launch_main_fp64_t2(block, grid, smem, a, s);
+        case kJobFp64 * 8 + 4: return launch_main_fp64_t4(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 1: return launch_main_split32_t1(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 2: return launch_main_split32_t2(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 4: return launch_main_split32_t4(block, grid, smem, a, s);

@@ -127,9 +127,9 @@ typedef struct gce_handle_s *gce_handle;
  * The workspace grows to the largest job seen and is kept until gce_destroy:
  * 16 bytes per point (FP64 and FIXED32: 32), 16 (SPLIT32) or 32 (FIXED32, FP64)
  * bytes per (P, Pdot) trial (where those of FP64 or FIXED32 do not fit, 8 or 16
- * per point and 16 or 32 per trial, at the speed of their own folds), 8 k bytes per (curve, warp of a trial tile) for top-k (24 more with
- * the significance), and 8 bytes per entry of the c ln c table (longest curve
- * + 1).  A grid of 5,183,995 periods x 512 Pdot values thus holds 42 GB of
+ * per point and 16 or 32 per trial, at the speed of their own folds), 8 k bytes per
+ * (curve, warp of a trial tile) for top-k (24 or 48 more with the significance),
+ * and 8 bytes per entry of the c ln c table (longest curve + 1).  A grid of 5,183,995 periods x 512 Pdot values thus holds 42 GB of
  * trial constants in SPLIT32.  Growing a buffer waits for the device. */
 gce_status gce_create(gce_handle *h, int32_t device);
 
@@ -174,9 +174,9 @@ gce_status gce_ce_topk(gce_handle h, const double *times, const double *mags,
 /* gce_ce_topk plus the significance of the minimum (Eq. 5, Sec. 2.3):
  * rho[c] = (mean[c] - topk_H[c*k]) / std[c], where mean and std (population,
  * ddof 0) are over all n_pdots * n_periods CE values of curve c.  The moments
- * are accumulated per trial tile and merged in a fixed order with Chan et al.'s
- * pairwise update (the batch-statistics merge of Sec. 4), so results are
- * deterministic.  mean, std: device double[n_curves]; rho: device
+ * are accumulated per list of 64 trials (32 with one trial per thread) and merged
+ * in a fixed order (the mean first, then the squared deviations from it: the
+ * batch-statistics merge of Sec. 4), so results are deterministic.  mean, std: device double[n_curves]; rho: device
  * float[n_curves] (0 when std is 0). */
 gce_status gce_ce_detect(gce_handle h, const double *times, const double *mags,
                          const int64_t *h_offsets, int32_t n_curves, const double *periods,
@@ -242,7 +242,8 @@ gce_status gce_ce_topk_host(gce_handle h, const double *h_times, const double *h
  * 32 MiB (about 16 B per point (FP64: 8) + 32 B per trial + 8 B per (curve, 64 trials,
  * k) + 0.5 MiB); use gce_ce_topk for larger jobs.  Returns
  * GCE_ERR_UNSUPPORTED when the bin counts need more shared memory than one CTA
- * of its fixed launch shape (256 threads, 2 trials each) can have.
+ * of 256 threads with 2 trials each can have.  The launch shape is the job's own
+ * or, where that needs more scratch or shared memory, that one.
  * Every call looks up the array's device address; the first call on a device
  * (and the first after a device reset, which moves the array) also fills a
  * table in it with a few synchronous CUDA calls: make the first call before

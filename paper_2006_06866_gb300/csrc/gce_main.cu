@@ -158,6 +158,9 @@ const void *main_kernel_ptr(int mode, int tpt, int block, int kv) {
         case GCE_PHASE_SPLIT32 * 8 + 1: return main_kernel_ptr_split32_t1(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 2: return main_kernel_ptr_split32_t2(block, kv);
         case GCE_PHASE_SPLIT32 * 8 + 4: return main_kernel_ptr_split32_t4(block, kv);
+        case GCE_PHASE_FIXED32 * 8 + 1: return main_kernel_ptr_fixed32own_t1(block, kv);
+        case GCE_PHASE_FIXED32 * 8 + 2: return main_kernel_ptr_fixed32own_t2(block, kv);
+        case GCE_PHASE_FIXED32 * 8 + 4: return main_kernel_ptr_fixed32own_t4(block, kv);
         case kJobFixed32 * 8 + 1: return main_kernel_ptr_fixed32_t1(block, kv);
         case kJobFixed32 * 8 + 2: return main_kernel_ptr_fixed32_t2(block, kv);
         case kJobFixed32 * 8 + 4: return main_kernel_ptr_fixed32_t4(block, kv);
@@ -197,6 +200,9 @@ cudaError_t launch_main(int mode, int tpt, int block, int grid, size_t smem, con
         case GCE_PHASE_SPLIT32 * 8 + 1: return launch_main_split32_t1(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 2: return launch_main_split32_t2(block, grid, smem, a, s);
         case GCE_PHASE_SPLIT32 * 8 + 4: return launch_main_split32_t4(block, grid, smem, a, s);
+        case GCE_PHASE_FIXED32 * 8 + 1: return launch_main_fixed32own_t1(block, grid, smem, a, s);
+        case GCE_PHASE_FIXED32 * 8 + 2: return launch_main_fixed32own_t2(block, grid, smem, a, s);
+        case GCE_PHASE_FIXED32 * 8 + 4: return launch_main_fixed32own_t4(block, grid, smem, a, s);
         case kJobFixed32 * 8 + 1: return launch_main_fixed32_t1(block, grid, smem, a, s);
         case kJobFixed32 * 8 + 2: return launch_main_fixed32_t2(block, grid, smem, a, s);
         case kJobFixed32 * 8 + 4: return launch_main_fixed32_t4(block, grid, smem, a, s);

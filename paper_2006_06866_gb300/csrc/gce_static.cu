@@ -206,7 +206,9 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     int kv = kernel_variant(overlap);
     if (fit_to_job(t, cfg, n_pdots, n_trials, n_curves, n_points, d->n_sm, false) && !overlap)
         kv = KV_SHARED;
-    int chunk = chunk_max, range = split_range(cfg->phase_mode, n_pdots, t.slot_range), mode = kmode;
+    const int prep_mode = job_prep_mode(cfg, n_trials, n_pdots, n_curves, d->n_sm);
+    const int main_kmode = main_mode(prep_mode, cfg->phase_mode);
+    int chunk = chunk_max, range = split_range(cfg->phase_mode, n_pdots, t.slot_range), mode = prep_mode;
     size_t smem = 0;
     int occ = 0;
     long long n_lists = 0, n_tiles = 0;
@@ -219,19 +221,19 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
             kv = kernel_variant(overlap);
             range = all_slots;
             // (coarse points in no more bytes than the mode's own)
-            if (coarse_mode(kmode)) chunk = chunk_max / 4;
+            if (coarse_mode(main_kmode)) chunk = chunk_max / 4;
         }
         const int tb = trial_threads(kv, t.block);
-        smem = main_smem_bytes(kmode, tb, t.tpt, chunk, cfg->n_phase_bins, cfg->n_mag_bins, table_smem,
+        smem = main_smem_bytes(main_kmode, tb, t.tpt, chunk, cfg->n_phase_bins, cfg->n_mag_bins, table_smem,
                                range, half);
-        occ = fitted(d, main_kernel_ptr(kmode, t.tpt, t.block, kv), kmode, t.tpt, t.block, kv, smem);
+        occ = fitted(d, main_kernel_ptr(main_kmode, t.tpt, t.block, kv), main_kmode, t.tpt, t.block, kv, smem);
         if (occ < 1) continue;
         tg = job_tiles(n_periods, n_pdots, tb, t.tpt);
         n_tiles = tg.n_tiles;
         n_lists = n_tiles * (tb / 32);  // one candidate list per warp and tile
         // the coarse payload and its tau take 32 bytes per point; where they don't fit,
         // the mode's own payload may
-        mode = job_prep_mode(cfg, n_trials, n_pdots, n_curves, d->n_sm);
+        mode = prep_mode;
         L = layout(n_points, n_curves, n_trials, cfg->n_mag_bins,
                    coarse_mode(mode) ? (int)sizeof(CoarsePoint) : 16, coarse_mode(mode) ? 8 : 0,
                    n_lists, k);
@@ -290,7 +292,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     if ((e = launch_prep(mode, pa, pdl, s)) != cudaSuccess) return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     MainArgs ma;
     ma.payload = b + L.payload;
-    ma.plain = mode == kmode ? 0 : 1;
+    ma.plain = mode == main_kmode ? 0 : 1;
     ma.tau = reinterpret_cast<const double *>(b + L.tau);
     ma.periods = periods;
     ma.pdots = pdots;
@@ -324,7 +326,7 @@ extern "C" gce_status gce_ce_topk_static(const double *times, const double *mags
     ma.kv = kv;
     ma.pdl = pdl ? 1 : 0;
     ma.state = state;
-    if ((e = launch_main(kmode, tpt, block, (int)grid, smem, ma, s)) != cudaSuccess)
+    if ((e = launch_main(main_kmode, tpt, block, (int)grid, smem, ma, s)) != cudaSuccess)
         return fail(GCE_ERR_CUDA, cudaGetErrorString(e));
     e = launch_topk_merge(ma.cand, n_curves, (int)n_lists, k, 1, topk_H, (long long *)topk_idx,
                           nullptr, nullptr, nullptr, nullptr, state, pdl, s);

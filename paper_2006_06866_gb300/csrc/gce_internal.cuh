@@ -477,11 +477,14 @@ constexpr unsigned int kCoarseOffset = 0u - (0x4E400000u << 6);  // cancels its 
 __device__ inline CoarsePoint coarse_point(double tau, int e) {
     CoarsePoint p;
     int hi, lo;
-    split_balanced(__double2ll_rn(scale2(tau, 58 - e)), &hi, &lo);
+    const long long T = __double2ll_rn(scale2(tau, 58 - e));
+    split_balanced(T, &hi, &lo);
     p.T1 = (unsigned int)hi;
     p.T1f = (float)hi;
     p.b = (float)lo * 2.3283064365386963e-10f;  // 2^-32
-    split_balanced(__double2ll_rn(scale2(__dmul_rn(tau, tau), 58 - 2 * e)), &hi, &lo);
+    // U = floor(T^2 / 2^58) in integers: tau^2 itself may be beyond binary64's range
+    const unsigned long long aT = (unsigned long long)(T < 0 ? -T : T);
+    split_balanced((long long)((__umul64hi(aT, aT) << 6) | ((aT * aT) >> 58)), &hi, &lo);
     p.U1 = (unsigned int)hi;
     p.U1f = (float)hi;
     p.ub = (float)lo * 2.3283064365386963e-10f;

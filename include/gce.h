@@ -31,6 +31,13 @@
  *     magnitudes, non-positive or non-finite periods, non-finite pdots, a trial
  *     range the chosen fold cannot represent) run on the GPU; they are reported
  *     by gce_stream_status(), and outputs of a flagged call are unspecified.
+ *   - Calls on one handle run one after another on the device, whatever streams
+ *     they are given: each waits there for the one before it.  A caller may
+ *     capture a call into a graph of its own (GCE_FLAG_NO_GRAPH, relaxed capture
+ *     mode, after a call of the same size has grown the workspace).  The graph
+ *     then uses the handle's workspace and its staged offsets: the caller orders
+ *     its replays with the handle's other calls, and replays it only while the
+ *     handle's last call had the same offsets.
  *   - Nothing throws across the ABI.  A handle is not thread-safe: use one per
  *     host thread.  CUDA failures return GCE_ERR_CUDA with the text available
  *     from gce_last_error().

@@ -190,10 +190,11 @@ struct gce_handle_s {
     long long *h_offsets = nullptr;
     size_t h_cap = 0;
     JobState *h_state = nullptr;         // pinned copy target for the check flags
-    cudaEvent_t staged = nullptr;        // staging buffers free again after this
+    cudaEvent_t staged = nullptr;        // after the last job: workspace and staging buffers free
     bool staged_pending = false;
+    cudaStream_t last_stream = nullptr;  // the stream of that event, and its id
+    unsigned long long last_id = 0;
     int staged_n = -1;                   // curves whose offsets and order the buffers hold
-    cudaStream_t last_stream = nullptr;  // of the last job (its event: staged)
     cudaEvent_t k0 = nullptr, k1 = nullptr;  // around the CE kernel (GCE_FLAG_TIME_KERNEL)
     bool timed = false;
     int launches = 0;                    // kernels the last job launched (directly or in its graph)
@@ -738,9 +739,25 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
     if (j.bands && (j.n_bands < 1 || j.n_bands > GCE_MAX_BANDS))
         return fail(h, GCE_ERR_INVALID, "n_bands must be 1 .. %d", GCE_MAX_BANDS);
     CUDA_TRY(h, cudaSetDevice(h->device));
-    // jobs on one stream follow one another; one on another stream waits on the
-    // device for the handle's workspace
-    if (h->staged_pending && s != h->last_stream) CUDA_TRY(h, cudaStreamWaitEvent(s, h->staged, 0));
+    // The job waits on the device for the handle's last one, which may still use the
+    // workspace, unless that ran on the very same stream (a small call is bound by the
+    // host, and the wait would take 1 to 3 of its 36 us).  A stream's handle value does
+    // not identify it: a destroyed stream's is given out again, so the ids are compared,
+    // and the per-thread default stream has one value in every thread, so it never
+    // counts as the same.  A stream that the caller is capturing cannot wait for an
+    // event from outside the capture: there the host waits.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (s != nullptr) CUDA_TRY(h, cudaStreamIsCapturing(s, &cap));
+    const bool captured = cap != cudaStreamCaptureStatusNone;
+    unsigned long long stream_id = 0;
+    if (s != nullptr && !captured) CUDA_TRY(h, cudaStreamGetId(s, &stream_id));
+    if (h->staged_pending && captured) {
+        CUDA_TRY(h, cudaEventSynchronize(h->staged));
+        h->staged_pending = false;
+    } else if (h->staged_pending &&
+               (s != h->last_stream || stream_id != h->last_id || s == cudaStreamPerThread)) {
+        CUDA_TRY(h, cudaStreamWaitEvent(s, h->staged, 0));
+    }
     {
         // arrays already checked by the previous call (same argument, same
         // pointer) need no new query
@@ -793,7 +810,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
         if ((st = ensure(h, h->table, 8 * (size_t)(pl.n_max + 1))) != GCE_OK) return st;
         CUDA_TRY(h, launch_table((unsigned long long *)h->table.p, pl.n_max, s));
         ++h->launches;
-        h->table_n = pl.n_max;
+        if (!captured) h->table_n = pl.n_max;  // (a captured launch has filled nothing yet)
     }
 
     // host staging (pinned): offsets and the longest-first curve order.  Every job's
@@ -826,11 +843,16 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
                            j.kind != JOB_SINGLE;
     h->timed = (j.cfg->flags & GCE_FLAG_TIME_KERNEL) != 0 && j.kind != JOB_COUNTS;
     if (!use_graph) {
-        // (the caller may be capturing the stream)
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (s != nullptr) CUDA_TRY(h, cudaStreamIsCapturing(s, &cap));
-        st = enqueue(h, j, pl, s, false, cap == cudaStreamCaptureStatusNone);
-        if (st != GCE_OK) return st;
+        st = enqueue(h, j, pl, s, false, !captured);
+        if (st != GCE_OK) {
+            // the kernels before the one that failed may be on the stream
+            if (!captured && cudaEventRecord(h->staged, s) == cudaSuccess) {
+                h->staged_pending = true;
+                h->last_stream = s;
+                h->last_id = stream_id;
+            }
+            return st;
+        }
     } else {
         GraphKey key{j.kind * 8 + (j.bands ? 4 : 0) + (j.rho ? 2 : 0) +
                          ((j.cfg->flags & GCE_FLAG_OVERLAP) ? 1 : 0),
@@ -903,9 +925,11 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
         }
         CUDA_TRY(h, cudaGraphLaunch(h->graphs[key].exec, s));
     }
+    if (captured) return GCE_OK;  // nothing has been submitted
     CUDA_TRY(h, cudaEventRecord(h->staged, s));
     h->staged_pending = true;
     h->last_stream = s;
+    h->last_id = stream_id;
     return GCE_OK;
 }
 

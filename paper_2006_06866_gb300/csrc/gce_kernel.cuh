@@ -328,8 +328,6 @@ __device__ __forceinline__ unsigned int own_bin(const MainArgs &a, long long k, 
     const double f = 1.0 / a.periods[t - q * a.n_periods];
     const double aa = (0.5 * a.pdots[q]) * f * f;
     const double tau = a.tau[k];
-    // t = t0: phase 0 in both folds (FIXED32's rounds to it exactly without Pdot)
-    if (tau == 0.0 && (MODE == kJobFp64 || aa == 0.0)) return 0u;
     if (MODE == kJobFp64) return (unsigned int)fold_fp64<true>(tau, f, aa, fk.nphi_d, fk.n_phase);
     const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
     return (unsigned int)fold_fixed<true>(fixed_point(tau, fs), fixed_prep(fixed_trial(f, aa, fs)),
@@ -345,20 +343,27 @@ struct Undecided {
 };
 
 // The undecided points of one trial per lane go where the mode's own fold puts them.
-// Called by the whole warp: lane after lane, all lanes test the points of that lane's
-// blocks with its trial (and the one that finds an undecided point decides it).  Rare
-// (a point-trial is undecided with probability 2 margin n_phase 2^-32, 8e-7 at 15
-// bins), but what matters is its latency, which the CTA's other warps wait for at
-// their next barrier: with each lane walking its own blocks it took 33 us and 12 % of
-// the kernel.
+// Called by the whole warp.  Few lanes with some: lane after lane, all lanes test the
+// points of that lane's blocks with its trial (and the one that finds an undecided point
+// decides it).  Rare (a point-trial is undecided with probability 2 margin n_phase 2^-32,
+// 8e-7 at 15 bins), but what matters is its latency, which the CTA's other warps wait for
+// at their next barrier: with each lane walking its own blocks it took 33 us and 12 % of
+// the kernel.  From kManyLanes lanes on each walks its own blocks all the same: a point
+// may be undecided in every trial (its time a rounding error away from t0, or a cadence
+// that the trial frequencies divide), and lane after lane those cost more than the fold.
+constexpr int kManyLanes = 4;
 template <int MODE, int SH>
 __device__ __noinline__ void settle(const MainArgs &a, Undecided u, CoarseTrial tr, long long t,
                                     long long pt0, CoarseSite site, bool half, int ka, int kb,
                                     unsigned int base, unsigned int inc, unsigned int thr, FoldConst fk) {
     const int lane = threadIdx.x & 31;
     if (t >= a.n_trials) u.mask = 0u;
-    for (unsigned int lanes = __ballot_sync(0xffffffffu, u.mask != 0u); lanes; lanes &= lanes - 1u) {
-        const int l = __ffs((int)lanes) - 1;
+    unsigned int lanes = __ballot_sync(0xffffffffu, u.mask != 0u);
+    const bool many = __popc(lanes) >= kManyLanes;
+    const int first = many ? 0 : lane, step = many ? 1 : 32;
+    while (lanes) {
+        const int l = many ? lane : __ffs((int)lanes) - 1;
+        lanes = many ? 0u : lanes & (lanes - 1u);
         CoarseTrial x;
         x.F1 = __shfl_sync(0xffffffffu, tr.F1, l);
         x.F0 = __shfl_sync(0xffffffffu, tr.F0, l);
@@ -372,7 +377,7 @@ __device__ __noinline__ void settle(const MainArgs &a, Undecided u, CoarseTrial 
         FoldConst xk = fk;
         xk.c0 = __shfl_sync(0xffffffffu, fk.c0, l);
         auto range = [&](int from, int to) {
-            for (int k = from + lane; k < to; k += 32) {
+            for (int k = from + first; k < to; k += step) {
                 CoarsePoint p[2];
                 if (half) {
                     staged_coarse<true, false>(site, k >> 1, p);
@@ -899,8 +904,9 @@ constexpr int main_min_blocks(int tpt, int log2b, int kv) {
                     : (log2b >= 9 ? 1 : (log2b == 8 ? 2 : (log2b == 7 ? 4 : 8)));
 }
 
-// LAYMODE: the fold mode that the launch's shared memory was laid out for.
-template <int MODE, int LAYMODE, int TPT, int LOG2B, int KV>
+// LAYMODE: the fold mode that the launch's shared memory was laid out for.  EPOCH: a
+// coarse job with points at the epoch (segment_word).
+template <int MODE, int LAYMODE, int TPT, int LOG2B, int KV, bool EPOCH>
 __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
     // the counter formats are fixed per instantiation (a kernel that carried
     // the overlapping-bin format with a run-time choice measured slower on the
@@ -1137,8 +1143,11 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                 staged_lo = lo;
             }
             for (int i = 0; i < n_mag; ++i) {
-                const int s0 = s_seg[i], s1 = s_seg[i + 1];
-                int ka = max(s0, lo), kb = min(s1, hi);
+                const int w0 = s_seg[i], w1 = s_seg[i + 1];
+                const int s0 = EPOCH ? segment_start((unsigned int)w0) : w0;
+                const int s1 = EPOCH ? segment_start((unsigned int)w1) : w1;
+                const int zeros = EPOCH ? segment_zeros((unsigned int)w0) : 0;
+                int ka = max(s0, lo), kb = min(s1 - zeros, hi);
                 if (SHARED_SET && ka < kb) {
                     // the warp's share, cut between pairs of points
                     const int per = (kb - ka + WARPS - 1) / WARPS, from = ka, to = kb;
@@ -1180,6 +1189,20 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
                     }
                 }
                 if (s1 > s0 && s1 > lo && s1 <= hi) {
+                    if constexpr (EPOCH) {
+                        const unsigned int inc = pk2 ? ((ended & 1) ? kPk2IncB : 1u) + kPk2IncC : 1u;
+                        if (zeros > 0 && (!SHARED_SET || warp == 0)) {
+#pragma unroll
+                            for (int s = 0; s < TPT; ++s) {
+                                const unsigned int j =
+                                    MODE == kJobFp64 ? 0u
+                                                     : __umulhi(g_tr[min(tt[s], a.n_trials - 1)].zero,
+                                                                (unsigned int)n_phase);
+                                bump<MODE, SH>(base[s], j << SH, fk, (unsigned int)zeros * inc);
+                            }
+                            compiler_fence();
+                        }
+                    }
                     // end of non-empty magnitude segment i: sweep its counts (FMT_PK2:
                     // after every second one); after the curve's last segment one sweep
                     // takes its counts and the cumulative ones (the marginal term) and
@@ -1304,11 +1327,18 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
     if (a.state->err) return;  // inputs failed the device checks: no work
     if constexpr (coarse_mode(MODE)) {
         if (a.plain || a.state->wide) {
-            ce_items<MODE == kJobFp64 ? GCE_PHASE_FP64 : GCE_PHASE_FIXED32, MODE, TPT, LOG2B, KV>(a, s_item);
+            ce_items<MODE == kJobFp64 ? GCE_PHASE_FP64 : GCE_PHASE_FIXED32, MODE, TPT, LOG2B, KV, false>(a, s_item);
+            return;
+        }
+        // (the code for points at the epoch apart from the code without: in one, its few
+        // instructions per segment cost 100 curves of 200..1000 points x 5e4 x 16 Pdot at
+        // 20 bins 1.0 to 1.7 %)
+        if (a.state->epoch) {
+            ce_items<MODE, MODE, TPT, LOG2B, KV, true>(a, s_item);
             return;
         }
     }
-    ce_items<MODE, MODE, TPT, LOG2B, KV>(a, s_item);
+    ce_items<MODE, MODE, TPT, LOG2B, KV, false>(a, s_item);
 }
 
 template <int MODE, int TPT, int LOG2B>

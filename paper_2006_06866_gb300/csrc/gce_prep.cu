@@ -24,6 +24,7 @@ __device__ __forceinline__ void clear_state(JobState *st) {
     st->err = 0u;
     st->work = 0ull;
     st->wide = 0u;
+    st->epoch = 0u;
 }
 __global__ void k_init(JobState *st, const long long *h_offsets, const int *h_order,
                        long long *offsets, int *order, int n_curves) {
@@ -67,6 +68,13 @@ __device__ inline double warp_min(double v) {
     return v;
 }
 
+// t - t0 == 0, on the bits (binary64 arithmetic bounds the preparation)
+__device__ inline bool at_epoch(double t, double t0) {
+    const unsigned long long x = (unsigned long long)__double_as_longlong(t);
+    const unsigned long long y = (unsigned long long)__double_as_longlong(t0);
+    return x == y || ((x | y) << 1) == 0ull;
+}
+
 // Checks every time, magnitude, period and period derivative; reduces
 // max |t - t0|, min P and max |Pdot|.
 __global__ void k_scan(const double *__restrict__ times, const double *__restrict__ mags,
@@ -74,7 +82,7 @@ __global__ void k_scan(const double *__restrict__ times, const double *__restric
                        const double *__restrict__ pdots, int n_pdots, double t0, JobState *st) {
     pdl_trigger();
     pdl_wait();
-    unsigned int err = 0u;
+    unsigned int err = 0u, epoch = 0u;
     double tmax = 0.0, pmin = INFINITY, dmax = 0.0;
     long long stride = (long long)gridDim.x * blockDim.x;
     long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -82,6 +90,7 @@ __global__ void k_scan(const double *__restrict__ times, const double *__restric
         double t = times[i], m = mags[i];
         if (!isfinite(t) || !isfinite(m)) err |= ERR_TIME;
         double tau = fabs(t - t0);
+        epoch |= at_epoch(t, t0) ? 1u : 0u;
         if (isfinite(tau)) tmax = fmax(tmax, tau);
         else err |= ERR_TIME;
     }
@@ -99,11 +108,13 @@ __global__ void k_scan(const double *__restrict__ times, const double *__restric
     dmax = warp_max(dmax);
     pmin = warp_min(pmin);
     err = __reduce_or_sync(0xffffffffu, err);
+    epoch = __reduce_or_sync(0xffffffffu, epoch);
     if ((threadIdx.x & 31) == 0) {
         if (tmax > 0.0) atomic_max_pos(&st->tau_max_bits, tmax);
         if (dmax > 0.0) atomic_max_pos(&st->pdot_max_bits, dmax);
         if (pmin < INFINITY) atomic_min_pos(&st->pmin_bits, pmin);
         if (err) atomicOr(&st->err, err);
+        if (epoch) st->epoch = 1u;
     }
 }
 
@@ -150,7 +161,7 @@ __global__ void k_trials(TrialArgs a) {
             reinterpret_cast<FixedTrial *>(a.trialc)[t] = fixed_trial(f, aa, fs);
         } else if (coarse_mode(MODE)) {
             reinterpret_cast<CoarseTrial *>(a.trialc)[t] =
-                coarse_trial(f, aa, fs.e_tau, MODE == kJobFixed32);
+                coarse_trial(f, aa, fs, MODE == kJobFixed32, a.state->epoch != 0u);
         } else {
             // f split, and -a split (the fold adds -a tau^2)
             const float fh = __double2float_rn(f);
@@ -424,11 +435,12 @@ struct MagView {
 // One CTA per curve: min/max of the magnitudes, magnitude bins, a counting sort
 // of the points by magnitude bin (segment starts written to seg), and the
 // points' fold payload written in the sorted order.  The order of points inside
-// a segment is arbitrary; counts do not depend on it.
+// a segment is arbitrary (counts do not depend on it), but that a coarse job's points
+// at the epoch come last (segment_word).
 template <int MODE>
 __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
     __shared__ unsigned long long sh_min[kPrepBlock / 32], sh_max[kPrepBlock / 32];
-    __shared__ int hist[GCE_MAX_MAG_BINS + 1];
+    __shared__ int hist[GCE_MAX_MAG_BINS + 1], zeros[GCE_MAX_MAG_BINS + 1];
     // the first points' magnitudes and bins, each computed once (binary64 arithmetic
     // bounds this kernel: the divisions of the filters' and the bins' normalisation)
     __shared__ double s_m[kPrepMags];
@@ -455,7 +467,7 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
         sh_min[threadIdx.x >> 5] = kmin;
         sh_max[threadIdx.x >> 5] = kmax;
     }
-    for (int i = threadIdx.x; i <= a.n_mag; i += blockDim.x) hist[i] = 0;
+    for (int i = threadIdx.x; i <= a.n_mag; i += blockDim.x) hist[i] = zeros[i] = 0;
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < kPrepBlock / 32; ++w) {
@@ -463,29 +475,32 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
         kmax = sh_max[w] > kmax ? sh_max[w] : kmax;
     }
     const MagBins bins(key_f64(kmin), key_f64(kmax), a.n_mag);
+    const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
+    const bool wide = coarse_mode(MODE) && !coarse_range_ok(a.state);
+    const bool apart = coarse_mode(MODE) && !wide && a.state->epoch;  // points at the epoch come last
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         const int b = bins(k < kPrepMags ? s_m[k] : m[k]);
         if (k < kPrepBins) s_bin[k] = (unsigned char)b;
         atomicAdd(&hist[b], 1);
+        if (apart && at_epoch(t[k], a.t0)) atomicAdd(&zeros[b], 1);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         int run = 0;
         int *seg = a.seg + (long long)c * (a.n_mag + 1);
         for (int i = 0; i < a.n_mag; ++i) {
-            int h = hist[i];
+            const int h = hist[i], z = zeros[i];
             hist[i] = run;
-            seg[i] = run;
+            seg[i] = (int)segment_word(run, z);
             run += h;
+            zeros[i] = run;
         }
         seg[a.n_mag] = run;
     }
     __syncthreads();
-    const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
-    const bool wide = coarse_mode(MODE) && !coarse_range_ok(a.state);
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         const int b = k < kPrepBins ? s_bin[k] : bins(k < kPrepMags ? s_m[k] : m[k]);
-        const int pos = atomicAdd(&hist[b], 1);
+        const int pos = apart && at_epoch(t[k], a.t0) ? atomicAdd(&zeros[b], -1) - 1 : atomicAdd(&hist[b], 1);
         const double tau = __dsub_rn(t[k], a.t0);
         if (coarse_mode(MODE)) a.tau[lo + pos] = tau;
         if (MODE == GCE_PHASE_FP64) {

@@ -73,7 +73,8 @@ typedef enum {
     /* FP32 double-float: tau, tau^2, f and a split into (hi, lo) float pairs,
      * error-free products via fmaf, integer cycles removed with a rounding
      * constant.  Phase error about 1e-7 cycles; needs |tau|/P < 2^21 and
-     * |Pdot| tau^2/(2 P^2) < 2^19 cycles. */
+     * |Pdot| tau^2/(2 P^2) < 2^19 cycles, and tau, 1/P and (with a nonzero Pdot)
+     * tau^2 and Pdot/(2 P^2) within the range of float. */
     GCE_PHASE_SPLIT32 = 1,
     /* fixed point: tau, tau^2, f and a as 64-bit integers split into 32-bit
      * limbs; the phase is the low 32 bits of their products (integer cycles wrap

@@ -118,6 +118,8 @@ __global__ void k_scan(const double *__restrict__ times, const double *__restric
     }
 }
 
+__device__ inline bool beyond_float(double v) { return isinf(__double2float_rn(v)); }
+
 // Per flat trial t = q n_periods + p: f = 1/P, a = (0.5 Pdot) f f (the oracle's
 // sequence), stored in the fold mode's format.  Bound by binary64 arithmetic at 2
 // lanes per clock and SM, so what binary32 holds exactly is done there, and nothing
@@ -142,6 +144,10 @@ __global__ void k_trials(TrialArgs a) {
             if (MODE == GCE_PHASE_SPLIT32) {
                 // |x| < 1 needs |c| + |c2| < 1/2: cycles < 2^21 and Pdot cycles < 2^19
                 bad = tau_max * fmax_ >= 2097152.0 || amax * tau_max * tau_max >= 524288.0;
+                // and every value that a fold reads split into finite floats: an infinite
+                // one makes the residual NaN, whose slot is no counter of the trial's
+                bad = bad || beyond_float(tau_max) || beyond_float(fmax_) ||
+                      (dmax > 0.0 && (beyond_float(amax) || beyond_float(tau_max * tau_max)));
             } else if (MODE == GCE_PHASE_FIXED32 || MODE == kJobFixed32) {
                 bad = !fixed_range_ok(fmax_, amax, fs.e_tau);
             }

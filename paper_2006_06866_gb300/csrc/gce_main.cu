@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(256) k_single(MainArgs a, int c) {
         const int s0 = seg[i], s1 = seg[i + 1];
         if (s1 == s0) continue;
         for (int k = s0; k < s1; ++k) {
-            const int j = fold_fp64<true>(__ldg(pts + k), tr.x, tr.y, (double)n_phase, n_phase);
+            // (a fold that overflows binary64 is NaN and has no bin: bin 0, as in k_main)
+            const int j = max(fold_fp64<true>(__ldg(pts + k), tr.x, tr.y, (double)n_phase, n_phase), 0);
             atomicAdd(cnt + j * B, 1u);
             if (a.overlap) atomicAdd(cnt + (j == 0 ? n_phase - 1 : j - 1) * B, 1u);
         }
@@ -135,6 +136,7 @@ __global__ void k_counts(MainArgs a, long long n_cells, const long long *cell_cu
                           : Fold<MODE>::template raw_slot<false>(pts[k], tr, fk)) -
                     Fold<MODE>::kSlotBias;
             if (j >= a.n_phase) j -= a.n_phase;  // SPLIT32's second slot of a bin
+            j = max(j, 0);                       // FP64's NaN (see k_single)
             out[i * a.n_phase + j] += 1u;
             if (a.overlap) out[i * a.n_phase + (j == 0 ? a.n_phase - 1 : j - 1)] += 1u;
         }

@@ -188,7 +188,7 @@ __device__ inline int mag_bin(double m, double mn, double mx, int n_mag) {
     if (mx == mn) return 0;
     double v = __ddiv_rn(__dsub_rn(m, mn), __dsub_rn(mx, mn));
     int i = __double2int_rd(__dmul_rn(v, (double)n_mag));
-    return min(i, n_mag - 1);
+    return max(min(i, n_mag - 1), 0);  // (a NaN, of flagged input or a range that overflows: bin 0)
 }
 
 // mag_bin, from a binary32 quotient where that decides it: four roundings leave v

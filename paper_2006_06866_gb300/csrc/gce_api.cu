@@ -17,6 +17,7 @@
 
 #include "gce_internal.cuh"
 #include "gce_topk.cuh"
+#include "gce_workspace.h"
 
 using namespace gce;
 
@@ -123,11 +124,6 @@ bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_t
 
 namespace {
 
-struct DevBuf {
-    void *p = nullptr;
-    size_t bytes = 0;
-};
-
 // mode, n_phase, n_mag, log2 bucket of N, Pdot axis (n_pdots > 1: period-major tiles)
 typedef std::tuple<int, int, int, int, int> TuneKey;
 
@@ -169,6 +165,7 @@ struct LaunchShape {
 };
 
 constexpr int kCheckedArrays = 14;
+constexpr int kWorkspaceBuffers = 12;
 
 struct CachedGraph {
     cudaGraphExec_t exec = nullptr;
@@ -224,29 +221,29 @@ static gce_status fail(gce_handle h, gce_status st, const char *fmt, ...) {
             return fail((h), GCE_ERR_CUDA, "%s failed: %s", #expr, cudaGetErrorString(e_)); \
     } while (0)
 
-static gce_status ensure(gce_handle h, DevBuf &b, size_t bytes) {
-    if (bytes <= b.bytes && b.p) return GCE_OK;
-    size_t want = std::max(bytes, (size_t)256);
-    want = std::max(want, b.bytes + b.bytes / 2);
-    if (b.p) {
-        // in-flight work may still read the old buffer
-        CUDA_TRY(h, cudaDeviceSynchronize());
-        CUDA_TRY(h, cudaFree(b.p));
-        b.p = nullptr;
-        b.bytes = 0;
-    }
-    if (cudaMalloc(&b.p, want) != cudaSuccess) {
+static const DevMemory kDevMemory = {
+    [](void **p, size_t bytes) {
+        if (cudaMalloc(p, bytes) == cudaSuccess) return true;
         cudaGetLastError();
-        b.p = nullptr;
-        if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            b.p = nullptr;
-            return fail(h, GCE_ERR_NOMEM, "device allocation of %zu bytes failed", bytes);
-        }
-        want = bytes;
-    }
-    b.bytes = want;
-    return GCE_OK;
+        return false;
+    },
+    [](void *p) { cudaFree(p); },
+    []() { return cudaDeviceSynchronize() == cudaSuccess; },
+    []() {
+        size_t free_bytes = 0, total = 0;
+        if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) cudaGetLastError();
+        return free_bytes;
+    }};
+
+static gce_status growth_status(gce_handle h, Growth g, size_t bytes) {
+    if (g == GROWN) return GCE_OK;
+    if (g == WAIT_FAILED)
+        return fail(h, GCE_ERR_CUDA, "cudaDeviceSynchronize failed: %s", cudaGetErrorString(cudaGetLastError()));
+    return fail(h, GCE_ERR_NOMEM, "device allocation of %zu bytes failed", bytes);
+}
+
+static gce_status ensure(gce_handle h, DevBuf &b, size_t bytes) {
+    return growth_status(h, grow(kDevMemory, b, bytes), bytes);
 }
 
 static int point_bytes(int mode) {
@@ -777,37 +774,40 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
     gce_status st = make_plan(h, j, pl);
     if (st != GCE_OK) return st;
 
-    // workspace
-    if (coarse_mode(pl.prep_mode) &&
-        (ensure(h, h->tau, 8 * (size_t)pl.n_points) != GCE_OK ||
-         ensure(h, h->payload, (size_t)point_bytes(pl.prep_mode) * pl.n_points) != GCE_OK ||
-         ensure(h, h->trialc, trial_bytes(pl.prep_mode) * (size_t)pl.n_trials) != GCE_OK)) {
-        h->last_error.clear();
-        pl.prep_mode = j.cfg->phase_mode;
-    }
+    // workspace (the first three buffers' size depends on the payload's form)
+    const bool new_table = pl.n_max > h->table_n;
+    const size_t nc = (size_t)j.n_curves, lists = nc * (size_t)pl.n_lists;
+    const bool topk = j.kind == JOB_TOPK;
+    auto needs = [&](int mode, Need (&need)[kWorkspaceBuffers]) {
+        const Need all[kWorkspaceBuffers] = {
+            {&h->payload, (size_t)point_bytes(mode) * pl.n_points},
+            {&h->trialc, trial_bytes(mode) * (size_t)pl.n_trials},
+            {&h->tau, coarse_mode(mode) ? 8 * (size_t)pl.n_points : 0},
+            {&h->seg, sizeof(int) * nc * (j.cfg->n_mag_bins + 1)},
+            {&h->order, sizeof(int) * nc},
+            {&h->offsets, sizeof(long long) * (nc + 1)},
+            {&h->band_stats, j.bands ? sizeof(double2) * nc * j.n_bands : 0},
+            {&h->cand, topk ? 8 * lists * j.k : 0},
+            {&h->stats, topk && j.rho ? sizeof(TileStats) * lists * pl.stats_per : 0},
+            {&h->cand2, topk ? 8 * nc * pl.n_groups * j.k : 0},
+            {&h->stats2, topk && j.rho ? sizeof(TileStats) * nc * pl.n_groups : 0},
+            {&h->table, new_table ? 8 * (size_t)(pl.n_max + 1) : 0}};
+        std::copy(all, all + kWorkspaceBuffers, need);
+    };
+    Need coarse[kWorkspaceBuffers], plain[kWorkspaceBuffers];
+    const bool try_coarse = coarse_mode(pl.prep_mode);
+    needs(pl.prep_mode, coarse);
+    needs(try_coarse ? j.cfg->phase_mode : pl.prep_mode, plain);
+    if (new_table) h->table_n = -1;  // (growing loses its contents)
+    bool is_coarse = false;
+    size_t most = 0;
+    for (const Need &x : plain) most = std::max(most, x.bytes);
+    st = growth_status(h, job_buffers(kDevMemory, try_coarse ? coarse : nullptr, plain,
+                                      kWorkspaceBuffers, 3, &is_coarse), most);
+    if (st != GCE_OK) return st;
+    if (try_coarse && !is_coarse) pl.prep_mode = j.cfg->phase_mode;
     const int mode = pl.prep_mode;
-    if ((st = ensure(h, h->payload, (size_t)point_bytes(mode) * pl.n_points)) != GCE_OK) return st;
-    if ((st = ensure(h, h->seg, sizeof(int) * (size_t)j.n_curves * (j.cfg->n_mag_bins + 1))) != GCE_OK) return st;
-    if ((st = ensure(h, h->trialc, trial_bytes(mode) * (size_t)pl.n_trials)) != GCE_OK) return st;
-    if ((st = ensure(h, h->order, sizeof(int) * (size_t)j.n_curves)) != GCE_OK) return st;
-    if ((st = ensure(h, h->offsets, sizeof(long long) * (size_t)(j.n_curves + 1))) != GCE_OK) return st;
-    if (j.bands &&
-        (st = ensure(h, h->band_stats, sizeof(double2) * (size_t)j.n_curves * j.n_bands)) != GCE_OK)
-        return st;
-    if (j.kind == JOB_TOPK &&
-        (st = ensure(h, h->cand, 8 * (size_t)j.n_curves * pl.n_lists * j.k)) != GCE_OK)
-        return st;
-    if (j.kind == JOB_TOPK && j.rho &&
-        (st = ensure(h, h->stats, sizeof(TileStats) * (size_t)j.n_curves * pl.n_lists * pl.stats_per)) != GCE_OK)
-        return st;
-    if (j.kind == JOB_TOPK && pl.n_groups > 0 &&
-        (st = ensure(h, h->cand2, 8 * (size_t)j.n_curves * pl.n_groups * j.k)) != GCE_OK)
-        return st;
-    if (j.kind == JOB_TOPK && pl.n_groups > 0 && j.rho &&
-        (st = ensure(h, h->stats2, sizeof(TileStats) * (size_t)j.n_curves * pl.n_groups)) != GCE_OK)
-        return st;
-    if (pl.n_max > h->table_n) {
-        if ((st = ensure(h, h->table, 8 * (size_t)(pl.n_max + 1))) != GCE_OK) return st;
+    if (new_table) {
         CUDA_TRY(h, launch_table((unsigned long long *)h->table.p, pl.n_max, s));
         ++h->launches;
         if (!captured) h->table_n = pl.n_max;  // (a captured launch has filled nothing yet)

@@ -305,8 +305,11 @@ gce_status gce_kernel_time(gce_handle h, float *ms);
 gce_status gce_last_launches(gce_handle h, int32_t *n);
 
 /* Time candidate launch shapes on a synthetic job of the given size and keep
- * the fastest for (phase mode, bins, curve-length bucket) in the handle's
- * cache; later calls with a matching key use it.  Jobs with a Pdot axis
+ * the fastest for (phase mode, bins, curve-length bucket, size class) in the
+ * handle's cache; later calls with a matching key use it.  The job's own shape,
+ * as an untuned call takes it, is one of the candidates.  The size class tells
+ * jobs of few trials x curves, whose own shape has fewer trials per thread, from
+ * the others (the line: 20 warps of 32 trials per warp scheduler, FP64 24).  Jobs with a Pdot axis
  * (n_pdots > 1, whose tiles pair one period with several Pdot values) are
  * tuned separately on a synthetic job with 8 Pdot values and cached under
  * their own entry.  Synchronous. */
@@ -317,18 +320,23 @@ gce_status gce_autotune(gce_handle h, const gce_config *cfg, int32_t n_obs_hint,
  * the candidate shapes are timed on a bounded slice of it -- a prefix of the
  * curves holding about 4e9 point-trials of the slice, at most 65536 periods and
  * 8 Pdot values, each a strided subset spanning the job's range -- and the
- * fastest is cached under the job's key (phase mode, bins, length bucket of
- * its longest curve, Pdot axis or not), which later calls on that job use.
+ * fastest, or the job's own shape, is cached under the job's key (phase mode,
+ * bins, length bucket of its longest curve, Pdot axis or not, size class), which
+ * later calls on that job use.
  * Synchronous; it allocates and frees a small scratch of its own. */
 gce_status gce_autotune_job(gce_handle h, const double *times, const double *mags,
                             const int64_t *h_offsets, int32_t n_curves, const double *periods,
                             int32_t n_periods, const double *pdots, int32_t n_pdots,
                             const gce_config *cfg);
 
-/* Read the launch shape the handle would use for a job with this config,
- * typical curve length and number of Pdot values (n_pdots_hint >= 1; > 1 means
- * a Pdot axis), or force one (gce_set_tuning replaces the cached choice for
- * that curve-length bucket, for jobs with and without a Pdot axis).
+/* Read the launch shape cached for jobs with this config, typical curve length
+ * and number of Pdot values (n_pdots_hint >= 1; > 1 means a Pdot axis), or force
+ * one (gce_set_tuning replaces the cached choice for that curve-length bucket,
+ * for jobs of every size, with and without a Pdot axis).  Where none is cached, or
+ * the tuner kept the jobs' own, it is the shape that their own is fitted from: the
+ * call still takes fewer trials per thread, or lets a CTA's warps share a set of
+ * them, in small jobs, and four trials per thread in large FP64 ones (a gce_tuning
+ * holds at most two there), so setting back what was read may run slower.
  * GCE_ERR_INVALID for n_pdots_hint < 1 or, from gce_set_tuning, for shapes
  * outside the documented ranges. */
 gce_status gce_get_tuning(gce_handle h, const gce_config *cfg, int32_t n_obs_hint,

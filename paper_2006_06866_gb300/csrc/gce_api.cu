@@ -69,6 +69,14 @@ gce_tuning default_tuning(const gce_config *cfg, int n_pdots) {
     return t;
 }
 
+// Jobs of so few warps (with one trial per thread) that fit_to_job leaves the default
+// shape.  A tuned shape serves jobs of its own class: one tuned on a survey batch costs a
+// single curve what its own shape gains (2000 points x 1000 periods, SPLIT32, the CE
+// kernel: 0.088 ms with a batch's 128 x 4, 0.022 with its own), and the other way round.
+static bool small_job(int mode, long long n_trials, int n_curves, int n_sm) {
+    return (n_trials + 31) / 32 * n_curves <= (mode == GCE_PHASE_FP64 ? 24 : 20) * 4ll * n_sm;
+}
+
 // Fewer trials per thread where the job's trials would not fill the device
 // otherwise.  w: warps per scheduler with one trial per thread.  SM cycles per warp
 // and point-trial of 300-point curves, SPLIT32 at 1 / 2 / 4 trials per thread: w =
@@ -111,7 +119,7 @@ bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_t
         fixed.phase_mode = GCE_PHASE_FIXED32;
         t.tpt = default_tuning(&fixed, n_pdots).tpt;
     }
-    if (warps <= (mode == GCE_PHASE_FP64 ? 24 : 20) * schedulers) t.tpt = std::min(t.tpt, 2);
+    if (small_job(mode, n_trials, n_curves, n_sm)) t.tpt = std::min(t.tpt, 2);
     if (few && !stats) t.tpt = 1;
     if (keep2) {
         t.tpt = std::max(t.tpt, 2);
@@ -124,8 +132,14 @@ bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_t
 
 namespace {
 
-// mode, n_phase, n_mag, log2 bucket of N, Pdot axis (n_pdots > 1: period-major tiles)
-typedef std::tuple<int, int, int, int, int> TuneKey;
+// mode, n_phase, n_mag, log2 bucket of N, Pdot axis (n_pdots > 1: period-major tiles),
+// size class (small_job)
+typedef std::tuple<int, int, int, int, int, int> TuneKey;
+// own: the tuner found the job's own shape the fastest (default_tuning, fit_to_job)
+struct Tuned {
+    gce_tuning t;
+    bool own;
+};
 
 enum JobKind { JOB_GRID = 0, JOB_TOPK = 1, JOB_SINGLE = 2, JOB_COUNTS = 3 };
 
@@ -195,7 +209,7 @@ struct gce_handle_s {
     cudaEvent_t k0 = nullptr, k1 = nullptr;  // around the CE kernel (GCE_FLAG_TIME_KERNEL)
     bool timed = false;
     int launches = 0;                    // kernels the last job launched (directly or in its graph)
-    std::map<TuneKey, gce_tuning> tune;
+    std::map<TuneKey, Tuned> tune;
     std::map<GraphKey, CachedGraph> graphs;
     std::map<ShapeKey, LaunchShape> shapes;  // launch shapes already fitted to the device
     const void *checked[kCheckedArrays] = {};  // arrays of the last call found on the device
@@ -272,22 +286,20 @@ static bool tuning_ok(const gce_tuning &t, int mode) {
            (t.slot_range == 0 || t.slot_range == 1);
 }
 
-static TuneKey tune_key(const gce_config *cfg, int n_obs, int pd_axis) {
+static TuneKey tune_key(const gce_config *cfg, int n_obs, int pd_axis, bool small) {
     return TuneKey(cfg->phase_mode, cfg->n_phase_bins, cfg->n_mag_bins,
-                   ilog2_ceil(std::max(n_obs, 1)), pd_axis);
+                   ilog2_ceil(std::max(n_obs, 1)), pd_axis, small ? 1 : 0);
 }
 
 // The cached shape for the key (a Pdot-axis job without its own entry uses the
 // plain one), or the default one (*tuned = false).
 static gce_tuning lookup_tuning(gce_handle h, const gce_config *cfg, int n_max, int n_pdots,
-                                bool *tuned = nullptr) {
+                                bool small, bool *tuned) {
     const int pd_axis = n_pdots > 1 ? 1 : 0;
-    if (tuned) *tuned = true;
-    auto it = h->tune.find(tune_key(cfg, n_max, pd_axis));
-    if (it == h->tune.end() && pd_axis) it = h->tune.find(tune_key(cfg, n_max, 0));
-    if (it != h->tune.end()) return it->second;
-    if (tuned) *tuned = false;
-    return default_tuning(cfg, n_pdots);
+    auto it = h->tune.find(tune_key(cfg, n_max, pd_axis, small));
+    if (it == h->tune.end() && pd_axis) it = h->tune.find(tune_key(cfg, n_max, 0, small));
+    *tuned = it != h->tune.end() && !it->second.own;
+    return *tuned ? it->second.t : default_tuning(cfg, n_pdots);
 }
 
 extern "C" const char *gce_status_string(gce_status s) {
@@ -401,6 +413,7 @@ struct Job {
     const int64_t *cell_curve, *cell_trial;
     uint32_t *counts;
     const gce_tuning *force;     // tuning override (autotuner)
+    bool own;                    // the job's own shape, whatever is cached (autotuner)
     const unsigned char *bands;  // multi-filter input (nullptr: one filter, raw magnitudes)
     int n_bands;
 };
@@ -500,7 +513,12 @@ gce_status make_plan(gce_handle h, const Job &j, Plan &pl) {
     for (int c = 0; c < j.n_curves; ++c) nmax = std::max<long long>(nmax, j.h_offsets[c + 1] - j.h_offsets[c]);
     pl.n_max = (int)nmax;
     bool tuned = true;
-    gce_tuning t = j.force ? *j.force : lookup_tuning(h, cfg, pl.n_max, j.n_pdots, &tuned);
+    gce_tuning t;
+    if (j.force) t = *j.force;
+    else if (j.own) t = default_tuning(cfg, j.n_pdots), tuned = false;
+    else
+        t = lookup_tuning(h, cfg, pl.n_max, j.n_pdots,
+                          small_job(cfg->phase_mode, pl.n_trials, j.n_curves, h->n_sm), &tuned);
     const bool shared_set = !tuned && fit_to_job(t, cfg, j.n_pdots, pl.n_trials, j.n_curves,
                                                  pl.n_points, h->n_sm, j.rho != nullptr);
     pl.range = split_range(cfg->phase_mode, j.n_pdots, t.slot_range);
@@ -1124,15 +1142,19 @@ extern "C" gce_status gce_last_launches(gce_handle h, int32_t *n) {
 extern "C" gce_status gce_get_tuning(gce_handle h, const gce_config *cfg, int32_t n_obs_hint,
                                      int32_t n_pdots_hint, gce_tuning *t) {
     if (!h || !cfg || !t || n_pdots_hint < 1) return GCE_ERR_INVALID;
-    *t = lookup_tuning(h, cfg, std::max(1, n_obs_hint), n_pdots_hint);
+    // a large job's shape, or a small one's where only that is cached
+    bool tuned = false;
+    *t = lookup_tuning(h, cfg, std::max(1, n_obs_hint), n_pdots_hint, false, &tuned);
+    if (!tuned) *t = lookup_tuning(h, cfg, std::max(1, n_obs_hint), n_pdots_hint, true, &tuned);
     return GCE_OK;
 }
 
 extern "C" gce_status gce_set_tuning(gce_handle h, const gce_config *cfg, int32_t n_obs_hint,
                                      const gce_tuning *t) {
     if (!h || !cfg || !t || !tuning_ok(*t, cfg->phase_mode)) return GCE_ERR_INVALID;
-    h->tune[tune_key(cfg, std::max(1, n_obs_hint), 0)] = *t;
-    h->tune[tune_key(cfg, std::max(1, n_obs_hint), 1)] = *t;
+    for (int pd_axis = 0; pd_axis < 2; ++pd_axis)
+        for (bool small : {false, true})
+            h->tune[tune_key(cfg, std::max(1, n_obs_hint), pd_axis, small)] = Tuned{*t, false};
     return GCE_OK;
 }
 
@@ -1161,14 +1183,17 @@ static std::vector<gce_tuning> tune_candidates(int mode, int n_obs, int slot_ran
 // Times every candidate on job j (one untimed run, then three timed ones), then
 // times the three fastest again over six runs each and leaves the fastest of
 // those in *best (a second look keeps close calls from being decided by one
-// noisy measurement); shapes that do not fit are skipped.  also_wide: each of
+// noisy measurement), or the job's own shape where that is faster still (it has
+// forms that a gce_tuning has not: warps that share a trial set, four trials per
+// thread for FP64); shapes that do not fit are skipped.  also_wide: each of
 // the three is timed with the wide slot range too (the candidates keep the mid
 // one, whose re-reduced warps can make it the slower on long baselines).
 static gce_status time_candidates(gce_handle h, Job j, const std::vector<gce_tuning> &cands,
                                   cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1,
-                                  gce_tuning *best, bool also_wide = false) {
-    auto timed = [&](const gce_tuning &cand, int reps, float *ms) -> gce_status {
-        j.force = &cand;
+                                  Tuned *best, bool also_wide = false) {
+    auto timed = [&](const gce_tuning *cand, int reps, float *ms) -> gce_status {
+        j.force = cand;
+        j.own = !cand;
         *ms = 1e30f;
         if (run_job(h, j, s) != GCE_OK) return GCE_OK;  // does not fit: stays 1e30
         cudaEventRecord(e0, s);
@@ -1183,7 +1208,7 @@ static gce_status time_candidates(gce_handle h, Job j, const std::vector<gce_tun
     std::vector<std::pair<float, size_t>> first;
     for (size_t i = 0; i < cands.size(); ++i) {
         float ms;
-        if (gce_status st = timed(cands[i], 3, &ms)) return st;
+        if (gce_status st = timed(&cands[i], 3, &ms)) return st;
         if (ms < 1e30f) first.emplace_back(ms, i);
     }
     if (first.empty()) return GCE_OK;
@@ -1194,13 +1219,16 @@ static gce_status time_candidates(gce_handle h, Job j, const std::vector<gce_tun
             gce_tuning c = cands[first[r].second];
             if (w) c.slot_range = 0;
             float ms;
-            if (gce_status st = timed(c, 6, &ms)) return st;
+            if (gce_status st = timed(&c, 6, &ms)) return st;
             if (ms < best_ms) {
                 best_ms = ms;
-                *best = c;
+                *best = Tuned{c, false};
             }
         }
     }
+    float ms;
+    if (gce_status st = timed(nullptr, 6, &ms)) return st;
+    if (ms < best_ms) best->own = true;
     return GCE_OK;
 }
 
@@ -1235,7 +1263,7 @@ extern "C" gce_status gce_autotune_job(gce_handle h, const double *times, const 
     cudaStream_t s = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     gce_status result = GCE_OK;
-    gce_tuning best = default_tuning(cfg, n_pdots);
+    Tuned best{default_tuning(cfg, n_pdots), true};
     gce_config c2cfg = *cfg;
     c2cfg.flags = (c2cfg.flags | GCE_FLAG_NO_GRAPH) & ~GCE_FLAG_TIME_KERNEL;
     do {
@@ -1268,7 +1296,9 @@ extern "C" gce_status gce_autotune_job(gce_handle h, const double *times, const 
     if (e1) cudaEventDestroy(e1);
     if (s) cudaStreamDestroy(s);
     cudaFree(d_p); cudaFree(d_q); cudaFree(d_H); cudaFree(d_I);
-    if (result == GCE_OK) h->tune[tune_key(cfg, (int)nmax, n_pdots > 1 ? 1 : 0)] = best;
+    if (result == GCE_OK)
+        h->tune[tune_key(cfg, (int)nmax, n_pdots > 1 ? 1 : 0,
+                         small_job(cfg->phase_mode, (long long)n_periods * n_pdots, n_curves, h->n_sm))] = best;
     return result;
 }
 
@@ -1310,7 +1340,7 @@ extern "C" gce_status gce_autotune(gce_handle h, const gce_config *cfg, int32_t 
     cudaStream_t s = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     gce_status result = GCE_OK;
-    gce_tuning best[2] = {default_tuning(cfg, 1), default_tuning(cfg, 8)};
+    Tuned best[2] = {{default_tuning(cfg, 1), true}, {default_tuning(cfg, 8), true}};
     gce_config c2 = *cfg;
     c2.flags |= GCE_FLAG_NO_GRAPH;
     do {
@@ -1348,8 +1378,9 @@ extern "C" gce_status gce_autotune(gce_handle h, const gce_config *cfg, int32_t 
     if (s) cudaStreamDestroy(s);
     cudaFree(d_t); cudaFree(d_m); cudaFree(d_p); cudaFree(d_pp); cudaFree(d_d); cudaFree(d_out);
     if (result == GCE_OK) {
-        h->tune[tune_key(cfg, n_obs, 0)] = best[0];
-        h->tune[tune_key(cfg, n_obs, 1)] = best[1];
+        const int mode = cfg->phase_mode;
+        h->tune[tune_key(cfg, n_obs, 0, small_job(mode, n_tr, n_curves, h->n_sm))] = best[0];
+        h->tune[tune_key(cfg, n_obs, 1, small_job(mode, n_trp * n_pd, n_curves, h->n_sm))] = best[1];
     }
     return result;
 }

@@ -834,7 +834,9 @@ bool fit_to_job(gce_tuning &t, const gce_config *cfg, int n_pdots, long long n_t
 // and its writes are visible.  Every kernel that launch_pdl starts calls it before it
 // touches what an earlier kernel writes (so completion is transitive), and
 // pdl_trigger() lets the next one be scheduled.  The first kernel of a call is
-// launched normally, after all of the caller's work.  Not under stream capture.
+// launched normally, after all of the caller's work.  Not under stream capture.  Only the
+// caller's arrays are `const __restrict__` in these kernels: the workspace is written
+// during a dependent kernel's lifetime.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 template <class... P, class... A>

@@ -16,7 +16,7 @@ constexpr int kMergeKeys = 16;  // keys a merging thread holds in registers
 // significance of Eq. 5 from the moment records.  Latency-bound (one CTA per curve):
 // up to 4096 keys are read once, into registers, and a round is one barrier.
 __global__ void __launch_bounds__(kMergeBlock)
-    k_topk_merge(const unsigned long long *__restrict__ cand, int n_tiles, int k, int stats_per,
+    k_topk_merge(const unsigned long long *cand, int n_tiles, int k, int stats_per,
                  float *topk_H, long long *topk_idx, const TileStats *stats, double *mean_out,
                  double *std_out, float *rho_out, const JobState *st) {
     constexpr int WARPS = kMergeBlock / 32;

@@ -350,7 +350,7 @@ __device__ double2 warp_band_stats(double *v, int cnt, unsigned int *hist) {
 // memory filter by filter, 58 us now).
 __global__ void __launch_bounds__(256) k_band_stats(const double *__restrict__ mags,
                                                     const unsigned char *__restrict__ bands,
-                                                    const long long *__restrict__ offsets,
+                                                    const long long *offsets,
                                                     int n_bands, double2 *stats, JobState *st) {
     __shared__ unsigned int hist[GCE_MAX_BANDS][256];
     __shared__ double vals[kBandCurve];

@@ -26,10 +26,10 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
 }
 
 __global__ void __launch_bounds__(kReduceBlock)
-    k_topk_reduce(const unsigned long long *__restrict__ cand, int n_tiles, int k,
+    k_topk_reduce(const unsigned long long *cand, int n_tiles, int k,
                   int tiles_per_group, int n_groups, int stats_per,
-                  const TileStats *__restrict__ stats,
-                  unsigned long long *__restrict__ cand2, TileStats *__restrict__ stats2,
+                  const TileStats *stats,
+                  unsigned long long *cand2, TileStats *stats2,
                   const JobState *st) {
     __shared__ unsigned long long s_keys[kReduceKeys];
     __shared__ unsigned long long s_warp[kReduceBlock / 32];

@@ -463,11 +463,11 @@ gce_status fit_shape(gce_handle h, const gce_config *cfg, const Plan &pl, const 
     };
     ls.smem = size();
     while (ls.smem > limit()) {
-        if (ls.chunk > 512) ls.chunk /= 2;
+        if (ls.chunk > 512) ls.chunk = half_chunk(ls.chunk);
         else if (ls.table_smem > 256) ls.table_smem /= 2;
         else if (ls.tpt > 1) ls.tpt /= 2;
         else if (ls.block > 64) ls.block /= 2;
-        else if (ls.chunk > 64) ls.chunk /= 2;
+        else if (ls.chunk > 64) ls.chunk = half_chunk(ls.chunk);
         else break;
         ls.smem = size();
     }
@@ -485,7 +485,7 @@ gce_status fit_shape(gce_handle h, const gce_config *cfg, const Plan &pl, const 
     int best_chunk = ls.chunk;
     size_t best_smem = ls.smem;
     for (int c = ls.chunk; c > 256;) {
-        c = std::max(256, (c / 2 + 31) / 32 * 32);
+        c = std::max(256, half_chunk(c));
         ls.chunk = c;
         const size_t sm2 = size();
         int occ2 = 0;

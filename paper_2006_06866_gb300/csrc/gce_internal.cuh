@@ -582,10 +582,12 @@ __host__ __device__ inline int slots_per_trial(int mode, int n_phase, int range)
 // Byte offsets of the CE kernel's dynamic shared-memory regions, in order: the
 // c ln c table (an even number of 8-byte entries, so the points after it stay
 // 16-byte aligned), the staged points (8 bytes each for FP64 and for half
-// points, else 16; the coarse fold's 12 and 24; chunk is a multiple of 32), the counters and the segment
-// starts.  The host sizes the launch with `total` and the kernel carves its
+// points, else 16; the coarse fold's 12 and 24), the counters and the segment
+// starts.  chunk is even, so that the words of the staged pairs lie on 16 bytes (a
+// multiple of 32, but in the static entry's last resort a multiple of 8).  The host sizes the launch with `total` and the kernel carves its
 // memory with the same offsets.  (k and block do not enter: each warp writes its
 // top-k keys and moments straight to global memory.)
+inline int half_chunk(int chunk) { return (chunk / 2 + 31) / 32 * 32; }
 struct MainSmemLayout {
     unsigned int pts, cnt, seg, total;
 };

@@ -232,10 +232,20 @@ PARITY_TOL = {"fp64": 1e-6, "split32": 1e-4, "fixed32": 1e-4}
 PARITY_EPS = {"fp64": 0.0, "split32": 2.5e-7, "fixed32": 4e-9}
 
 
+def entropy_of(counts):
+    """H of Eq. 4 per cell from 2-D counts [cells, n_mag, n_phase] (float64)."""
+    c = counts.astype(np.float64)
+    ent = lambda x: np.where(x > 1, x * np.log(np.maximum(x, 1)), 0.0)
+    return (ent(c.sum(1)).sum(1) - ent(c).sum((1, 2))) / c.sum((1, 2))
+
+
 def parity_block(g, h, dev, stream, sample, ref, dmin, overlap, n_count_cells=2000):
     """Per fold: CE error and argmin agreement of the device grid against the
-    oracle grid of the CPU-baseline sample, and exact-count agreement on seeded
-    sampled cells (gce_ce_counts against the oracle's counts)."""
+    oracle grid of the CPU-baseline sample; exact-count agreement on seeded sampled
+    cells (gce_ce_counts, the mode's own fold, against the oracle's counts); and the
+    searched fold against its own: the grid's sampled cells against the entropy of
+    those counts, and every cell of the FP64 grid bit for bit against the
+    one-launch-per-curve kernel, which runs the binary64 fold on every point."""
     import torch
     nc = sample.n_curves
     flat, dm = ref.reshape(nc, -1), dmin.reshape(nc, -1)
@@ -268,8 +278,17 @@ def parity_block(g, h, dev, stream, sample, ref, dmin, overlap, n_count_cells=20
             if g.gce_stream_status(h, stream) != g.GCE_OK:
                 out[mode] = {"error": "device input check failed"}
                 continue
+            search_ok = True
+            search = {}
+            if mode == "fp64":
+                one = g.gce_ce_grid_single(h, cfg=cfg, stream=stream, **args)
+                search["grid_cells_unlike_single"] = int((got != one).sum())
+                search_ok = search["grid_cells_unlike_single"] == 0
+                del one
             got = got.cpu().numpy().astype(np.float64).reshape(nc, -1)
             cnt = cnt.cpu().numpy().astype(np.int64)
+            search["max_abs_dH_of_counts"] = float(np.abs(got[cc, ct] - entropy_of(cnt)).max())
+            search_ok = search_ok and search["max_abs_dH_of_counts"] <= 3e-7
             err = np.abs(got - flat)
             near = dm <= 4 * PARITY_EPS[mode]
             agree = ambiguous = 0
@@ -291,7 +310,9 @@ def parity_block(g, h, dev, stream, sample, ref, dmin, overlap, n_count_cells=20
                 "argmin_tie_ambiguous": ambiguous,
                 "counts_exact": int(same.sum()), "counts_exact_off_edge": int(same[cfar].sum()),
                 "count_cells_off_edge": int(cfar.sum()),
-                "pass": bool(err[~near].max() <= PARITY_TOL[mode] if (~near).any() else True)
+                **search,
+                "pass": search_ok
+                and bool(err[~near].max() <= PARITY_TOL[mode] if (~near).any() else True)
                 and agree == nc - ambiguous
                 and (mode != "fp64" or bool(same.all())),
             }

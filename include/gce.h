@@ -275,7 +275,10 @@ gce_status gce_ce_grid_single(gce_handle h, const double *times, const double *m
                               void *stream);
 
 /* Diagnostic: the full 2-D histogram of selected cells, computed with the same
- * fold and binning device code as the batched kernel for cfg->phase_mode.
+ * magnitude bins as the batched kernel and with cfg->phase_mode's own fold on every
+ * point.  (SPLIT32 searches run that fold too; FP64 and FIXED32 ones decide most
+ * points by a coarser one that has to agree with it, so comparing a grid with the
+ * entropy of these counts checks the search.)
  * cell_curve / cell_trial: device int64[n_cells] (curve index, flat trial
  * index).  counts: device uint32[n_cells][n_mag_bins][n_phase_bins]. */
 gce_status gce_ce_counts(gce_handle h, const double *times, const double *mags,

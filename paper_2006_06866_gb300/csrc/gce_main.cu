@@ -113,7 +113,8 @@ __global__ void __launch_bounds__(256) k_single(MainArgs a, int c) {
             __dmul_rn(__ll2double_rn(d), kTabInvScale / (double)(n * (a.overlap ? 2 : 1))));
 }
 
-// Diagnostic: full 2-D counts of selected cells through the same fold code.
+// Diagnostic: full 2-D counts of selected cells, the mode's own fold on every point (FP64
+// and FIXED32 searches run the coarse fold, which is checked against these).
 template <int MODE>
 __global__ void k_counts(MainArgs a, long long n_cells, const long long *cell_curve,
                          const long long *cell_trial, unsigned int *counts) {

@@ -33,11 +33,10 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
-#include <map>
 #include <mutex>
-#include <utility>
 
 #include "gce_internal.cuh"
+#include "gce_occ_cache.h"
 
 using namespace gce;
 
@@ -51,8 +50,7 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 struct DeviceSetup {
     bool done = false;
-    // CTAs per SM of the launch shapes used so far (0: does not fit)
-    std::map<std::pair<const void *, size_t>, int> occ;
+    OccCache occ;  // CTAs per SM of the last launch shapes (0: does not fit)
     unsigned char *base = nullptr;  // device address of g_scratch
     int n_sm = 0;
     int smem_optin = 0;
@@ -127,18 +125,16 @@ gce_status setup(int dev, DeviceSetup *&out) {
 // the driver the first time.
 int fitted(DeviceSetup *d, const void *kern, int kmode, int tpt, int block, int kv, size_t smem) {
     std::lock_guard<std::mutex> lock(g_mutex);
-    const auto key = std::make_pair(kern, smem);
-    const auto it = d->occ.find(key);
-    if (it != d->occ.end()) return it->second;
     int occ = 0;
+    if (d->occ.find(kern, smem, &occ)) return occ;
     if (!kern || smem > main_dynamic_smem_limit(kmode, tpt, block, kv, (size_t)d->smem_optin) ||
         main_kernel_attrs(kmode, tpt, block, kv, (size_t)d->smem_optin) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess) {
         cudaGetLastError();
         occ = 0;
     }
-    if (d->occ.size() >= 256) d->occ.clear();
-    return d->occ[key] = occ;
+    d->occ.put(kern, smem, occ);
+    return occ;
 }
 
 // A device array of the call must be on the current device: memory that the

@@ -32,20 +32,22 @@ sys.path.insert(0, ROOT)
 METRIC = "folded point-trials/s (N_obs×N_P×N_Ṗ) on 1 GB300; FP64 vs split-FP32 phase"
 UNIT = "point-trials/s"
 # Roofline of k_main.  The peak is instruction issue, 4 schedulers x 32 lanes =
-# 128 thread-instructions per clock per SM, and the algorithmic work is the
-# instructions a scalar thread-per-trial fold cannot avoid per point-trial -- the
-# fold's arithmetic, one slot address and one shared-memory increment:
+# 128 thread-instructions per clock per SM, and the algorithmic work is the issue
+# slots that the fold cannot do without per point-trial: its arithmetic, one slot
+# address and one shared-memory increment (not the point loads and the entropy
+# sweeps, so the fraction stays below the issue rate that ncu measures):
 #   split32: 6 FP32 operations (rounding FMA, subtract, residual FMA, two cross
-#            FMAs, bin FMA); with Pdot 15 (the Pdot product reduced the same
-#            way, two more cross FMAs, the sum reduced once more).  The kernel
-#            folds two points per packed instruction, so the fraction is of
-#            equivalent scalar work;
+#            FMAs, bin FMA), two points per packed instruction, so 3 slots; with Pdot
+#            10 (the Pdot product reduced the same way, two more cross FMAs, the sum
+#            reduced once more, the bin) and the 5 of the period part, which four
+#            trials of a thread share: 5.625;
 #   fixed32, fp64: multiply-add, two cross FMAs, shift-add, bin multiply; with
-#            Pdot 8 (one more multiply-add, two more cross FMAs).  FP64 counts are
-#            those of the binary64 sequence, which runs on the points near a bin
-#            edge only.
+#            Pdot 5 (multiply-add, two cross FMAs, shift-add, bin multiply) and the 3
+#            of the period part shared: 5.75.  FP64 counts are those of the binary64
+#            sequence, which runs on the points near a bin edge only.
 # Measured (ncu): issue slots 65..70 % busy, the shared-memory pipe 59..72 %.
-FOLD_OPS = {"split32": (6, 15), "fixed32": (5, 8), "fp64": (5, 8)}
+FOLD_SLOTS = {"split32": (3, 5.625), "fixed32": (5, 5.75), "fp64": (5, 5.75)}
+FOLD_FP32 = {"split32": (6, 11.25)}
 ISSUE_LANES = 128
 FP32_LANES = 128
 
@@ -79,7 +81,7 @@ def parse():
                          "32, 128 and 512; 0 = the workload's)")
     ap.add_argument("--shape", default="",
                     help="block,tpt,chunk[,slot_range]: fixed launch shape instead of autotuning "
-                         "(profiling runs)")
+                         "(profiling runs); own: the job's own shape, untuned")
     return ap.parse_args()
 
 
@@ -496,7 +498,9 @@ def main():
     def timed_steps(mode, warmup, steps, with_kernel=False):
         if mode not in tuned:  # launch-shape autotuning is part of the untimed warm-up
             cfg = g.Config(batch.n_phase, batch.n_mag, mode, t0=batch.t0, overlap=ovl)
-            if args.shape:
+            if args.shape == "own":
+                pass
+            elif args.shape:
                 sh = [int(x) for x in args.shape.split(",")]
                 g.gce_set_tuning(h, cfg, int(batch.n_obs.max()), block=sh[0], tpt=sh[1], chunk=sh[2],
                                  slot_range=sh[3] if len(sh) > 3 else 0)
@@ -649,7 +653,7 @@ def main():
     roof = None
     if kern_ms:
         has_pdot = bool(np.any(batch.pdots != 0.0))
-        fold = FOLD_OPS[args.mode][1 if has_pdot else 0]
+        pd = 1 if has_pdot else 0
         rate = pt_step / (kern_ms / 1e3)
         # the peak's SM count and maximum SM clock are the device's own: the SM
         # count from the device properties, the clock from the sampler (the
@@ -657,11 +661,11 @@ def main():
         n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
         sm_max = clocks.get("sm_max_mhz") or query_max_sm_mhz(local)
         clk = n_sm * sm_max * 1e6
-        ops, lanes = fold + 2, ISSUE_LANES
+        ops, lanes = FOLD_SLOTS[args.mode][pd] + 2, ISSUE_LANES
         pipe = "issue slots (fold arithmetic + slot address + shared increment)"
         achieved = ops * rate / 1e9
         peak = lanes * clk / 1e9
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gop/s",
+        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "G issue slots/s",
                 "frac": achieved / peak,
                 "traffic": profiled_traffic(args.mode, args.workload, batch.n_curves),
                 "kernel": "k_main", "kernel_ms": kern_ms, "kernel_point_trials_per_s": rate,
@@ -671,9 +675,9 @@ def main():
                 "sm_count_from": "torch.cuda.get_device_properties().multi_processor_count",
                 "sm_max_mhz_from": "nvidia-smi clocks.max.sm, sampled during the timed steps"
                 if clocks.get("sm_max_mhz") else "nvidia-smi clocks.max.sm, queried once",
-                "ops_per_point_trial": ops}
-        if args.mode == "split32":
-            roof["fp32_pipe_frac"] = fold * rate / (FP32_LANES * clk)
+                "issue_slots_per_point_trial": ops}
+        if args.mode in FOLD_FP32:
+            roof["fp32_pipe_frac"] = FOLD_FP32[args.mode][pd] * rate / (FP32_LANES * clk)
 
     if rank == 0:
         line = {

@@ -4,6 +4,7 @@
 // (Eq. 4).  Nothing here is part of the C ABI.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -21,13 +22,21 @@ struct JobState {
     unsigned long long pmin_bits;       // min period as binary64 bits
     unsigned long long pdot_max_bits;   // max |Pdot| as binary64 bits
     unsigned long long work;            // next work item (persistent kernel)
+    // (err, wide and epoch in one 16-byte load: a load of its own for each puts half a
+    // microsecond more before the first work of a small call's kernels)
     unsigned int err;                   // ERR_* bits
     // FP64 and FIXED32 jobs prepared for the coarse fold: 1 when the job's range is
-    // beyond it, so that the mode's own fold runs on every point (set by k_trials)
+    // beyond it, so that the mode's own fold runs on every point (set by k_trials,
+    // read by the kernels after it)
     unsigned int wide;
     unsigned int epoch;                 // 1 when some point has tau = 0
     unsigned int pad;
 };
+static_assert(offsetof(JobState, err) == 32 && sizeof(JobState) == 48, "job_flags' layout");
+// {err, wide, epoch, 0}; the state's buffer is aligned
+__device__ __forceinline__ uint4 job_flags(const JobState *st) {
+    return *reinterpret_cast<const uint4 *>(&st->err);
+}
 
 enum : unsigned int {
     ERR_TIME = 1u,      // non-finite time or magnitude

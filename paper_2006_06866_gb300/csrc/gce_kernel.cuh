@@ -1324,16 +1324,17 @@ __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k
     __shared__ long long s_item;
     pdl_trigger();
     pdl_wait();
-    if (a.state->err) return;  // inputs failed the device checks: no work
+    const uint4 flags = job_flags(a.state);
+    if (flags.x) return;  // inputs failed the device checks: no work
     if constexpr (coarse_mode(MODE)) {
-        if (a.plain || a.state->wide) {
+        if (a.plain || flags.y) {
             ce_items<MODE == kJobFp64 ? GCE_PHASE_FP64 : GCE_PHASE_FIXED32, MODE, TPT, LOG2B, KV, false>(a, s_item);
             return;
         }
         // (the code for points at the epoch apart from the code without: in one, its few
         // instructions per segment cost 100 curves of 200..1000 points x 5e4 x 16 Pdot at
         // 20 bins 1.0 to 1.7 %)
-        if (a.state->epoch) {
+        if (flags.z) {
             ce_items<MODE, MODE, TPT, LOG2B, KV, true>(a, s_item);
             return;
         }

@@ -456,6 +456,12 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
     const int c = blockIdx.x;
     const long long lo = a.offsets[c];
     const int n = (int)(a.offsets[c + 1] - lo);
+    // (the state first: its loads run beside the magnitudes', and k_trials, which is over,
+    // has taken the binary64 division that decides wide)
+    const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
+    const uint4 flags = job_flags(a.state);
+    const bool wide = coarse_mode(MODE) && flags.y;
+    const bool apart = coarse_mode(MODE) && !wide && flags.z;  // points at the epoch come last
     const MagView m{a.mags + lo, a.bands ? a.bands + lo : nullptr,
                     a.bands ? a.band_stats + (long long)c * a.n_bands : nullptr, a.n_bands};
     const double *t = a.times + lo;
@@ -481,9 +487,6 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
         kmax = sh_max[w] > kmax ? sh_max[w] : kmax;
     }
     const MagBins bins(key_f64(kmin), key_f64(kmax), a.n_mag);
-    const FixedScale fs = fixed_scale_from(__longlong_as_double((long long)a.state->tau_max_bits));
-    const bool wide = coarse_mode(MODE) && !coarse_range_ok(a.state);
-    const bool apart = coarse_mode(MODE) && !wide && a.state->epoch;  // points at the epoch come last
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         const int b = bins(k < kPrepMags ? s_m[k] : m[k]);
         if (k < kPrepBins) s_bin[k] = (unsigned char)b;
@@ -495,11 +498,11 @@ __global__ void __launch_bounds__(kPrepBlock) k_prep(PrepArgs a) {
         int run = 0;
         int *seg = a.seg + (long long)c * (a.n_mag + 1);
         for (int i = 0; i < a.n_mag; ++i) {
-            const int h = hist[i], z = zeros[i];
+            const int h = hist[i], z = apart ? zeros[i] : 0;
             hist[i] = run;
             seg[i] = (int)segment_word(run, z);
             run += h;
-            zeros[i] = run;
+            if (apart) zeros[i] = run;
         }
         seg[a.n_mag] = run;
     }

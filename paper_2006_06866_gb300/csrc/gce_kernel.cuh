@@ -886,9 +886,10 @@ __device__ __forceinline__ void split_slot_window(bool pdot, float cyc_max, int 
 }
 
 // CTAs per SM the register allocation is sized for.  With two trials per
-// thread the counters (and FP64's wider staged points) already limit shared
-// memory to about three 256-thread CTAs per SM at 15 phase bins, so those
-// kernels take the registers that frees (80 at 256 threads) instead of 64.
+// thread the counters already limit shared memory to about three 256-thread
+// CTAs per SM at 15 phase bins, so those kernels take the registers that frees
+// (80 at 128 and 256 threads) instead of 64; the coarse fold's two-trial ones
+// spill there, what their own shape (four trials) does not reach.
 // Four trials per thread need four times the counters of one: at most 512
 // threads per SM fit, and those kernels take up to 128 registers.  One trial
 // per thread is the shape for many phase bins (50 and up), where the counters
@@ -1318,7 +1319,8 @@ __device__ __forceinline__ void ce_items(const MainArgs &a, long long &s_item) {
 // point-trial (three with Pdot; 300 curves x 300..900 points x 2e4 periods 1.54 ms, 20
 // x 200..1000 x 5e4 x 16 Pdot 4.49 ms).  The coarse fold has one: 0.80, 0.87, 1.42 and
 // 4.09 ms, of which keeping the distance to the edges takes a tenth.  Bound by issue
-// (nine instructions per point-trial) and latency at 16 to 24 warps per SM.
+// (ten to eleven instructions per point-trial, the sweeps' included) and latency at 16
+// to 24 warps per SM.
 template <int MODE, int TPT, int LOG2B, int KV>
 __global__ void __launch_bounds__(1 << LOG2B, main_min_blocks(TPT, LOG2B, KV)) k_main(const __grid_constant__ MainArgs a) {
     __shared__ long long s_item;

@@ -197,6 +197,7 @@ struct gce_handle_s {
     DevBuf payload, tau, seg, trialc, order, offsets, cand, stats, table, state, in_times, in_mags,
         in_periods, in_pdots, out_H, out_idx, band_stats, cand2, stats2;
     int table_n = -1;                    // largest count the table covers
+    bool ask_memory = false;             // a growth to the coarse form has failed (job_buffers)
     int *h_order = nullptr;              // pinned staging
     long long *h_offsets = nullptr;
     size_t h_cap = 0;
@@ -821,7 +822,7 @@ gce_status run_job(gce_handle h, const Job &j, cudaStream_t s) {
     size_t most = 0;
     for (const Need &x : plain) most = std::max(most, x.bytes);
     st = growth_status(h, job_buffers(kDevMemory, try_coarse ? coarse : nullptr, plain,
-                                      kWorkspaceBuffers, 3, &is_coarse), most);
+                                      kWorkspaceBuffers, 3, &is_coarse, &h->ask_memory), most);
     if (st != GCE_OK) return st;
     if (try_coarse && !is_coarse) pl.prep_mode = j.cfg->phase_mode;
     const int mode = pl.prep_mode;

@@ -63,8 +63,10 @@ inline Growth grow_all(const DevMemory &m, const Need *need, int n) {
 }
 
 // Whether the buffers that have to grow find the memory (each rounded up to the
-// allocator's 2 MiB pages; what they hold is given back first).
-inline bool fits(const DevMemory &m, const Need *need, int n) {
+// allocator's 2 MiB pages; what they hold is given back first).  Asking the device takes
+// some 25 us, a fifth of a small job's first call, so a growth of up to 64 MiB is tried
+// without asking until one has failed (ask).
+inline bool fits(const DevMemory &m, const Need *need, int n, bool ask) {
     const size_t page = (size_t)2 << 20;
     size_t more = 0, back = 0;
     for (int i = 0; i < n; ++i)
@@ -72,7 +74,8 @@ inline bool fits(const DevMemory &m, const Need *need, int n) {
             more += (need[i].bytes + page - 1) / page * page;
             back += need[i].buf->bytes;
         }
-    return more == 0 || more <= m.available() + back;
+    if (more == 0 || (!ask && more <= ((size_t)64 << 20))) return true;
+    return more <= m.available() + back;
 }
 
 // The buffers of a job.  coarse (or nullptr) and plain: its needs in either form, of the
@@ -80,13 +83,15 @@ inline bool fits(const DevMemory &m, const Need *need, int n) {
 // it is taken only where all of the job's buffers fit beside it, asked before anything is
 // given up, so that a job that does not fit runs plain call after call without allocating.
 // The first n_forms buffers are the ones whose size the form decides: where the plain form
-// does not fit either, what they hold from other jobs is given back first.
+// does not fit either, what they hold from other jobs is given back first.  ask: the
+// handle's (see fits).
 inline Growth job_buffers(const DevMemory &m, const Need *coarse, const Need *plain, int n,
-                          int n_forms, bool *is_coarse) {
+                          int n_forms, bool *is_coarse, bool *ask) {
     *is_coarse = coarse != nullptr;
-    if (coarse && fits(m, coarse, n)) {
+    if (coarse && fits(m, coarse, n, *ask)) {
         const Growth g = grow_all(m, coarse, n);
         if (g != NO_MEMORY) return g;
+        *ask = true;
     }
     *is_coarse = false;
     Growth g = grow_all(m, plain, n);

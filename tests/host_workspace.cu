@@ -48,19 +48,19 @@ int main() {
             g_live.clear();
             DevBuf b[4];
             Need cn[4], pn[4];
-            bool coarse = false;
+            bool coarse = false, ask = false;
             for (int i = 0; i < 4; ++i) {
                 cn[i] = {&b[i], before == 1 ? c[i] / 4 : c[i]};
                 pn[i] = {&b[i], before == 2 ? q[i] / 2 : q[i]};
             }
-            if (before) CHECK(job_buffers(kFake, before == 1 ? cn : nullptr, pn, 4, 3, &coarse) == GROWN);
+            if (before) CHECK(job_buffers(kFake, before == 1 ? cn : nullptr, pn, 4, 3, &coarse, &ask) == GROWN);
             if (g_used > budget) continue;
             g_budget = budget;
             for (int i = 0; i < 4; ++i) {
                 cn[i] = {&b[i], c[i]};
                 pn[i] = {&b[i], q[i]};
             }
-            const Growth g = job_buffers(kFake, cn, pn, 4, 3, &coarse);
+            const Growth g = job_buffers(kFake, cn, pn, 4, 3, &coarse, &ask);
             // what fits plain (340 MiB) is taken, whatever the buffers held
             CHECK((g == GROWN) == (budget >= 340 * M));
             CHECK(g_used <= g_budget);
@@ -72,10 +72,33 @@ int main() {
             // the same call again allocates and frees nothing
             const int ops = g_ops;
             bool again = false;
-            CHECK(job_buffers(kFake, cn, pn, 4, 3, &again) == GROWN && again == coarse && g_ops == ops);
+            CHECK(job_buffers(kFake, cn, pn, 4, 3, &again, &ask) == GROWN && again == coarse && g_ops == ops);
             // with memory to spare again, it runs coarse
             g_budget = 2000 * M;
-            CHECK(job_buffers(kFake, cn, pn, 4, 3, &again) == GROWN && again);
+            CHECK(job_buffers(kFake, cn, pn, 4, 3, &again, &ask) == GROWN && again);
+        }
+    }
+    // small growth: tried without asking, and after one that failed asked for, so that calls
+    // in the plain form allocate nothing from the second on
+    const size_t K = (size_t)1 << 10;
+    for (size_t budget = 0; budget <= 900 * K; budget += K) {
+        g_budget = budget;
+        g_used = 0;
+        g_live.clear();
+        DevBuf b[4];
+        Need cn[4], pn[4];
+        bool coarse = false, ask = false;
+        for (int i = 0; i < 4; ++i) {
+            cn[i] = {&b[i], c[i] / M * K};
+            pn[i] = {&b[i], q[i] / M * K};
+        }
+        const Growth g = job_buffers(kFake, cn, pn, 4, 3, &coarse, &ask);
+        CHECK((g == GROWN) == (budget >= 340 * K) && coarse == (budget >= 740 * K) && g_used <= g_budget);
+        if (g != GROWN) continue;
+        const int ops = g_ops;
+        for (int rep = 0; rep < 3; ++rep) {
+            bool again = false;
+            CHECK(job_buffers(kFake, cn, pn, 4, 3, &again, &ask) == GROWN && again == coarse && g_ops == ops);
         }
     }
     std::printf("ok\n");

